@@ -1350,14 +1350,14 @@ void ggemm(Plan &P, const G &g, const int32_t *targets, int64_t a, int64_t e, in
 // far-image composite; FP64 sums, one block.  With dbar (FP32-based modes)
 // the mean goes to dbar and the mean-free rest to d.
 template <typename T>
-__global__ void k_far_root(int ns, const double *__restrict__ Ft, const double *__restrict__ u, T *__restrict__ d,
-                           double *__restrict__ dbar) {
+__global__ void __launch_bounds__(1024) k_far_root(int ns, const double *__restrict__ Ft, const double *__restrict__ u,
+                                                   T *__restrict__ d, double *__restrict__ dbar) {
     __shared__ double v[kMaxNs];
     __shared__ double red[32];
     for (int j = threadIdx.x; j < ns; j += blockDim.x) {
-        double acc = 0.0;
-        for (int k = 0; k < ns; ++k) acc += Ft[(size_t)k * ns + j] * u[k];
-        v[j] = acc;
+        double tot = 0.0;
+        for (int q = 0; q < parts; ++q) tot += pv[q * ns + j];
+        v[j] = tot;
     }
     __syncthreads();
     double mean = 0.0;
@@ -1392,7 +1392,16 @@ __global__ void k_moment_term(int64_t nl, const double *__restrict__ leaf_q2, in
         b += __shfl_xor_sync(0xffffffffu, b, o);
     }
     if ((threadIdx.x & 31) == 0) {
+    __shared__ double pv[1024];
         red[0][threadIdx.x >> 5] = a;
+    const int parts = max(1, (int)blockDim.x / ns), part = threadIdx.x / ns, jp = threadIdx.x - part * ns;
+    const int chunk = (ns + parts - 1) / parts;
+    static_assert(kMaxNs <= 1024, "a thread per output");
+    double acc = 0.0;
+    if (part < parts)
+        for (int k = part * chunk; k < min(ns, (part + 1) * chunk); ++k) acc += Ft[(size_t)k * ns + jp] * u[k];
+    pv[threadIdx.x] = acc;
+    __syncthreads();
         red[1][threadIdx.x >> 5] = b;
     }
     __syncthreads();
@@ -1405,22 +1414,34 @@ __global__ void k_moment_term(int64_t nl, const double *__restrict__ leaf_q2, in
 
 // FP32-based periodic plans: the root's upward check potential in FP64 from
 // its children's (M2M composites in FP64, stored [k][j]); a root that is a
-// leaf keeps its own.  One block.
-__global__ void k_root_up64(int ns, const int32_t *__restrict__ child8, const int32_t *__restrict__ nchild,
-                            const double *__restrict__ m2m64, const float *__restrict__ u, double *__restrict__ u64) {
-    for (int j = threadIdx.x; j < ns; j += blockDim.x) {
-        double acc = 0.0;
-        if (nchild[0] == 0) {
-            acc = (double)u[j];
-        } else {
-            for (int c = 0; c < 8; ++c) {
-                const int32_t ch = child8[c];
-                if (ch < 0) continue;
-                const double *M = m2m64 + (size_t)c * ns * ns;
-                for (int k = 0; k < ns; ++k) acc += M[(size_t)k * ns + j] * (double)u[(size_t)ch * ns + k];
-            }
+// leaf keeps its own.  8 n_s^2 FP64 products at two lanes per clock and SM:
+// eight outputs per block spread them over the SMs (one block: 330 us at
+// n_s = 152), 32 threads sharing each output's 8 n_s terms.
+constexpr int kRootCols = 8;
+__global__ void __launch_bounds__(32 * kRootCols) k_root_up64(int ns, const int32_t *__restrict__ child8,
+                                                              const int32_t *__restrict__ nchild,
+                                                              const double *__restrict__ m2m64,
+                                                              const float *__restrict__ u, double *__restrict__ u64) {
+    __shared__ double red[32][kRootCols];
+    const int c = threadIdx.x % kRootCols, p = threadIdx.x / kRootCols;
+    const int j = blockIdx.x * kRootCols + c;
+    double acc = 0.0;
+    if (nchild[0] == 0) {
+        if (j < ns && p == 0) acc = (double)u[j];
+    } else if (j < ns) {
+        const int o = p >> 2;  // four threads per child octant
+        const int32_t ch = child8[o];
+        if (ch >= 0) {
+            const double *M = m2m64 + (size_t)o * ns * ns + j;
+            for (int k = p & 3; k < ns; k += 4) acc += M[(size_t)k * ns] * (double)u[(size_t)ch * ns + k];
         }
-        u64[j] = acc;
+    }
+    red[p][c] = acc;
+    __syncthreads();
+    if (threadIdx.x < kRootCols && j < ns) {
+        double tot = 0.0;
+        for (int q = 0; q < 32; ++q) tot += red[q][threadIdx.x];
+        u64[j] = tot;
     }
 }
 
@@ -1481,11 +1502,11 @@ cudaError_t evaluate_t(Plan &P, void *pot, void *grad, double *energy, cudaStrea
         if constexpr (sizeof(T) == 8) {
             u_root = (const double *)u;
         } else {
-            ++g_launches, k_root_up64<<<1, 256, 0, s>>>(ns, P.child8, P.nchild, P.m2m64, u, P.u_root64);
+            ++g_launches, k_root_up64<<<grid_for(ns, kRootCols), 32 * kRootCols, 0, s>>>(ns, P.child8, P.nchild, P.m2m64, u, P.u_root64);
             u_root = P.u_root64;
         }
         // the far images, on the root (box 0) before the downward pass
-        ++g_launches, k_far_root<T><<<1, 256, 0, s>>>(ns, P.far_t, u_root, d, split_mean ? P.dbar : nullptr);
+        ++g_launches, k_far_root<T><<<1, 1024, 0, s>>>(ns, P.far_t, u_root, d, split_mean ? P.dbar : nullptr);
     }
     // downward pass: per level, per octant class of the child
     stage_begin(P, KIFMM_STAGE_L2L, s);
