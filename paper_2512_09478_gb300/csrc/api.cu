@@ -75,16 +75,19 @@ bool tuning_wanted(const Plan &P, cudaStream_t s) {
     return st == cudaStreamCaptureStatusNone;
 }
 
+void plan_free(Plan &P, void **ptr) {
+    if (!*ptr) return;
+    for (auto it = P.owned.begin(); it != P.owned.end(); ++it)
+        if (it->ptr == *ptr) {
+            cudaFree(it->ptr);
+            P.owned.erase(it);
+            break;
+        }
+    *ptr = nullptr;
+}
+
 cudaError_t plan_alloc(Plan &P, void **ptr, size_t bytes) {
-    if (*ptr) {
-        for (auto it = P.owned.begin(); it != P.owned.end(); ++it)
-            if (it->ptr == *ptr) {
-                cudaFree(it->ptr);
-                P.owned.erase(it);
-                break;
-            }
-        *ptr = nullptr;
-    }
+    plan_free(P, ptr);
     void *p = nullptr;
     cudaError_t e = cudaMalloc(&p, bytes > 0 ? bytes : 16);
     if (e != cudaSuccess) return e;
@@ -280,7 +283,15 @@ kifmm_status kifmm_plan_create(const kifmm_plan_desc *desc, kifmm_plan **out) {
         e = m2l_tensor_setup(P);
         if (e == cudaErrorNotSupported) return fail(KIFMM_ERR_ARG);
         if (e != cudaSuccess) return fail(KIFMM_ERR_CUDA);
+    } else if (m2l_uses_simt(P)) {
+        if (m2l_simt_setup(P) != cudaSuccess) return fail(KIFMM_ERR_CUDA);
+    } else if (m2l_exact_setup(P, 0, P.m2l_t, P.op_ld) != cudaSuccess) {
+        return fail(KIFMM_ERR_CUDA);
     }
+    if (!P.stokes && !P.periodic && m2l_exact_setup(P, 1, P.adj_m2l, P.ns) != cudaSuccess) return fail(KIFMM_ERR_CUDA);
+    // the kernels read their own operator forms from here on
+    if (!m2l_uses_simt(P)) plan_free(P, &P.m2l_t);
+    plan_free(P, &P.adj_m2l);
     // workspace for n_max particles
     const int64_t n = d.n_max;
     P.n_cap = n;
@@ -342,6 +353,7 @@ kifmm_status kifmm_plan_destroy(kifmm_plan *pl) {
     if (!pl) return KIFMM_ERR_ARG;
     cudaDeviceSynchronize();
     m2l_tensor_release(pl->P);
+    m2l_exact_release(pl->P);
     for (auto &b : pl->P.owned) cudaFree(b.ptr);
     pl->P.owned.clear();
     if (pl->P.rb) cudaFreeHost(pl->P.rb);
@@ -442,8 +454,12 @@ static kifmm_status set_sources_impl(Plan &P, const void *xyz, const void *q, cu
         partition_finish(P);
     }
     if (st != 0) return (kifmm_status)st;
-    // tiles of the tensor-core M2L (kept lists: the same tiles)
-    if (P.desc.precision == KIFMM_MIXED_FP16 && !P.lists_reused) API_CUDA(m2l_tensor_tiles(P, s));
+    // tiles and workspace of the M2L kernels (kept lists: the same tiles)
+    if (!P.lists_reused) {
+        API_CUDA(m2l_tiles_build(P, s));
+        if (P.desc.precision == KIFMM_MIXED_FP16) API_CUDA(m2l_tensor_prepare(P));
+        API_CUDA(m2l_exact_prepare(P));
+    }
     if (!P.lists_reused) {
         P.prev_nb = P.nb;
         P.prev_sys_off = P.sys_off_h;

@@ -273,8 +273,8 @@ __global__ void k_p2l(const int32_t *__restrict__ nx, const int32_t *__restrict_
 // 160); each thread keeps an 8 x 5 register tile (targets 8 ty .. 8 ty + 7,
 // outputs tx + 32 c).  Operators are stored transposed ([k][j]); k advances in
 // chunks of 8 through shared memory with the next chunk prefetched into
-// registers.  Used for M2L (189 V slots), M2M (8 child octants), L2L (parent)
-// and the two factors of the leaf pseudo-inverses.
+// registers.  Used for M2M (8 child octants), L2L (parent) and the two factors
+// of the leaf pseudo-inverses.
 // ---------------------------------------------------------------------------
 constexpr int kGK = 16;
 
@@ -285,16 +285,6 @@ struct ClassRanges {
 
 // Operator blocks are [k][ld]: ld = n_s, or n_s + 1 when column n_s holds the
 // mean row of a mean-free check-to-check block (FP32-based modes).
-template <typename T>
-struct GatherM2L {
-    const int32_t *vdense;
-    const int *slot_off;
-    const T *ops;
-    int ns, ld;
-    __device__ int src(int t, int s, int) const { return vdense[(size_t)t * kVSlots + s]; }
-    __device__ const T *op(int s, int cls) const { return ops + (size_t)slot_off[cls * kVSlots + s] * ns * ld; }
-    __device__ double mean_base(int, const double *) const { return 0.0; }
-};
 template <typename T>
 struct GatherChild {
     const int32_t *child8;
@@ -1348,12 +1338,23 @@ void ggemm(Plan &P, const G &g, const int32_t *targets, int64_t a, int64_t e, in
 // Periodic cell (Sec. 2.4): the images beyond the 26 nearest act on the
 // root's downward check potential, d(root) += F u(root), with F the
 // far-image composite; FP64 sums, one block.  With dbar (FP32-based modes)
-// the mean goes to dbar and the mean-free rest to d.
+// the mean goes to dbar and the mean-free rest to d.  n_s^2 FP64 products on
+// one SM's two FP64 lanes (6 us at n_s = 152); each output's sum is cut into
+// blockDim / n_s parts so that the loads overlap (one part: 48 us).
 template <typename T>
 __global__ void __launch_bounds__(1024) k_far_root(int ns, const double *__restrict__ Ft, const double *__restrict__ u,
                                                    T *__restrict__ d, double *__restrict__ dbar) {
     __shared__ double v[kMaxNs];
+    __shared__ double pv[1024];
     __shared__ double red[32];
+    const int parts = max(1, (int)blockDim.x / ns), part = threadIdx.x / ns, jp = threadIdx.x - part * ns;
+    const int chunk = (ns + parts - 1) / parts;
+    static_assert(kMaxNs <= 1024, "a thread per output");
+    double acc = 0.0;
+    if (part < parts)
+        for (int k = part * chunk; k < min(ns, (part + 1) * chunk); ++k) acc += Ft[(size_t)k * ns + jp] * u[k];
+    pv[threadIdx.x] = acc;
+    __syncthreads();
     for (int j = threadIdx.x; j < ns; j += blockDim.x) {
         double tot = 0.0;
         for (int q = 0; q < parts; ++q) tot += pv[q * ns + j];
@@ -1392,16 +1393,7 @@ __global__ void k_moment_term(int64_t nl, const double *__restrict__ leaf_q2, in
         b += __shfl_xor_sync(0xffffffffu, b, o);
     }
     if ((threadIdx.x & 31) == 0) {
-    __shared__ double pv[1024];
         red[0][threadIdx.x >> 5] = a;
-    const int parts = max(1, (int)blockDim.x / ns), part = threadIdx.x / ns, jp = threadIdx.x - part * ns;
-    const int chunk = (ns + parts - 1) / parts;
-    static_assert(kMaxNs <= 1024, "a thread per output");
-    double acc = 0.0;
-    if (part < parts)
-        for (int k = part * chunk; k < min(ns, (part + 1) * chunk); ++k) acc += Ft[(size_t)k * ns + jp] * u[k];
-    pv[threadIdx.x] = acc;
-    __syncthreads();
         red[1][threadIdx.x >> 5] = b;
     }
     __syncthreads();
@@ -1484,8 +1476,12 @@ cudaError_t evaluate_t(Plan &P, void *pot, void *grad, double *energy, cudaStrea
     if (tensor) {
         KIFMM_CUDA_TRY(m2l_tensor(P, s));
     } else {
-        ggemm_classes<T>(P, GatherM2L<T>{P.vdense, P.slot_off, (const T *)P.m2l_t, ns, P.op_ld}, P.part_list[0],
-                         P.part_start[0].data(), 8, kVSlots, u, d, 0, s, P.op_ld, split_mean ? P.dbar : nullptr);
+        if constexpr (sizeof(T) == 4) {
+            if (m2l_uses_simt(P)) KIFMM_CUDA_TRY(m2l_simt(P, u, d, P.dbar, s));
+            else KIFMM_CUDA_TRY(m2l_exact(P, 0, u, d, 0, P.dbar, s));
+        } else {
+            KIFMM_CUDA_TRY(m2l_exact(P, 0, u, d, 0, nullptr, s));
+        }
     }
     stage_end(P, KIFMM_STAGE_M2L, s);
     if (P.n_x > 0) {
@@ -1877,8 +1873,8 @@ cudaError_t evaluate_stokes_t(Plan &P, void *vel, cudaStream_t s) {
     stage_end(P, KIFMM_STAGE_M2M, s);
     stage_begin(P, KIFMM_STAGE_M2L, s);
     KIFMM_CUDA_TRY(cudaMemsetAsync(d, 0, sizeof(T) * (size_t)P.nb * ns, s));
-    ggemm_classes<T>(P, GatherM2L<T>{P.vdense, P.slot_off, (const T *)P.m2l_t, ns, P.op_ld}, P.part_list[0],
-                     P.part_start[0].data(), 8, kVSlots, u, d, 0, s, P.op_ld, nullptr);
+    if constexpr (sizeof(T) == 4) KIFMM_CUDA_TRY(m2l_simt(P, u, d, nullptr, s));
+    else KIFMM_CUDA_TRY(m2l_exact(P, 0, u, d, 0, nullptr, s));
     stage_end(P, KIFMM_STAGE_M2L, s);
     if (P.n_x > 0) {
         stage_begin(P, KIFMM_STAGE_P2L, s);
@@ -2106,8 +2102,7 @@ cudaError_t backward_t(Plan &P, const void *w_user, const void *g_user, const do
         ggemm<T>(P, GatherChild<T>{P.child8, (const T *)P.adj_l2l, ns}, P.part_list[1], P.part_start[1][1 + l],
                  P.part_start[1][2 + l], 8, db, db, 1, s);
     // M2L^T (V lists are symmetric; operator at the negated offset, transposed)
-    ggemm_classes<T>(P, GatherM2L<T>{P.vdense, P.slot_off, (const T *)P.adj_m2l, ns, ns}, P.part_list[0],
-                     P.part_start[0].data(), 8, kVSlots, db, ub, 1, s);
+    KIFMM_CUDA_TRY(m2l_exact(P, 1, db, ub, 1, nullptr, s));
     // M2M^T, top-down
     for (int l = 1; l <= P.max_level; ++l)
         ggemm_classes<T>(P, GatherParent<T>{P.parent, (const T *)P.adj_m2m, ns, ns}, P.part_list[3],

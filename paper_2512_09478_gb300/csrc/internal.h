@@ -70,7 +70,7 @@ struct Plan {
     // transposed ([o][k][j]) in the compute type:
     void *m2m_t = nullptr;      // [8][ns][ns]   u(child)  -> u(parent)
     void *l2l_t = nullptr;      // [8][ns][op_ld]   d(parent) -> d(child)
-    void *m2l_t = nullptr;      // [316][ns][op_ld] u(source) -> d(target)
+    void *m2l_t = nullptr;      // [316][ns][op_ld] u(source) -> d(target); kept (padded) for the SIMT M2L only
     // FP32-based modes: l2l_t and m2l_t are mean-free over their outputs,
     // stored [blk][k][ns + 1] with the mean row in column ns (op_ld = ns + 1;
     // ns otherwise); d is then the mean-free part and dbar (FP64, per box)
@@ -114,6 +114,10 @@ struct Plan {
     bool fwd_res_valid = false; // ... and res still holds its field (no backward since)
     // Tensor-core M2L operands (mixed modes), built lazily.
     void *m2l_tc = nullptr;     // layout owned by the tensor-core kernel
+    void *m2l_ex = nullptr;     // operator slices of the exact-split M2L (FP64 / FP32 modes, every adjoint)
+    void *m2l_tiles = nullptr;  // target tiles shared by both M2L kernels
+    void *m2l_part = nullptr;   // partial sums of their slot splits
+    size_t m2l_part_bytes = 0;
     float *m2l_tc_scale = nullptr;
     int *slot_off = nullptr;    // [8][189] V slot -> M2L offset index (-1 unused)
     // Compressed M2L (desc.m2l_eps > 0, tensor-core mode): d = U C_o W u with
@@ -260,6 +264,7 @@ struct Plan {
 // keep_bytes of the old contents.
 cudaError_t plan_alloc(Plan &P, void **ptr, size_t bytes);
 cudaError_t plan_grow(Plan &P, void **ptr, size_t bytes, size_t keep_bytes);
+void plan_free(Plan &P, void **ptr);
 cudaError_t grow_tree_arrays(Plan &P, int64_t new_cap, int64_t keep);
 
 // Stage bracketing (no-ops unless profiling is enabled).
@@ -299,9 +304,30 @@ cudaError_t far_image_operator(int p, double L, double *T);
 // skin half-widths of the finest level (refresh_sources' reuse test); enqueues only.
 cudaError_t check_leaves(Plan &P, const void *xyz, double skin, int *moved_dev, cudaStream_t s);
 cudaError_t m2l_tensor_setup(Plan &P);
-cudaError_t m2l_tensor_tiles(Plan &P, cudaStream_t s);
+cudaError_t m2l_tensor_prepare(Plan &P);
 cudaError_t m2l_tensor(Plan &P, cudaStream_t s);
 void m2l_tensor_release(Plan &P);
+
+// target tiles of both M2L kernels (after the partitions are known)
+cudaError_t m2l_tiles_build(Plan &P, cudaStream_t s);
+int m2l_tiles_128(const Plan &P);          // tiles of 128 targets
+const int4 *m2l_tiles_dev(const Plan &P);  // (class, begin, end, 0) each
+cudaError_t m2l_part_reserve(Plan &P, size_t bytes);
+
+// ---- m2l_exact.cu (FP64 and FP32 modes, Stokeslet, every plan's adjoint) ----
+// dir 0 forward, 1 adjoint; ops [316][n_s][ld], device, compute type
+cudaError_t m2l_exact_setup(Plan &P, int dir, const void *ops, int ld);
+cudaError_t m2l_exact_prepare(Plan &P);
+cudaError_t m2l_exact(Plan &P, int dir, const void *u, void *d, int accumulate, double *dbar, cudaStream_t s);
+void m2l_exact_release(Plan &P);
+int m2l_slot_split(int64_t units, int num_sms);
+
+// ---- m2l_simt.cu (FP32 Stokeslet and FP32 periodic plans) ----
+inline bool m2l_uses_simt(const Plan &P) {
+    return !P.f64 && P.desc.precision != KIFMM_MIXED_FP16 && (P.stokes || P.periodic);
+}
+cudaError_t m2l_simt_setup(Plan &P);
+cudaError_t m2l_simt(Plan &P, const float *u, float *d, double *dbar, cudaStream_t s);
 
 // ---- fmm.cu ----
 // Autotuning: true when desc.autotune asks for it, something is still

@@ -26,6 +26,11 @@
 //              and frees the stage with tcgen05.commit on its "empty" barrier.
 //   8 warps    drain: each V slot's partial accumulator is added in IEEE FP32
 //              to running sums held in registers, then unscaled and stored.
+// Small trees have too few tiles for the SMs: blockIdx.z then takes a range of
+// the 189 slots (tc_shape), every slot's partial product is stored and a second
+// kernel adds them in slot order, the additions (and so the bits) of the
+// unsplit form.  A tree of up to 19 k targets took 495 us whatever its size,
+// the latency of 945 stages in a row.
 // Every wait is bounded; on time-out the CTA records KIFMM_ERR_TIMEOUT, drains
 // its own copies and MMAs (bounded), frees TMEM and returns.
 #include <cuda_fp16.h>
@@ -67,6 +72,8 @@ struct TileArgs {
     const float *level_unscale;  // 1 / (sigma_A(level) sigma_B)
     float *d;                 // [nb][ns]
     double *dbar;             // [nb] output column ns (the mean row), or nullptr
+    float *part;              // SPLIT: [189][tile of 128][np][128] partial products
+    int n_tiles;              // tiles of 128
     int ns, kp, np, nstages;  // np: operator rows (output columns) incl. padding
     int ncb;                  // column blocks (np = ncb NT)
     long long wait_polls;     // bound of the pipeline's barrier waits (the clean-up waits keep kWaitIters)
@@ -78,7 +85,7 @@ __device__ __forceinline__ uint32_t swz64(int r, int c) {
     return (uint32_t)(r * kRowBytes + ((c ^ ((r >> 1) & 3)) << 4));
 }
 
-template <int NCH, int PW, int TL>
+template <int NCH, int PW, int TL, bool SPLIT = false>
 __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
     constexpr int NT = 32 * NCH;  // output columns of this CTA (MMA N)
     constexpr int kProdWarps = PW;
@@ -139,7 +146,10 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
     tc_fence_after();
     const uint32_t tmem = tmem_base_s;
     const int kblocks = kp / kKBlock;
-    const int iters = kVSlots * kblocks;
+    // this CTA's slots
+    const int s_lo = SPLIT ? (int)(kVSlots * blockIdx.z / gridDim.z) : 0;
+    const int s_hi = SPLIT ? (int)(kVSlots * (blockIdx.z + 1) / gridDim.z) : kVSlots;
+    const int iters = (s_hi - s_lo) * kblocks;
 
     if (warp < kProdWarps) {
         // ---------------- producers ----------------
@@ -155,23 +165,23 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
         for (int i = 0; i < kRowsPerThread; ++i) {
             const int32_t tg = tgt_s[r0 + 8 * kProdWarps * i];
             src[i] = -1;
-            src_next[i] = (tg >= 0) ? a.vdense[(size_t)tg * kVSlots] : -1;
+            src_next[i] = (tg >= 0) ? a.vdense[(size_t)tg * kVSlots + s_lo] : -1;
         }
         const bool leader = threadIdx.x == 0;
-        int o_cur = 0, o_next = leader ? a.slot_off[cls * kVSlots] : 0, last_it = -1;
+        int o_cur = 0, o_next = leader ? a.slot_off[cls * kVSlots + s_lo] : 0, last_it = -1;
         for (int it = 0; it < iters; ++it) {
             const int stage = it % NS;
-            const int s = it / kblocks, kb = it - s * kblocks;
+            const int s = s_lo + it / kblocks, kb = it - (s - s_lo) * kblocks;
             if (kb == 0) {
 #pragma unroll
                 for (int i = 0; i < kRowsPerThread; ++i) {
                     src[i] = src_next[i];
                     const int32_t tg = tgt_s[r0 + 8 * kProdWarps * i];
-                    if (s + 1 < kVSlots) src_next[i] = (tg >= 0) ? a.vdense[(size_t)tg * kVSlots + s + 1] : -1;
+                    if (s + 1 < s_hi) src_next[i] = (tg >= 0) ? a.vdense[(size_t)tg * kVSlots + s + 1] : -1;
                 }
                 if (leader) {
                     o_cur = o_next;
-                    if (s + 1 < kVSlots) o_next = a.slot_off[cls * kVSlots + s + 1];
+                    if (s + 1 < s_hi) o_next = a.slot_off[cls * kVSlots + s + 1];
                 }
             }
             if (!mbar_wait(smem_u32(&empty_bar[stage]), ((it / NS) & 1) ^ 1, &abort_s, a.wait_polls)) {
@@ -220,7 +230,7 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
         if (lane == 0) {
             int it = 0;
             const uint32_t id = idesc_f16(NT);
-            for (int s = 0; s < kVSlots && !abort_s; ++s) {
+            for (int s = 0; s < s_hi - s_lo && !abort_s; ++s) {
                 uint32_t tacc[TL];
                 bool ok = true;
                 for (int t = 0; t < ntl; ++t) {
@@ -282,50 +292,80 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
         const int q = warp & 3, h = (d >> 2) & 1;
         const uint32_t lane_off = (uint32_t)(q * 32) << 16;
         const int c_base = h * (NT / 2);
-        float acc[NT / 2];
+        if constexpr (SPLIT) {
+            // every slot's partial product, columns of 128 rows (tile.w: the
+            // CTA's first tile of 128): a warp stores whole 128-byte lines
+            if (t < ntl) {
+                float *out = a.part + (((size_t)s_lo * a.n_tiles + tile.w + t) * a.np + cb * NT + c_base) * kTcRows +
+                             q * 32 + lane;
+                for (int s = 0; s < s_hi - s_lo; ++s, out += (size_t)a.n_tiles * a.np * kTcRows) {
+                    const int u = s * ntl + t, buf = u % kAccBufs;
+                    bool ok = mbar_wait(smem_u32(&accfull_bar[buf]), (u / kAccBufs) & 1, &abort_s, a.wait_polls);
+                    ok = __all_sync(0xffffffffu, ok);  // warp-uniform: tcgen05.ld is .sync.aligned
+                    if (!ok) {
+                        set_status(a.status, KIFMM_ERR_TIMEOUT);
+                        abort_s = 1;
+                        break;
+                    }
+                    tc_fence_after();
 #pragma unroll
-        for (int j = 0; j < NT / 2; ++j) acc[j] = 0.f;
-        bool ok = true;
-        if (t < ntl) {
-            for (int s = 0; s < kVSlots; ++s) {
-                const int u = s * ntl + t, buf = u % kAccBufs;
-                ok = mbar_wait(smem_u32(&accfull_bar[buf]), (u / kAccBufs) & 1, &abort_s, a.wait_polls);
-                ok = __all_sync(0xffffffffu, ok);  // warp-uniform: tcgen05.ld is .sync.aligned
-                if (!ok) {
-                    set_status(a.status, KIFMM_ERR_TIMEOUT);
-                    abort_s = 1;
-                    break;
+                    for (int c = 0; c < NT / 32; ++c) {
+                        float p[16];
+                        tmem_ld16(tmem + lane_off + (uint32_t)(buf * NT + c_base + 16 * c), p);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) out[(16 * c + j) * kTcRows] = p[j];
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&accfree_bar[buf]));
                 }
-                tc_fence_after();
-                // (two tiles: eight columns per load, the running sums take
-                // most of the registers)
-                constexpr int LW = TL == 2 ? 8 : 16;
-#pragma unroll
-                for (int c = 0; c < NT / (2 * LW); ++c) {
-                    float p[LW];
-                    if constexpr (LW == 8)
-                        tmem_ld8(tmem + lane_off + (uint32_t)(buf * NT + c_base + LW * c), p);
-                    else
-                        tmem_ld16(tmem + lane_off + (uint32_t)(buf * NT + c_base + LW * c), p);
-#pragma unroll
-                    for (int j = 0; j < LW; ++j) acc[LW * c + j] += p[j];
-                }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&accfree_bar[buf]));
             }
-        }
-        ok = ok && !abort_s && t < ntl;
-        const int row = t * kTcRows + q * 32 + lane;
-        const int32_t tb = tgt_s[row];
-        if (ok && tb >= 0) {
-            const float scale = a.level_unscale[a.lvl[tb]];
-            const int col0 = cb * NT + c_base;
-            float *out = a.d + (size_t)tb * a.ns + col0;
+        } else {
+            float acc[NT / 2];
 #pragma unroll
-            for (int j = 0; j < NT / 2; ++j) {
-                if (col0 + j < a.ns) out[j] = acc[j] * scale;
-                else if (col0 + j == a.ns && a.dbar) a.dbar[tb] = (double)(acc[j] * scale);
+            for (int j = 0; j < NT / 2; ++j) acc[j] = 0.f;
+            bool ok = true;
+            if (t < ntl) {
+                for (int s = 0; s < kVSlots; ++s) {
+                    const int u = s * ntl + t, buf = u % kAccBufs;
+                    ok = mbar_wait(smem_u32(&accfull_bar[buf]), (u / kAccBufs) & 1, &abort_s, a.wait_polls);
+                    ok = __all_sync(0xffffffffu, ok);  // warp-uniform: tcgen05.ld is .sync.aligned
+                    if (!ok) {
+                        set_status(a.status, KIFMM_ERR_TIMEOUT);
+                        abort_s = 1;
+                        break;
+                    }
+                    tc_fence_after();
+                    // (two tiles: eight columns per load, the running sums take
+                    // most of the registers)
+                    constexpr int LW = TL == 2 ? 8 : 16;
+#pragma unroll
+                    for (int c = 0; c < NT / (2 * LW); ++c) {
+                        float p[LW];
+                        if constexpr (LW == 8)
+                            tmem_ld8(tmem + lane_off + (uint32_t)(buf * NT + c_base + LW * c), p);
+                        else
+                            tmem_ld16(tmem + lane_off + (uint32_t)(buf * NT + c_base + LW * c), p);
+#pragma unroll
+                        for (int j = 0; j < LW; ++j) acc[LW * c + j] += p[j];
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&accfree_bar[buf]));
+                }
+            }
+            ok = ok && !abort_s && t < ntl;
+            const int row = t * kTcRows + q * 32 + lane;
+            const int32_t tb = tgt_s[row];
+            if (ok && tb >= 0) {
+                const float scale = a.level_unscale[a.lvl[tb]];
+                const int col0 = cb * NT + c_base;
+                float *out = a.d + (size_t)tb * a.ns + col0;
+#pragma unroll
+                for (int j = 0; j < NT / 2; ++j) {
+                    if (col0 + j < a.ns) out[j] = acc[j] * scale;
+                    else if (col0 + j == a.ns && a.dbar) a.dbar[tb] = (double)(acc[j] * scale);
+                }
             }
         }
     }
@@ -340,6 +380,35 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols) : "memory");
     }
+}
+
+// Slot splits: the running sums of the drain warps (slot order), from the
+// stored partial products; a thread per target row and output column, the
+// rows of a tile adjacent.
+__global__ void __launch_bounds__(128) k_m2l_slot_sum(const int32_t *__restrict__ targets, const int4 *__restrict__ tiles,
+                                                      int n_tiles, int ns, int np,
+                                                      const float *__restrict__ part, const int32_t *__restrict__ lvl,
+                                                      const float *__restrict__ level_unscale, float *__restrict__ d,
+                                                      double *__restrict__ dbar) {
+    static_assert(kTcRows == 128, "a thread per row");
+    const int4 tile = tiles[blockIdx.x];
+    const int i = tile.y + threadIdx.x, j = blockIdx.y;
+    if (i >= tile.z) return;
+    const float *src = part + ((size_t)blockIdx.x * np + j) * kTcRows + threadIdx.x;
+    const size_t step = (size_t)n_tiles * np * kTcRows;
+    float a = 0.f;
+    static_assert(kVSlots % 21 == 0, "slots in rounds of 21 loads");
+    for (int s0 = 0; s0 < kVSlots; s0 += 21) {
+        float v[21];
+#pragma unroll
+        for (int k = 0; k < 21; ++k) v[k] = src[(s0 + k) * step];
+#pragma unroll
+        for (int k = 0; k < 21; ++k) a += v[k];
+    }
+    const int32_t t = targets[i];
+    const float v = a * level_unscale[lvl[t]];
+    if (j < ns) d[(size_t)t * ns + j] = v;
+    else dbar[t] = (double)v;
 }
 
 // max |u| per level, as float bits (non-negative floats order like integers).
@@ -485,21 +554,24 @@ __global__ void k_absmax_f32(int64_t n, const float *__restrict__ x, unsigned *o
 
 int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
-template <int PW, int TL>
+template <int PW, int TL, bool SP>
 cudaError_t set_smem_attr_v(int nt, int bytes) {
+    constexpr auto dyn = cudaFuncAttributeMaxDynamicSharedMemorySize;
     switch (nt) {
-        case 32: return cudaFuncSetAttribute(k_m2l_tc<1, PW, TL>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        case 64: return cudaFuncSetAttribute(k_m2l_tc<2, PW, TL>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        case 96: return cudaFuncSetAttribute(k_m2l_tc<3, PW, TL>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        case 128: return cudaFuncSetAttribute(k_m2l_tc<4, PW, TL>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        case 160: return cudaFuncSetAttribute(k_m2l_tc<5, PW, TL>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        case 32: return cudaFuncSetAttribute(k_m2l_tc<1, PW, TL, SP>, dyn, bytes);
+        case 64: return cudaFuncSetAttribute(k_m2l_tc<2, PW, TL, SP>, dyn, bytes);
+        case 96: return cudaFuncSetAttribute(k_m2l_tc<3, PW, TL, SP>, dyn, bytes);
+        case 128: return cudaFuncSetAttribute(k_m2l_tc<4, PW, TL, SP>, dyn, bytes);
+        case 160: return cudaFuncSetAttribute(k_m2l_tc<5, PW, TL, SP>, dyn, bytes);
         default: return cudaErrorNotSupported;
     }
 }
 cudaError_t set_smem_attr(int nt, int bytes) {
-    KIFMM_CUDA_TRY((set_smem_attr_v<2, 1>(nt, bytes)));
-    KIFMM_CUDA_TRY((set_smem_attr_v<4, 1>(nt, bytes)));
-    return set_smem_attr_v<2, 2>(nt, bytes);
+    KIFMM_CUDA_TRY((set_smem_attr_v<2, 1, false>(nt, bytes)));
+    KIFMM_CUDA_TRY((set_smem_attr_v<4, 1, false>(nt, bytes)));
+    KIFMM_CUDA_TRY((set_smem_attr_v<2, 1, true>(nt, bytes)));
+    KIFMM_CUDA_TRY((set_smem_attr_v<2, 2, true>(nt, bytes)));
+    return set_smem_attr_v<2, 2, false>(nt, bytes);
 }
 
 // Kernel variants the tuner chooses between: (producer warps, tiles per
@@ -514,7 +586,6 @@ struct TcState {
     float sigma_b = 1.f;
     int pw = 2;               // producer warps
     int tl = 1;               // target tiles (of 128) per CTA, sharing each B block
-    int n_tiles[2] = {0, 0};  // CTAs (entries of tiles) for 1 and 2 tiles per CTA
     size_t stage_bytes(int t) const { return (size_t)t * 2 * kTcRows * kRowBytes + 2 * (size_t)nt * kRowBytes; }
     int nstages_max(int t) const { return (int)std::min<size_t>(16, (227 * 1024 - 4096) / stage_bytes(t)); }
     __half *bhl = nullptr;    // operators, hi and lo blocks interleaved per (o, kb, cb)
@@ -522,15 +593,20 @@ struct TcState {
     int64_t u_cap = 0;
     unsigned *level_max = nullptr;
     float *level_sigma = nullptr, *level_unscale = nullptr;
+    size_t smem = 0;
+    int n_in = 0, n_out = 0, ld = 0;  // operator inputs, outputs (mean excluded), stored columns
+};
+
+// Target tiles of the M2L kernels and the partial sums of their slot splits.
+struct M2lTiles {
+    int n_tiles[2] = {0, 0};  // CTAs (entries of tiles) for 1 and 2 tiles per CTA
     int4 *tiles = nullptr;
     int64_t tiles_cap = 0;
     std::vector<int4> tiles_h;
-    size_t smem = 0;
-    int n_in = 0, n_out = 0, ld = 0;  // operator inputs, outputs (mean excluded), stored columns
     int4 *tiles_pin = nullptr;        // pinned staging of tiles_h (a pageable copy stalls the stream)
     size_t tiles_pin_cap = 0;
     cudaEvent_t tiles_copied = nullptr;  // the last upload from tiles_pin
-    ~TcState() {
+    ~M2lTiles() {
         if (tiles_copied) {
             cudaEventSynchronize(tiles_copied);
             cudaEventDestroy(tiles_copied);
@@ -538,6 +614,21 @@ struct TcState {
         if (tiles_pin) cudaFreeHost(tiles_pin);
     }
 };
+
+static M2lTiles &tile_state(Plan &P) {
+    if (!P.m2l_tiles) P.m2l_tiles = new M2lTiles();
+    return *(M2lTiles *)P.m2l_tiles;
+}
+int m2l_tiles_128(const Plan &P) { return P.m2l_tiles ? ((const M2lTiles *)P.m2l_tiles)->n_tiles[0] : 0; }
+const int4 *m2l_tiles_dev(const Plan &P) { return ((const M2lTiles *)P.m2l_tiles)->tiles; }
+
+cudaError_t m2l_part_reserve(Plan &P, size_t bytes) {
+    if (bytes <= P.m2l_part_bytes) return cudaSuccess;
+    P.m2l_part_bytes = 0;
+    KIFMM_CUDA_TRY(plan_alloc(P, &P.m2l_part, bytes));
+    P.m2l_part_bytes = bytes;
+    return cudaSuccess;
+}
 
 static TcState &tc_state(Plan &P) {
     if (!P.m2l_tc) P.m2l_tc = new TcState();
@@ -562,10 +653,10 @@ bool m2l_tensor_pin(Plan &P, int producers, int tiles, int stages) {
 }
 
 void m2l_tensor_release(Plan &P) {
-    if (P.m2l_tc) {
-        delete (TcState *)P.m2l_tc;
-        P.m2l_tc = nullptr;
-    }
+    delete (TcState *)P.m2l_tc;
+    P.m2l_tc = nullptr;
+    delete (M2lTiles *)P.m2l_tiles;
+    P.m2l_tiles = nullptr;
 }
 
 // Plan time: FP16 hi/lo operators with one power-of-two scale.
@@ -615,14 +706,20 @@ cudaError_t m2l_tensor_setup(Plan &P) {
 
 // After set_sources: tiles of 128 targets within each octant class (one per
 // CTA), then tiles of 256 (two per CTA, the second possibly short or empty).
-cudaError_t m2l_tensor_tiles(Plan &P, cudaStream_t s) {
-    TcState &S = tc_state(P);
+cudaError_t m2l_tiles_build(Plan &P, cudaStream_t s) {
+    M2lTiles &S = tile_state(P);
     S.tiles_h.clear();
+    auto n128 = [&](int cls) {  // tiles of 128 before class cls
+        int n = 0;
+        for (int c = 0; c < cls; ++c) n += (int)((P.m2l_class_start[c + 1] - P.m2l_class_start[c] + kTcRows - 1) / kTcRows);
+        return n;
+    };
     for (int t = 1; t <= 2; ++t) {
         const int64_t rows = (int64_t)t * kTcRows;
         for (int c = 0; c < 8; ++c)
             for (int64_t b = P.m2l_class_start[c]; b < P.m2l_class_start[c + 1]; b += rows)
-                S.tiles_h.push_back(make_int4(c, (int)b, (int)std::min<int64_t>(b + rows, P.m2l_class_start[c + 1]), 0));
+                S.tiles_h.push_back(make_int4(c, (int)b, (int)std::min<int64_t>(b + rows, P.m2l_class_start[c + 1]),
+                                              n128(c) + (int)((b - P.m2l_class_start[c]) / kTcRows)));
         S.n_tiles[t - 1] = (int)S.tiles_h.size() - (t == 2 ? S.n_tiles[0] : 0);
     }
     if ((int64_t)S.tiles_h.size() > S.tiles_cap) {
@@ -646,17 +743,56 @@ cudaError_t m2l_tensor_tiles(Plan &P, cudaStream_t s) {
                                        cudaMemcpyHostToDevice, s));
         KIFMM_CUDA_TRY(cudaEventRecord(S.tiles_copied, s));
     }
+    return cudaGetLastError();
+}
+
+// Slot split z and tiles per CTA (of 128 targets) of an untuned launch: the
+// pair with the shortest estimated time.  A stage takes 0.53 us with one tile
+// per CTA, 0.82 with two (measured: 12k and 1M packings); a CTA costs about
+// four slots of set-up and fill beside its 189 / z; a split writes and reads
+// every slot's partial products (about 5 TB/s).  So trees of up to some 6 k
+// targets split and larger ones run unsplit.  Measured, both sides: 12k
+// particles (585 boxes) 957 -> 537 us a step; 120k in a periodic cell (4681
+// boxes) 1885 -> 1171 (with the root's own kernels); 1M (150 CTAs of two
+// tiles) runs unsplit as before, 2531 us.
+static void tc_shape(int n1, int n2, int64_t n_t, int ncb, int np, int kblocks, int num_sms, int *z_out,
+                     int *tl_out) {
+    double least = 1e30;
+    *z_out = 1;
+    *tl_out = 1;
+    const double traffic_us = 2.0 * kVSlots * (double)n_t * np * 4.0 / 5e6 + 4.0;
+    for (int z = 1; z <= 63 && (z == 1 || (int64_t)n1 * ncb * z <= 8 * (int64_t)num_sms); ++z)
+        for (int tl = 1; tl <= 2; ++tl) {
+            if (tl == 2 && n2 == n1) continue;
+            const int64_t ctas = (int64_t)(tl == 1 ? n1 : n2) * ncb * z;
+            const double t = (double)((ctas + num_sms - 1) / num_sms) * ((kVSlots + z - 1) / z + 4.0) * kblocks *
+                                 (tl == 1 ? 0.53 : 0.82) +
+                             (z > 1 ? traffic_us : 0.0);
+            if (t < 0.98 * least) {
+                least = t;
+                *z_out = z;
+                *tl_out = tl;
+            }
+        }
+}
+// Room for the split expansions and the slot splits' partial sums.
+cudaError_t m2l_tensor_prepare(Plan &P) {
+    TcState &S = tc_state(P);
     if (P.nb > S.u_cap) {
         S.u_cap = P.list_cap;
         KIFMM_CUDA_TRY(plan_alloc(P, (void **)&S.uh, sizeof(__half) * S.u_cap * S.kp));
         KIFMM_CUDA_TRY(plan_alloc(P, (void **)&S.ul, sizeof(__half) * S.u_cap * S.kp));
     }
-    return cudaGetLastError();
+    const M2lTiles &TS = tile_state(P);
+    int z, tl;
+    tc_shape(TS.n_tiles[0], TS.n_tiles[1], P.m2l_class_start[8], S.ncb, S.np, S.kp / kKBlock, P.num_sms, &z, &tl);
+    return m2l_part_reserve(P, z > 1 ? sizeof(float) * kVSlots * (size_t)TS.n_tiles[0] * kTcRows * S.np : 0);
 }
 
 cudaError_t m2l_tensor(Plan &P, cudaStream_t s) {
     TcState &S = tc_state(P);
-    if (S.tiles_h.empty()) return cudaSuccess;  // no V-list targets
+    const M2lTiles &TS = tile_state(P);
+    if (TS.tiles_h.empty()) return cudaSuccess;  // no V-list targets
     const int nlev = P.max_level + 1;
     const bool comp = P.m2l_rl > 0;
     const float *u = (const float *)P.u_chk;
@@ -672,7 +808,7 @@ cudaError_t m2l_tensor(Plan &P, cudaStream_t s) {
                                                                        S.level_sigma, S.uh, S.ul);
     TileArgs a;
     a.targets = P.m2l_targets;
-    a.tiles = S.tiles;
+    a.tiles = TS.tiles;
     a.vdense = P.vdense;
     a.slot_off = P.slot_off;
     a.uh = S.uh;
@@ -688,21 +824,27 @@ cudaError_t m2l_tensor(Plan &P, cudaStream_t s) {
     a.kp = S.kp;
     a.np = S.np;
     a.status = P.status;
-    auto launch_v = [&](auto pwc, auto tlc, int nst) -> cudaError_t {
+    int z, tl_default;
+    tc_shape(TS.n_tiles[0], TS.n_tiles[1], P.m2l_class_start[8], S.ncb, S.np, S.kp / kKBlock, P.num_sms, &z,
+             &tl_default);
+    a.part = z > 1 ? (float *)P.m2l_part : nullptr;
+    a.n_tiles = TS.n_tiles[0];
+    auto launch_v = [&](auto pwc, auto tlc, auto spl, int nst) -> cudaError_t {
         constexpr int PW = decltype(pwc)::value, TL = decltype(tlc)::value;
-        const int n = S.n_tiles[TL - 1];
+        constexpr bool SP = decltype(spl)::value;
+        const int n = TS.n_tiles[TL - 1];
         if (n == 0) return cudaSuccess;
         a.nstages = nst;
-        a.tiles = S.tiles + (TL == 2 ? S.n_tiles[0] : 0);
-        const dim3 grid((unsigned)n, (unsigned)S.ncb);
+        a.tiles = TS.tiles + (TL == 2 ? TS.n_tiles[0] : 0);
+        const dim3 grid((unsigned)n, (unsigned)S.ncb, (unsigned)z);
         const size_t smem = (size_t)nst * S.stage_bytes(TL) + 1024;
         const int thr = tc_threads(PW, TL);
         switch (S.nt) {
-            case 32: ++g_launches, k_m2l_tc<1, PW, TL><<<grid, thr, smem, s>>>(a); break;
-            case 64: ++g_launches, k_m2l_tc<2, PW, TL><<<grid, thr, smem, s>>>(a); break;
-            case 96: ++g_launches, k_m2l_tc<3, PW, TL><<<grid, thr, smem, s>>>(a); break;
-            case 128: ++g_launches, k_m2l_tc<4, PW, TL><<<grid, thr, smem, s>>>(a); break;
-            case 160: ++g_launches, k_m2l_tc<5, PW, TL><<<grid, thr, smem, s>>>(a); break;
+            case 32: ++g_launches, k_m2l_tc<1, PW, TL, SP><<<grid, thr, smem, s>>>(a); break;
+            case 64: ++g_launches, k_m2l_tc<2, PW, TL, SP><<<grid, thr, smem, s>>>(a); break;
+            case 96: ++g_launches, k_m2l_tc<3, PW, TL, SP><<<grid, thr, smem, s>>>(a); break;
+            case 128: ++g_launches, k_m2l_tc<4, PW, TL, SP><<<grid, thr, smem, s>>>(a); break;
+            case 160: ++g_launches, k_m2l_tc<5, PW, TL, SP><<<grid, thr, smem, s>>>(a); break;
             default: return cudaErrorNotSupported;
         }
         return cudaGetLastError();
@@ -711,13 +853,13 @@ cudaError_t m2l_tensor(Plan &P, cudaStream_t s) {
     using I4 = std::integral_constant<int, 4>;
     using I1 = std::integral_constant<int, 1>;
     auto launch_with = [&](int pw, int tl, int nst) -> cudaError_t {
-        if (tl == 2) return launch_v(I2{}, I2{}, nst);
-        return pw == 4 ? launch_v(I4{}, I1{}, nst) : launch_v(I2{}, I1{}, nst);
+        // (slot splits, bound by the stores, take two producer warps)
+        if (z > 1) return tl == 2 ? launch_v(I2{}, I2{}, std::true_type{}, nst) : launch_v(I2{}, I1{}, std::true_type{}, nst);
+        if (tl == 2) return launch_v(I2{}, I2{}, std::false_type{}, nst);
+        return pw == 4 ? launch_v(I4{}, I1{}, std::false_type{}, nst) : launch_v(I2{}, I1{}, std::false_type{}, nst);
     };
     if (!P.tuned_m2l) {
-        // untuned: two tiles per CTA (each operator block read once for 256
-        // targets) when that still gives every SM a CTA, else one
-        const bool two = S.n_tiles[1] >= P.num_sms;
+        const bool two = tl_default == 2;  // each operator block read once for 256 targets
         S.pw = 2;
         S.tl = two ? 2 : 1;
         S.nstages = two ? std::min(3, S.nstages_max(2)) : S.nstages_max(1);
@@ -750,6 +892,12 @@ cudaError_t m2l_tensor(Plan &P, cudaStream_t s) {
         P.tuned_m2l = true;
     }
     KIFMM_CUDA_TRY(launch_with(S.pw, S.tl, S.nstages));
+    if (z > 1) {
+        const int cols = S.n_out + (a.dbar ? 1 : 0);
+        ++g_launches, k_m2l_slot_sum<<<dim3((unsigned)TS.n_tiles[0], (unsigned)cols), kTcRows, 0, s>>>(
+                          P.m2l_targets, TS.tiles, TS.n_tiles[0], a.ns, S.np, a.part, P.lvl, S.level_unscale,
+                          a.d, a.dbar);
+    }
     if (comp) {  // back to the mean-free check potential of every target
         const int64_t nt = P.m2l_class_start[8];
         ++g_launches, k_rowmat<<<dim3((unsigned)((nt + 63) / 64), (unsigned)((P.ns + 63) / 64)), 256, 0, s>>>(

@@ -78,10 +78,10 @@ __device__ __forceinline__ uint64_t sdesc_sw64(uint32_t addr) {
     return d;
 }
 
-// Instruction descriptor, kind::f16: FP16 A and B, FP32 accumulate, both
-// K-major, M = 128, N = n.
-__device__ __forceinline__ uint32_t idesc_f16(int n) {
-    return (1u << 4) | (0u << 7) | (0u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTcRows >> 4) << 24);
+// Instruction descriptor, kind::f16: FP16 (fmt 0) or BF16 (fmt 1) A and B,
+// FP32 accumulate, both K-major, M = 128, N = n.
+__device__ __forceinline__ uint32_t idesc_f16(int n, uint32_t fmt = 0) {
+    return (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTcRows >> 4) << 24);
 }
 
 __device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
@@ -94,13 +94,22 @@ __device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t a, uint64_t b,
 }
 
 // The same with the A operand kept in the tensor core's collector buffer:
-// _fill reads A from shared memory and keeps it, _lastuse reuses the kept A
-// (the same descriptor) and releases it, so A is read once for two products.
+// _fill reads A from shared memory and keeps it, _use reuses the kept A (the
+// same descriptor), _lastuse reuses and releases it, so A is read once for
+// several products.
 __device__ __forceinline__ void mma_f16_fill(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        : "memory");
+}
+__device__ __forceinline__ void mma_f16_use(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
         "l"(a), "l"(b), "r"(idesc), "r"(acc)
         : "memory");
 }
@@ -154,6 +163,21 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float *v) {
     for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// The same without the wait: several loads in flight, then one tmem_wait_ld
+// before their registers are read.
+__device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t *r) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+// Waits for the warp's TMEM loads; ties the registers so that no use of them
+// moves above the wait.
+template <int N>
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[N]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < N; ++i) asm volatile("" : "+r"(r[i]));
+}
 
 }  // namespace
 }  // namespace kifmm
