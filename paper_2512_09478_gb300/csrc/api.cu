@@ -68,6 +68,16 @@ LeafTiling leaf_tiling_candidate(int c) {
     return t;
 }
 
+// FP64 is bound by the FP64 unit, which idle lanes take like busy ones: 17 to
+// 24 targets run as a pass of 16 and one of 8 (four source groups each)
+// instead of one of 32 lanes.
+LeafTiling leaf_tiling_f64() {
+    LeafTiling t = leaf_tiling_candidate(0);
+    t.set(1, 1);
+    t.set(2, 1);
+    return t;
+}
+
 bool tuning_wanted(const Plan &P, cudaStream_t s) {
     if (!P.desc.autotune) return false;
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
@@ -265,7 +275,7 @@ kifmm_status kifmm_plan_create(const kifmm_plan_desc *desc, kifmm_plan **out) {
     // ~30x and so does the FP32 rounding of every translation).
     P.eps = (d.pinv_eps != 0.0) ? d.pinv_eps : (P.f64 ? 1e-12 : 1e-9);
     P.direct_thr = (d.direct_max < 0) ? -1 : (d.direct_max == 0 ? P.nsurf : d.direct_max);
-    P.leaf_tile = leaf_tiling_candidate(0);
+    P.leaf_tile = P.f64 ? leaf_tiling_f64() : leaf_tiling_candidate(0);
     P.periodic = d.cell > 0.0;
     P.cell = d.cell;
     auto fail = [&](kifmm_status st) {

@@ -175,95 +175,107 @@ __global__ void k_p2m_f32(const int32_t *__restrict__ leaves, int64_t n_leaves, 
 }
 
 // P2L: d(b)_j += (1/h_b) sum_{a in X(b)} sum_i q_i / |1.05 S_j - (x_i - c_b)/h_b|
+// One block per box, few of which have an X list, but those up to 26 leaves of
+// it: a block's length is the launch's.  A thread per check point (tpg of them:
+// n_s rounded up to a warp; with 128 threads, two rounds over the sources, the
+// second for the last 24 points of n_s = 152).  FP64, bound by the FP64 unit,
+// also cuts the sources into blockDim / tpg interleaved groups, whose sums are
+// added in group order.  60k Plummer, FP64: 1.18 -> 0.44 ms.
 template <typename T>
-__global__ void k_p2l(const int32_t *__restrict__ nx, const int32_t *__restrict__ xdense,
-                      const int32_t *__restrict__ lvl, const int32_t *__restrict__ cx,
-                      const int32_t *__restrict__ cy, const int32_t *__restrict__ cz,
-                      const int32_t *__restrict__ first, const int32_t *__restrict__ cnt,
-                      const typename Vec4<T>::type *__restrict__ pts, const T *__restrict__ surf, int ns,
-                      T *__restrict__ d, const T *__restrict__ wts = nullptr, int adj = 0,
-                      double *__restrict__ dbar = nullptr, const T *__restrict__ dip = nullptr,
-                      const int8_t *__restrict__ x_sh = nullptr) {
+__global__ void __launch_bounds__(1024, 1)
+    k_p2l(int tpg, const int32_t *__restrict__ nx, const int32_t *__restrict__ xdense, const int32_t *__restrict__ lvl,
+          const int32_t *__restrict__ cx, const int32_t *__restrict__ cy, const int32_t *__restrict__ cz,
+          const int32_t *__restrict__ first, const int32_t *__restrict__ cnt,
+          const typename Vec4<T>::type *__restrict__ pts, const T *__restrict__ surf, int ns, T *__restrict__ d,
+          const T *__restrict__ wts = nullptr, int adj = 0, double *__restrict__ dbar = nullptr,
+          const T *__restrict__ dip = nullptr, const int8_t *__restrict__ x_sh = nullptr) {
     // With dbar (FP32-based modes) the mean of this box's contribution goes
     // to dbar and only the mean-free remainder to d.  With dip (adjoint of
     // M2P under a loss on the gradient) every particle also carries a dipole.
     __shared__ T sx[kLeafThreads], sy[kLeafThreads], sz[kLeafThreads], sq[kLeafThreads];
     __shared__ T gx[kLeafThreads], gy[kLeafThreads], gz[kLeafThreads];
     __shared__ T cv[kMaxNs];
-    __shared__ double red[kLeafThreads / 32];
+    __shared__ double red[32];
     const int b = blockIdx.x;
     if (nx[b] == 0) return;
     const int lb = lvl[b];
     const T hb = box_half<T>(lb), hinv = T(1) / hb;
     const T cbx = box_center<T>(cx[b], lb), cby = box_center<T>(cy[b], lb), cbz = box_center<T>(cz[b], lb);
     const T al = (T)kAlphaInner;
-    for (int j0 = 0; j0 < ns; j0 += blockDim.x) {
-        const int j = j0 + threadIdx.x;
-        T px = 0, py = 0, pz = 0;
-        if (j < ns) {
-            px = al * surf[3 * j];
-            py = al * surf[3 * j + 1];
-            pz = al * surf[3 * j + 2];
+    const int ng = blockDim.x / tpg, grp = threadIdx.x / tpg, j = threadIdx.x - grp * tpg;
+    T px = 0, py = 0, pz = 0;
+    if (j < ns) {
+        px = al * surf[3 * j];
+        py = al * surf[3 * j + 1];
+        pz = al * surf[3 * j + 2];
+    }
+    T acc = 0;
+    for (int e = 0; e < nx[b]; ++e) {
+        const int a = xdense[(size_t)b * kMaxCoarse + e];
+        const int la = lvl[a];
+        T ox = box_center<T>(cx[a], la) - cbx, oy = box_center<T>(cy[a], la) - cby,
+          oz = box_center<T>(cz[a], la) - cbz;
+        if (x_sh) {  // the source leaf's image (periodic cell)
+            T ix, iy, iz;
+            image_offset<T>(x_sh[(size_t)b * kMaxCoarse + e], ix, iy, iz);
+            ox += ix, oy += iy, oz += iz;
         }
-        T acc = 0;
-        for (int e = 0; e < nx[b]; ++e) {
-            const int a = xdense[(size_t)b * kMaxCoarse + e];
-            const int la = lvl[a];
-            T ox = box_center<T>(cx[a], la) - cbx, oy = box_center<T>(cy[a], la) - cby,
-              oz = box_center<T>(cz[a], la) - cbz;
-            if (x_sh) {  // the source leaf's image (periodic cell)
-                T ix, iy, iz;
-                image_offset<T>(x_sh[(size_t)b * kMaxCoarse + e], ix, iy, iz);
-                ox += ix, oy += iy, oz += iz;
-            }
-            const int n = cnt[a], f = first[a];
-            for (int c0 = 0; c0 < n; c0 += kLeafThreads) {
-                __syncthreads();
-                if (c0 + threadIdx.x < n) {
-                    const auto v = pts[f + c0 + threadIdx.x];
-                    sx[threadIdx.x] = (ox + v.x) * hinv;
-                    sy[threadIdx.x] = (oy + v.y) * hinv;
-                    sz[threadIdx.x] = (oz + v.z) * hinv;
-                    sq[threadIdx.x] = wts ? wts[f + c0 + threadIdx.x] : v.w;
-                    if (dip) {
-                        const size_t k = 3 * (size_t)(f + c0 + threadIdx.x);
-                        gx[threadIdx.x] = dip[k] * hinv;
-                        gy[threadIdx.x] = dip[k + 1] * hinv;
-                        gz[threadIdx.x] = dip[k + 2] * hinv;
-                    }
-                }
-                __syncthreads();
-                const int m = min(kLeafThreads, n - c0);
+        const int n = cnt[a], f = first[a];
+        for (int c0 = 0; c0 < n; c0 += kLeafThreads) {
+            __syncthreads();
+            const int m = min(kLeafThreads, n - c0);
+            for (int i = threadIdx.x; i < m; i += blockDim.x) {
+                const auto v = pts[f + c0 + i];
+                sx[i] = (ox + v.x) * hinv;
+                sy[i] = (oy + v.y) * hinv;
+                sz[i] = (oz + v.z) * hinv;
+                sq[i] = wts ? wts[f + c0 + i] : v.w;
                 if (dip) {
-                    for (int i = 0; i < m; ++i) {
-                        const T rx = px - sx[i], ry = py - sy[i], rz = pz - sz[i];
-                        const T ri = rsqrt_t<T>(rx * rx + ry * ry + rz * rz);
-                        acc += sq[i] * ri + (gx[i] * rx + gy[i] * ry + gz[i] * rz) * (ri * ri * ri);
-                    }
-                } else {
-                    for (int i = 0; i < m; ++i) acc += sq[i] * lap_pot<T>(px - sx[i], py - sy[i], pz - sz[i]);
+                    const size_t k = 3 * (size_t)(f + c0 + i);
+                    gx[i] = dip[k] * hinv;
+                    gy[i] = dip[k + 1] * hinv;
+                    gz[i] = dip[k + 2] * hinv;
                 }
             }
-        }
-        if (j < ns) {
-            const T v = adj ? acc : acc * hinv;
-            if (dbar) cv[j] = v; else d[(size_t)b * ns + j] += v;
+            __syncthreads();
+            if (dip) {
+                for (int i = grp; i < m; i += ng) {
+                    const T rx = px - sx[i], ry = py - sy[i], rz = pz - sz[i];
+                    const T ri = rsqrt_t<T>(rx * rx + ry * ry + rz * rz);
+                    acc += sq[i] * ri + (gx[i] * rx + gy[i] * ry + gz[i] * rz) * (ri * ri * ri);
+                }
+            } else {
+#pragma unroll 4
+                for (int i = grp; i < m; i += ng) acc += sq[i] * lap_pot<T>(px - sx[i], py - sy[i], pz - sz[i]);
+            }
         }
     }
-    if (dbar) {
+    for (int g = 0; g < ng; ++g) {  // the groups' sums, in group order
+        if (grp == g && j < ns) cv[j] = g == 0 ? acc : cv[j] + acc;
         __syncthreads();
+    }
+    if (!adj) {
+        if (grp == 0 && j < ns) cv[j] *= hinv;
+        __syncthreads();
+    }
+    if (!dbar) {
+        if (grp == 0 && j < ns) d[(size_t)b * ns + j] += cv[j];
+        return;
+    }
+    // (the mean's sum over 128 lanes, four warps, whatever the block)
+    if (threadIdx.x < kLeafThreads) {
         double sum = 0.0;
-        for (int j = threadIdx.x; j < ns; j += blockDim.x) sum += (double)cv[j];
+        for (int k = threadIdx.x; k < ns; k += kLeafThreads) sum += (double)cv[k];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
-        __syncthreads();
-        double tot = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
-        const double mean = tot / ns;
-        for (int j = threadIdx.x; j < ns; j += blockDim.x) d[(size_t)b * ns + j] += (T)((double)cv[j] - mean);
-        if (threadIdx.x == 0) dbar[b] += mean;
     }
+    __syncthreads();
+    double tot = 0.0;
+    for (int w = 0; w < kLeafThreads / 32; ++w) tot += red[w];
+    const double mean = tot / ns;
+    for (int k = threadIdx.x; k < ns; k += blockDim.x) d[(size_t)b * ns + k] += (T)((double)cv[k] - mean);
+    if (threadIdx.x == 0) dbar[b] += mean;
 }
 
 // ---------------------------------------------------------------------------
@@ -924,11 +936,14 @@ __device__ __forceinline__ void leaf_store(LeafSmem<T> &S, int slot, const typen
     }
 }
 
-template <typename T, int TPL, int G>
+// WPP warps share a pass (all warps of the block): warp `sub` takes every
+// WPP-th chunk of the stream, and the totals are added in warp order.
+template <typename T, int TPL, int G, int WPP>
 __device__ void leaf_pass(const LeafCtx &C, int b, int tbase, const typename Vec4<T>::type *__restrict__ pts,
-                          const T *__restrict__ surf, const LeafW<T> &W, LeafSmem<T> &S,
+                          const T *__restrict__ surf, const LeafW<T> &W, LeafSmem<T> *bufs, int sub,
                           double4 *__restrict__ res) {
     using V4 = typename Vec4<T>::type;
+    LeafSmem<T> &S = bufs[sub];
     constexpr int LG = 32 / G;  // lanes per group
     const int lane = threadIdx.x & 31, grp = lane / LG, mem = lane % LG;
     const int lb = C.lvl[b], bx = C.cx[b], by = C.cy[b], bz = C.cz[b];
@@ -1020,25 +1035,47 @@ __device__ void leaf_pass(const LeafCtx &C, int b, int tbase, const typename Vec
         typename Vec4<T>::type raw[kLK];
         int rs[kLK];
         const int nchunks = (total + kLChunk - 1) / kLChunk;
-        for (int c = 0; c < nchunks; ++c) {
+        for (int c = WPP > 1 ? sub : 0, slot = 0; c < nchunks; c += WPP, slot ^= 1) {
             // double-buffered: the slot written here was last read two chunks ago
             leaf_fetch<T>(S, c, total, nb, pts, surf, W, raw, rs);
-            leaf_store<T, G>(S, c & 1, raw, rs);
+            leaf_store<T, G>(S, slot, raw, rs);
             __syncwarp();
             const int c0 = c * kLChunk;
-            leaf_chunk<T, TPL, G>(L, S.buf[c & 1], min(kLChunk, total - c0), olo - c0, ohi - c0, grp);
+            leaf_chunk<T, TPL, G>(L, S.buf[slot], min(kLChunk, total - c0), olo - c0, ohi - c0, grp);
         }
     }
     leaf_flush<T, TPL>(L);
+    double totals[TPL][4];
 #pragma unroll
-    for (int k = 0; k < TPL; ++k) {
-        double tot[4];
+    for (int k = 0; k < TPL; ++k)
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            tot[c] = (double)L.acc[k][c] + (double)L.cmp[k][c];
+            totals[k][c] = (double)L.acc[k][c] + (double)L.cmp[k][c];
 #pragma unroll
-            for (int o = 16; o >= LG; o >>= 1) tot[c] += __shfl_xor_sync(0xffffffffu, tot[c], o);
+            for (int o = 16; o >= LG; o >>= 1) totals[k][c] += __shfl_xor_sync(0xffffffffu, totals[k][c], o);
         }
+    if constexpr (WPP > 1) {
+        // each warp's totals through its own staging buffer (its chunks are done)
+        static_assert(sizeof(S.buf) >= sizeof(double) * 32 * TPL * 4, "room for a warp's totals");
+        __syncwarp();
+        double *own = reinterpret_cast<double *>(&S.buf[0][0]);
+#pragma unroll
+        for (int k = 0; k < TPL; ++k)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) own[(4 * k + c) * 32 + lane] = totals[k][c];
+        __syncthreads();
+        if (sub != 0) return;
+        for (int w = 1; w < WPP; ++w) {
+            const double *o = reinterpret_cast<const double *>(&bufs[w].buf[0][0]);
+#pragma unroll
+            for (int k = 0; k < TPL; ++k)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) totals[k][c] += o[(4 * k + c) * 32 + lane];
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < TPL; ++k) {
+        double(&tot)[4] = totals[k];
         if (C.dbar) tot[0] += C.dbar[b];  // the constant part of the local expansion
         const int i = tbase + mem + LG * k;
         if (grp == 0 && i < n) {
@@ -1101,25 +1138,48 @@ __global__ void k_leaf_partition(int64_t n_leaves, const int32_t *__restrict__ l
     }
 }
 
-// Each warp takes the next pass from a shared counter as it finishes one
-// (passes differ in length by their source lists; a fixed stride left the
-// last warps running alone).  Every pass writes only its own targets, so the
-// order passes are taken in does not change any result.
+// Each warp (FP64: each block) takes the next pass from a shared counter as it
+// finishes one (passes differ in length by their source lists; a fixed stride
+// left the last warps running alone).  Every pass writes only its own targets,
+// so the order passes are taken in does not change any result.
+//
+// FP64 is bound by the FP64 unit (two lanes per clock and SM, some 19
+// operations per pair), so a pass of one warp is long: 32 targets of a leaf
+// with 6000 sources take 3.5 ms, and a 60k Plummer cloud spent two thirds of
+// its leaf stage waiting for the last of them.  The four warps of a block
+// therefore share each pass (that cloud, p = 6: the whole step 12.3 -> 9.0 ms;
+// 4096 points, p = 4: 2.06 -> 1.43 ms).
+template <typename T>
+__host__ __device__ constexpr int leaf_blocks_per_sm(int tpl) {
+    return sizeof(T) == 4 ? (tpl == 1 ? 5 : 4) : 3;
+}
 template <typename T, int TPL, int G>
-__global__ void __launch_bounds__(32 * kLW, sizeof(T) == 4 ? (TPL == 1 ? 5 : 4) : 2)
+__global__ void __launch_bounds__(32 * kLW, leaf_blocks_per_sm<T>(TPL))
     k_leaf_all(LeafCtx C, const int2 *__restrict__ list, const int32_t *__restrict__ count, int32_t *next,
                const typename Vec4<T>::type *__restrict__ pts, const T *__restrict__ surf, LeafW<T> W,
                double4 *__restrict__ res) {
     __shared__ LeafSmem<T> bufs[kLW];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nl = *count;
-    while (true) {
-        int li = 0;
-        if (lane == 0) li = atomicAdd(next, 1);
-        li = __shfl_sync(0xffffffffu, li, 0);
-        if (li >= nl) break;
-        const int2 it = list[li];
-        leaf_pass<T, TPL, G>(C, it.x, it.y, pts, surf, W, bufs[warp], res);
+    if constexpr (sizeof(T) == 8) {
+        __shared__ int taken;
+        while (true) {
+            __syncthreads();  // the previous pass is done with taken and the buffers
+            if (threadIdx.x == 0) taken = atomicAdd(next, 1);
+            __syncthreads();
+            if (taken >= nl) break;
+            const int2 it = list[taken];
+            leaf_pass<T, TPL, G, kLW>(C, it.x, it.y, pts, surf, W, bufs, warp, res);
+        }
+    } else {
+        while (true) {
+            int li = 0;
+            if (lane == 0) li = atomicAdd(next, 1);
+            li = __shfl_sync(0xffffffffu, li, 0);
+            if (li >= nl) break;
+            const int2 it = list[li];
+            leaf_pass<T, TPL, G, 1>(C, it.x, it.y, pts, surf, W, bufs, warp, res);
+        }
     }
 }
 
@@ -1129,8 +1189,8 @@ void leaf_launch_variant(const Plan &P, const LeafCtx &C, int v, const typename 
     // on the variant's own stream, after the partition; joined back below
     cudaStream_t s = P.leaf_streams[v];
     cudaStreamWaitEvent(s, P.leaf_fork, 0);
-    constexpr int occ = sizeof(T) == 4 ? (TPL == 1 ? 5 : 4) : 2;
-    const int64_t want = (P.n_leaves + kLW - 1) / kLW;
+    constexpr int occ = leaf_blocks_per_sm<T>(TPL);
+    const int64_t want = sizeof(T) == 8 ? P.n_leaves : (P.n_leaves + kLW - 1) / kLW;
     const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)P.num_sms * occ));
     ++g_launches, k_leaf_all<T, TPL, G><<<g, 32 * kLW, 0, s>>>(C, P.leaf_vlist + (int64_t)v * P.leaf_item_cap,
                                                                 P.leaf_vcnt + v, P.leaf_vcnt + 8 + v, pts, surf,
@@ -1242,6 +1302,12 @@ inline unsigned grid_for(int64_t n, int block) { return (unsigned)((n + block - 
 
 // k_p2m launch shape: a thread per check point, four staged values per thread.
 inline int p2m_threads(const Plan &P) { return (P.ns + 31) / 32 * 32; }
+// k_p2l: a thread per check point and, in FP64, up to four source groups.
+template <typename T>
+inline int p2l_threads(const Plan &P) {
+    const int t = p2m_threads(P);
+    return sizeof(T) == 8 ? t * std::max(1, std::min(4, 640 / t)) : t;
+}
 template <typename T>
 inline size_t p2m_smem(const Plan &P) { return 7 * sizeof(T) * (size_t)p2m_threads(P); }
 
@@ -1486,10 +1552,9 @@ cudaError_t evaluate_t(Plan &P, void *pot, void *grad, double *energy, cudaStrea
     stage_end(P, KIFMM_STAGE_M2L, s);
     if (P.n_x > 0) {
         stage_begin(P, KIFMM_STAGE_P2L, s);
-        ++g_launches, k_p2l<T><<<(unsigned)P.nb, kLeafThreads, 0, s>>>(P.nx, P.xdense, P.lvl, P.cx, P.cy, P.cz,
-                                                                        P.first, P.cnt, pts, surf, ns, d, nullptr,
-                                                                        0, split_mean ? P.dbar : nullptr, nullptr,
-                                                                        P.periodic ? P.x_sh : nullptr);
+        ++g_launches, k_p2l<T><<<(unsigned)P.nb, p2l_threads<T>(P), 0, s>>>(
+                          p2m_threads(P), P.nx, P.xdense, P.lvl, P.cx, P.cy, P.cz, P.first, P.cnt, pts, surf, ns, d,
+                          nullptr, 0, split_mean ? P.dbar : nullptr, nullptr, P.periodic ? P.x_sh : nullptr);
         stage_end(P, KIFMM_STAGE_P2L, s);
     }
     // the root's upward check potential in FP64 (periodic cell)
@@ -2091,9 +2156,9 @@ cudaError_t backward_t(Plan &P, const void *w_user, const void *g_user, const do
     // M2P^T: W-list sources a receive h_a * sum w / |UE_a - x| (+ dipoles) from the leaves of X(a)
     if (P.n_x > 0) {
         KIFMM_CUDA_TRY(cudaMemsetAsync(e2, 0, sizeof(T) * (size_t)P.nb * ns, s));
-        ++g_launches, k_p2l<T><<<(unsigned)P.nb, kLeafThreads, 0, s>>>(P.nx, P.xdense, P.lvl, P.cx, P.cy, P.cz,
-                                                                        P.first, P.cnt, pts, surf, ns, e2, ws, 1,
-                                                                        nullptr, gs);
+        ++g_launches, k_p2l<T><<<(unsigned)P.nb, p2l_threads<T>(P), 0, s>>>(
+                          p2m_threads(P), P.nx, P.xdense, P.lvl, P.cx, P.cy, P.cz, P.first, P.cnt, pts, surf, ns, e2,
+                          ws, 1, nullptr, gs);
         ggemm<T>(P, GatherSelf<T>{adjp + 1 * nn}, P.part_list[2], 0, P.part_start[2][1], 1, e2, tmp, 0, s);
         ggemm<T>(P, GatherSelf<T>{adjp}, P.part_list[2], 0, P.part_start[2][1], 1, tmp, ub, 0, s);
     }

@@ -40,6 +40,7 @@ __host__ __device__ inline int leaf_variant(const LeafTiling &t, int n) { return
 // Candidate c of the tuner (c = 0 is the default): the variant for up to 8,
 // 16, 24, 32, 64 and more remaining targets.
 LeafTiling leaf_tiling_candidate(int c);
+LeafTiling leaf_tiling_f64();  // the FP64 mode's default
 
 struct DevBuf {
     void *ptr = nullptr;
