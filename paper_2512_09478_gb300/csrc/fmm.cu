@@ -1719,6 +1719,83 @@ __global__ void k_finalize_adj(int64_t n, const double4 *__restrict__ res, const
     }
 }
 
+// Sums of many terms: FP64 as they are, FP32 compensated (two-sum of every
+// term, about 48 bits), in place of FP64 sums of FP32 terms: ten of those per
+// pair, conversions included, kept the FP64 unit (two lanes per clock and SM)
+// busy for 2.4 ms on 100k particles.
+template <typename T>
+struct TermSum;
+template <>
+struct TermSum<double> {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double x) { s += x; }
+    __device__ __forceinline__ double total() const { return s; }
+};
+template <>
+struct TermSum<float> {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float x) {  // (no contraction into the term's own product)
+        const float t = __fadd_rn(s, x), bb = __fsub_rn(t, s);
+        c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(x, bb)));
+        s = t;
+    }
+    __device__ __forceinline__ double total() const { return (double)s + (double)c; }
+};
+
+// The U-list particles of leaf b, laid end to end and staged by the whole
+// block, kLeafThreads at a time: load(slot, particle, ox, oy, oz) stages one
+// (its leaf's centre relative to b's), body(m) sums m staged ones.
+template <typename T>
+struct UStage {
+    T ox[kLeafThreads], oy[kLeafThreads], oz[kLeafThreads];
+    int first[kLeafThreads], start[kLeafThreads + 1], wsum[kLeafThreads / 32];
+};
+template <typename T, class Load, class Body>
+__device__ __forceinline__ void for_u_sources(const LeafCtx &C, int b, UStage<T> &S, Load &&load, Body &&body) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int lb = C.lvl[b], bx = C.cx[b], by = C.cy[b], bz = C.cz[b];
+    const uint32_t u0 = C.u_ptr[b];
+    const int nu = (int)(C.u_ptr[b + 1] - u0);
+    for (int sb = 0; sb < nu; sb += kLeafThreads) {
+        __syncthreads();  // the previous batch is done with the segment arrays
+        int c = 0;
+        if (sb + tid < nu) {
+            const int a = C.u_idx[u0 + sb + tid], la = C.lvl[a];
+            S.ox[tid] = centre_diff<T>(C.cx[a], la, bx, lb);
+            S.oy[tid] = centre_diff<T>(C.cy[a], la, by, lb);
+            S.oz[tid] = centre_diff<T>(C.cz[a], la, bz, lb);
+            S.first[tid] = C.first[a];
+            c = C.cnt[a];
+        }
+        int incl = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        if (lane == 31) S.wsum[warp] = incl;
+        __syncthreads();
+        for (int w = 0; w < warp; ++w) incl += S.wsum[w];
+        S.start[tid + 1] = incl;
+        if (tid == 0) S.start[0] = 0;
+        __syncthreads();
+        const int total = S.start[kLeafThreads];
+        for (int c0 = 0; c0 < total; c0 += kLeafThreads) {
+            __syncthreads();
+            if (c0 + tid < total) {
+                int lo = 0, hi = kLeafThreads;  // the last segment that starts at or before c0 + tid
+                while (hi - lo > 1) {
+                    const int mid = (lo + hi) >> 1;
+                    if (S.start[mid] <= c0 + tid) lo = mid; else hi = mid;
+                }
+                load(tid, S.first[lo] + c0 + tid - S.start[lo], S.ox[lo], S.oy[lo], S.oz[lo]);
+            }
+            __syncthreads();
+            body(min(kLeafThreads, total - c0));
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------
 // The Stokeslet (the tensor kernel Eq. 1 admits; Stokes flow, Sec. 2.4):
 // G(r) = I / |r| + r r^T / |r|^3, the 1 / (8 pi) and coef applied at the
@@ -1818,81 +1895,102 @@ __global__ void k_p2l_stokes(const int32_t *__restrict__ nx, const int32_t *__re
 
 // Leaves: L2P (own downward density on the 2.95 h_b surface), M2P (the W
 // boxes' upward densities on their 1.05 h_a surfaces) and P2P (the U-list
-// particles' forces, r = 0 skipped); root units, FP64 sums; one block per
-// leaf, a thread per target.
+// particles' forces, r = 0 skipped); root units; one block per leaf, up to 32
+// targets at a time with the sources dealt out to its warps and lane groups as
+// in k_adj_leaf.
 template <typename T>
 __global__ void __launch_bounds__(kLeafThreads) k_leaf_stokes(LeafCtx C, const int32_t *__restrict__ leaves,
                                                               const typename Vec4<T>::type *__restrict__ pts,
                                                               const T *__restrict__ frc, const T *__restrict__ surf,
                                                               int npt, const T *__restrict__ dn_dens,
                                                               const T *__restrict__ up_dens, double4 *__restrict__ res) {
-    __shared__ T sx[kLeafThreads], sy[kLeafThreads], sz[kLeafThreads], sfx[kLeafThreads], sfy[kLeafThreads],
-        sfz[kLeafThreads];
+    using V4 = typename Vec4<T>::type;
+    __shared__ V4 src[kLeafThreads], sf[kLeafThreads];
+    __shared__ UStage<T> U;
+    __shared__ double red[kLeafThreads / 32 - 1][3][32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = leaves[blockIdx.x];
-    const int lb = C.lvl[b], n = C.cnt[b], f = C.first[b];
+    const int lb = C.lvl[b], bx = C.cx[b], by = C.cy[b], bz = C.cz[b], n = C.cnt[b], f = C.first[b];
     const T hb = box_half<T>(lb);
-    const uint32_t w0 = C.w_ptr[b], u0 = C.u_ptr[b];
-    const int nw = (int)(C.w_ptr[b + 1] - w0), nu = (int)(C.u_ptr[b + 1] - u0);
-    for (int t0 = 0; t0 < n; t0 += kLeafThreads) {
-        const int i = t0 + threadIdx.x;
+    const uint32_t w0 = C.w_ptr[b];
+    const int nw = (int)(C.w_ptr[b + 1] - w0);
+    for (int t0 = 0; t0 < n; t0 += 32) {
+        const int rest = min(32, n - t0);
+        const int ng = rest <= 8 ? 4 : (rest <= 16 ? 2 : 1), lg = 32 / ng;  // lane groups, lanes per group
+        const int grp = lane / lg, i = t0 + lane - grp * lg;
         const bool valid = i < n;
         T x = 0, y = 0, z = 0;
         if (valid) {
-            const auto v = pts[f + i];
+            const V4 v = pts[f + i];
             x = v.x, y = v.y, z = v.z;
         }
-        double vx = 0, vy = 0, vz = 0;
-        auto add = [&](T rx, T ry, T rz, T fx, T fy, T fz) {
-            T ux = 0, uy = 0, uz = 0;
-            stokes_acc<T>(rx, ry, rz, fx, fy, fz, ux, uy, uz);
-            vx += (double)ux, vy += (double)uy, vz += (double)uz;
+        TermSum<T> vx, vy, vz;
+        const int k_first = warp * ng + grp, k_step = ng * (kLeafThreads / 32);
+        auto add = [&](T rx, T ry, T rz, const V4 &w) {
+            const T r2 = rx * rx + ry * ry + rz * rz;
+            // the particle itself and coincident points add nothing
+            const T ri = r2 > T(0) ? rsqrt_t<T>(r2) : T(0);
+            const T rf = (rx * w.x + ry * w.y + rz * w.z) * (ri * ri * ri);
+            vx.add(w.x * ri + rx * rf);
+            vy.add(w.y * ri + ry * rf);
+            vz.add(w.z * ri + rz * rf);
         };
-        if (valid) {
-            const T a = (T)kAlphaOuter * hb;
-            for (int k = 0; k < npt; ++k) {
-                const T *w = dn_dens + (size_t)b * 3 * npt + 3 * k;
-                add(x - a * surf[3 * k], y - a * surf[3 * k + 1], z - a * surf[3 * k + 2], w[0] * hb, w[1] * hb,
-                    w[2] * hb);
+        auto sum = [&](int m) {
+            for (int k = k_first; k < m; k += k_step) {
+                const V4 v = src[k];
+                add(x - v.x, y - v.y, z - v.z, sf[k]);
             }
-            for (int e = 0; e < nw; ++e) {
-                const int a_ = C.w_idx[w0 + e], la = C.lvl[a_];
-                const T ha = box_half<T>(la), al = (T)kAlphaInner * ha;
-                const T ox = centre_diff<T>(C.cx[a_], la, C.cx[b], lb), oy = centre_diff<T>(C.cy[a_], la, C.cy[b], lb),
-                        oz = centre_diff<T>(C.cz[a_], la, C.cz[b], lb);
-                for (int k = 0; k < npt; ++k) {
-                    const T *w = up_dens + (size_t)a_ * 3 * npt + 3 * k;
-                    add(x - (ox + al * surf[3 * k]), y - (oy + al * surf[3 * k + 1]), z - (oz + al * surf[3 * k + 2]),
-                        w[0] * ha, w[1] * ha, w[2] * ha);
-                }
-            }
-        }
-        for (int e = 0; e < nu; ++e) {
-            const int a_ = C.u_idx[u0 + e], la = C.lvl[a_];
-            const T ox = centre_diff<T>(C.cx[a_], la, C.cx[b], lb), oy = centre_diff<T>(C.cy[a_], la, C.cy[b], lb),
-                    oz = centre_diff<T>(C.cz[a_], la, C.cz[b], lb);
-            const int na = C.cnt[a_], fa = C.first[a_];
-            for (int c0 = 0; c0 < na; c0 += kLeafThreads) {
+        };
+        // a surface of forces: points o + r S_k, forces h wts[3 k ..]
+        auto surface = [&](T ox, T oy, T oz, T r, const T *wts, T h) {
+            for (int c0 = 0; c0 < npt; c0 += kLeafThreads) {
                 __syncthreads();
-                if (c0 + threadIdx.x < na) {
-                    const int j = fa + c0 + threadIdx.x;
-                    const auto v = pts[j];
-                    sx[threadIdx.x] = ox + v.x, sy[threadIdx.x] = oy + v.y, sz[threadIdx.x] = oz + v.z;
-                    sfx[threadIdx.x] = frc[3 * (size_t)j], sfy[threadIdx.x] = frc[3 * (size_t)j + 1],
-                    sfz[threadIdx.x] = frc[3 * (size_t)j + 2];
+                const int k = c0 + tid;
+                if (k < npt) {
+                    V4 v, w;
+                    v.x = ox + r * surf[3 * k], v.y = oy + r * surf[3 * k + 1], v.z = oz + r * surf[3 * k + 2], v.w = T(0);
+                    w.x = wts[3 * k] * h, w.y = wts[3 * k + 1] * h, w.z = wts[3 * k + 2] * h, w.w = T(0);
+                    src[tid] = v;
+                    sf[tid] = w;
                 }
                 __syncthreads();
-                const int m = min(kLeafThreads, na - c0);
-                if (valid)
-                    for (int k = 0; k < m; ++k) {
-                        const T rx = x - sx[k], ry = y - sy[k], rz = z - sz[k];
-                        if (!(rx * rx + ry * ry + rz * rz > T(0))) continue;  // the particle itself, coincident points
-                        add(rx, ry, rz, sfx[k], sfy[k], sfz[k]);
-                    }
+                sum(min(kLeafThreads, npt - c0));
             }
+        };
+        surface(T(0), T(0), T(0), (T)kAlphaOuter * hb, dn_dens + (size_t)b * 3 * npt, hb);
+        for (int e = 0; e < nw; ++e) {
+            const int a = C.w_idx[w0 + e], la = C.lvl[a];
+            const T ha = box_half<T>(la);
+            surface(centre_diff<T>(C.cx[a], la, bx, lb), centre_diff<T>(C.cy[a], la, by, lb),
+                    centre_diff<T>(C.cz[a], la, bz, lb), (T)kAlphaInner * ha, up_dens + (size_t)a * 3 * npt, ha);
         }
-        if (valid) {
-            res[f + i] = make_double4(vx, vy, vz, 0.0);
-            if (!isfinite(vx + vy + vz)) set_status(C.status, KIFMM_ERR_NONFINITE);
+        for_u_sources<T>(
+            C, b, U,
+            [&](int slot, int j, T ox, T oy, T oz) {
+                const V4 v = pts[j];
+                V4 p, w;
+                p.x = ox + v.x, p.y = oy + v.y, p.z = oz + v.z, p.w = T(0);
+                w.x = frc[3 * (size_t)j], w.y = frc[3 * (size_t)j + 1], w.z = frc[3 * (size_t)j + 2], w.w = T(0);
+                src[slot] = p;
+                sf[slot] = w;
+            },
+            sum);
+        // lane groups, then warps, in order
+        double tot[3] = {vx.total(), vy.total(), vz.total()};
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            for (int o = 16; o >= lg; o >>= 1) tot[q] += __shfl_xor_sync(0xffffffffu, tot[q], o);
+        if (warp > 0) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) red[warp - 1][q][lane] = tot[q];
+        }
+        __syncthreads();
+        if (warp == 0 && grp == 0 && valid) {
+            for (int w = 0; w < kLeafThreads / 32 - 1; ++w)
+#pragma unroll
+                for (int q = 0; q < 3; ++q) tot[q] += red[w][q][lane];
+            res[f + i] = make_double4(tot[0], tot[1], tot[2], 0.0);
+            if (!isfinite(tot[0] + tot[1] + tot[2])) set_status(C.status, KIFMM_ERR_NONFINITE);
         }
     }
 }
@@ -2002,8 +2100,8 @@ __global__ void k_gather_g(int64_t n, const uint32_t *__restrict__ perm, const i
     for (int d = 0; d < 3; ++d) gs[3 * i + d] = (T)((double)g[3 * j + d] / side);
 }
 
-// The leaf-level terms of a loss on the gradient, one block per leaf b (its
-// targets in chunks of the block), root units, FP64 sums:
+// The leaf-level terms of a loss on the gradient, one block per leaf b, root
+// units:
 //  hg[i]  = H_i g_i, the Hessian of the forward field at particle i applied
 //           to its own dipole (the gradient's dependence on the particle's
 //           position), from b's forward sources: its downward equivalent
@@ -2013,96 +2111,120 @@ __global__ void k_gather_g(int64_t n, const uint32_t *__restrict__ perm, const i
 //           particles j != i (the near field of the transposed gradient).
 // With H = grad grad (1/r), r = x_i - y:  H g = (3 (r.g) r - r^2 g) / r^5;
 // a dipole g at y gives psi(x) = g . r / r^3, grad psi = g / r^3 - 3 (g.r) r / r^5.
+//
+// Some 85 FP32 operations per pair bound it.  Up to 32 targets at a time, one
+// per lane of every warp (8 or 16 targets: four or two lanes each), so that a
+// leaf of 24 uses all four warps: the sources (surfaces; then the U list's
+// particles laid end to end) are staged 128 at a time and dealt out to the
+// warps and lane groups, whose sums are added in order at the end.
 template <typename T>
 __global__ void __launch_bounds__(kLeafThreads) k_adj_leaf(LeafCtx C, const int32_t *__restrict__ leaves,
                                                            const typename Vec4<T>::type *__restrict__ pts,
                                                            const T *__restrict__ surf, const T *__restrict__ dn_dens,
                                                            const T *__restrict__ up_dens, const T *__restrict__ gs,
                                                            double4 *__restrict__ hg, double4 *__restrict__ pd) {
-    __shared__ T sx[kLeafThreads], sy[kLeafThreads], sz[kLeafThreads], sq[kLeafThreads];
-    __shared__ T sgx[kLeafThreads], sgy[kLeafThreads], sgz[kLeafThreads];
+    using V4 = typename Vec4<T>::type;
+    __shared__ V4 src[kLeafThreads], dip[kLeafThreads];
+    __shared__ UStage<T> U;
+    __shared__ double red[kLeafThreads / 32 - 1][7][32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = leaves[blockIdx.x];
-    const int lb = C.lvl[b], n = C.cnt[b], f = C.first[b], ns = C.ns;
+    const int lb = C.lvl[b], bx = C.cx[b], by = C.cy[b], bz = C.cz[b], n = C.cnt[b], f = C.first[b], ns = C.ns;
     const T hb = box_half<T>(lb);
-    const uint32_t w0 = C.w_ptr[b], u0 = C.u_ptr[b];
-    const int nw = (int)(C.w_ptr[b + 1] - w0), nu = (int)(C.u_ptr[b + 1] - u0);
-    for (int t0 = 0; t0 < n; t0 += kLeafThreads) {
-        const int i = t0 + threadIdx.x;
+    const uint32_t w0 = C.w_ptr[b];
+    const int nw = (int)(C.w_ptr[b + 1] - w0);
+    for (int t0 = 0; t0 < n; t0 += 32) {
+        const int rest = min(32, n - t0);
+        const int ng = rest <= 8 ? 4 : (rest <= 16 ? 2 : 1), lg = 32 / ng;  // lane groups, lanes per group
+        const int grp = lane / lg, i = t0 + lane - grp * lg;
         const bool valid = i < n;
         T x = 0, y = 0, z = 0, g0 = 0, g1 = 0, g2 = 0;
         if (valid) {
-            const auto v = pts[f + i];
+            const V4 v = pts[f + i];
             x = v.x, y = v.y, z = v.z;
             g0 = gs[3 * (size_t)(f + i)], g1 = gs[3 * (size_t)(f + i) + 1], g2 = gs[3 * (size_t)(f + i) + 2];
         }
-        double h0 = 0, h1 = 0, h2 = 0, p0 = 0, p1 = 0, p2 = 0, p3 = 0;
-        // Hessian of one monopole w at offset (rx, ry, rz) = x_i - y, applied to g
-        auto hess = [&](T rx, T ry, T rz, T w) {
-            const T r2 = rx * rx + ry * ry + rz * rz;
-            const T ri = rsqrt_t<T>(r2), ri2 = ri * ri, ri3 = ri * ri2;
+        TermSum<T> h0, h1, h2, p0, p1, p2, p3;
+        const int k_first = warp * ng + grp, k_step = ng * (kLeafThreads / 32);
+        // Hessian of one monopole w at offset r = x_i - y, applied to g
+        auto hess = [&](T rx, T ry, T rz, T w, T ri2, T ri3) {
             const T rg3 = T(3) * (rx * g0 + ry * g1 + rz * g2) * ri2;
-            h0 += (double)(w * ri3 * (rg3 * rx - g0));
-            h1 += (double)(w * ri3 * (rg3 * ry - g1));
-            h2 += (double)(w * ri3 * (rg3 * rz - g2));
+            h0.add(w * ri3 * (rg3 * rx - g0));
+            h1.add(w * ri3 * (rg3 * ry - g1));
+            h2.add(w * ri3 * (rg3 * rz - g2));
         };
-        if (valid) {
-            // own downward equivalent surface (weights dn_dens h_b)
-            const T a = (T)kAlphaOuter * hb;
-            for (int k = 0; k < ns; ++k)
-                hess(x - a * surf[3 * k], y - a * surf[3 * k + 1], z - a * surf[3 * k + 2],
-                     dn_dens[(size_t)b * ns + k] * hb);
-            // W boxes' upward equivalent surfaces (weights up_dens h_a)
-            for (int e = 0; e < nw; ++e) {
-                const int a_ = C.w_idx[w0 + e], la = C.lvl[a_];
-                const T ha = box_half<T>(la), al = (T)kAlphaInner * ha;
-                const T ox = centre_diff<T>(C.cx[a_], la, C.cx[b], lb), oy = centre_diff<T>(C.cy[a_], la, C.cy[b], lb),
-                        oz = centre_diff<T>(C.cz[a_], la, C.cz[b], lb);
-                for (int k = 0; k < ns; ++k)
-                    hess(x - (ox + al * surf[3 * k]), y - (oy + al * surf[3 * k + 1]), z - (oz + al * surf[3 * k + 2]),
-                         up_dens[(size_t)a_ * ns + k] * ha);
-            }
-        }
-        // U-list particles, staged through shared memory
-        for (int e = 0; e < nu; ++e) {
-            const int a_ = C.u_idx[u0 + e], la = C.lvl[a_];
-            const T ox = centre_diff<T>(C.cx[a_], la, C.cx[b], lb), oy = centre_diff<T>(C.cy[a_], la, C.cy[b], lb),
-                    oz = centre_diff<T>(C.cz[a_], la, C.cz[b], lb);
-            const int na = C.cnt[a_], fa = C.first[a_];
-            for (int c0 = 0; c0 < na; c0 += kLeafThreads) {
+        // a surface of monopoles: points o + r S_k, weights h wts[k]
+        auto surface = [&](T ox, T oy, T oz, T r, const T *wts, T h) {
+            for (int c0 = 0; c0 < ns; c0 += kLeafThreads) {
                 __syncthreads();
-                if (c0 + threadIdx.x < na) {
-                    const int j = fa + c0 + threadIdx.x;
-                    const auto v = pts[j];
-                    sx[threadIdx.x] = ox + v.x;
-                    sy[threadIdx.x] = oy + v.y;
-                    sz[threadIdx.x] = oz + v.z;
-                    sq[threadIdx.x] = v.w;
-                    sgx[threadIdx.x] = gs[3 * (size_t)j];
-                    sgy[threadIdx.x] = gs[3 * (size_t)j + 1];
-                    sgz[threadIdx.x] = gs[3 * (size_t)j + 2];
+                if (c0 + tid < ns) {
+                    V4 v;
+                    v.x = ox + r * surf[3 * (c0 + tid)];
+                    v.y = oy + r * surf[3 * (c0 + tid) + 1];
+                    v.z = oz + r * surf[3 * (c0 + tid) + 2];
+                    v.w = wts[c0 + tid] * h;
+                    src[tid] = v;
                 }
                 __syncthreads();
-                const int m = min(kLeafThreads, na - c0);
-                if (valid) {
-                    for (int k = 0; k < m; ++k) {
-                        const T rx = x - sx[k], ry = y - sy[k], rz = z - sz[k];
-                        const T r2 = rx * rx + ry * ry + rz * rz;
-                        if (!(r2 > T(0))) continue;  // the particle itself and coincident points
-                        hess(rx, ry, rz, sq[k]);
-                        const T ri = rsqrt_t<T>(r2), ri2 = ri * ri, ri3 = ri * ri2;
-                        const T gr = sgx[k] * rx + sgy[k] * ry + sgz[k] * rz;
-                        const T gr3 = T(3) * gr * ri2;
-                        p0 += (double)(gr * ri3);
-                        p1 += (double)(ri3 * (sgx[k] - gr3 * rx));
-                        p2 += (double)(ri3 * (sgy[k] - gr3 * ry));
-                        p3 += (double)(ri3 * (sgz[k] - gr3 * rz));
-                    }
+                const int m = min(kLeafThreads, ns - c0);
+                for (int k = k_first; k < m; k += k_step) {
+                    const V4 v = src[k];
+                    const T rx = x - v.x, ry = y - v.y, rz = z - v.z;
+                    const T ri = rsqrt_t<T>(rx * rx + ry * ry + rz * rz), ri2 = ri * ri;
+                    hess(rx, ry, rz, v.w, ri2, ri * ri2);
                 }
             }
+        };
+        // own downward equivalent surface (weights dn_dens h_b), then the W
+        // boxes' upward equivalent surfaces (weights up_dens h_a)
+        surface(T(0), T(0), T(0), (T)kAlphaOuter * hb, dn_dens + (size_t)b * ns, hb);
+        for (int e = 0; e < nw; ++e) {
+            const int a_ = C.w_idx[w0 + e], la = C.lvl[a_];
+            const T ha = box_half<T>(la);
+            surface(centre_diff<T>(C.cx[a_], la, bx, lb), centre_diff<T>(C.cy[a_], la, by, lb),
+                    centre_diff<T>(C.cz[a_], la, bz, lb), (T)kAlphaInner * ha, up_dens + (size_t)a_ * ns, ha);
         }
-        if (valid) {
-            hg[f + i] = make_double4(h0, h1, h2, 0.0);
-            pd[f + i] = make_double4(p0, p1, p2, p3);
+        for_u_sources<T>(
+            C, b, U,
+            [&](int slot, int j, T ox, T oy, T oz) {
+                const V4 v = pts[j];
+                V4 p, d;
+                p.x = ox + v.x, p.y = oy + v.y, p.z = oz + v.z, p.w = v.w;
+                d.x = gs[3 * (size_t)j], d.y = gs[3 * (size_t)j + 1], d.z = gs[3 * (size_t)j + 2], d.w = T(0);
+                src[slot] = p;
+                dip[slot] = d;
+            },
+            [&](int m) {
+                for (int k = k_first; k < m; k += k_step) {
+                    const V4 v = src[k], d = dip[k];
+                    const T rx = x - v.x, ry = y - v.y, rz = z - v.z;
+                    const T r2 = rx * rx + ry * ry + rz * rz;
+                    // the particle itself and coincident points add nothing
+                    const T ri = r2 > T(0) ? rsqrt_t<T>(r2) : T(0), ri2 = ri * ri, ri3 = ri * ri2;
+                    hess(rx, ry, rz, v.w, ri2, ri3);
+                    const T gr = d.x * rx + d.y * ry + d.z * rz;
+                    const T gr3 = T(3) * gr * ri2;
+                    p0.add(gr * ri3);
+                    p1.add(ri3 * (d.x - gr3 * rx));
+                    p2.add(ri3 * (d.y - gr3 * ry));
+                    p3.add(ri3 * (d.z - gr3 * rz));
+                }
+            });
+        // lane groups, then warps, in order
+        double tot[7] = {h0.total(), h1.total(), h2.total(), p0.total(), p1.total(), p2.total(), p3.total()};
+#pragma unroll
+        for (int q = 0; q < 7; ++q)
+            for (int o = 16; o >= lg; o >>= 1) tot[q] += __shfl_xor_sync(0xffffffffu, tot[q], o);
+        if (warp > 0)
+#pragma unroll
+            for (int q = 0; q < 7; ++q) red[warp - 1][q][lane] = tot[q];
+        __syncthreads();
+        if (warp == 0 && grp == 0 && valid) {
+            for (int w = 0; w < kLeafThreads / 32 - 1; ++w)
+#pragma unroll
+                for (int q = 0; q < 7; ++q) tot[q] += red[w][q][lane];
+            hg[f + i] = make_double4(tot[0], tot[1], tot[2], 0.0);
+            pd[f + i] = make_double4(tot[3], tot[4], tot[5], tot[6]);
         }
     }
 }
