@@ -286,6 +286,7 @@ kifmm_status kifmm_plan_create(const kifmm_plan_desc *desc, kifmm_plan **out) {
     if (cudaGetDevice(&P.device) != cudaSuccess) return fail(KIFMM_ERR_CUDA);
     cudaDeviceGetAttribute(&P.num_sms, cudaDevAttrMultiProcessorCount, P.device);
     std::string err;
+    if (rows_setup() != cudaSuccess) return fail(KIFMM_ERR_CUDA);
     cudaError_t e = build_operators(P, err);
     if (e == cudaErrorInvalidValue) return fail(KIFMM_ERR_ARG);
     if (e != cudaSuccess) return fail(KIFMM_ERR_CUDA);
@@ -320,7 +321,6 @@ kifmm_status kifmm_plan_create(const kifmm_plan_desc *desc, kifmm_plan **out) {
         {(void **)&P.adj_hg, sizeof(double) * 4 * n},
         {(void **)&P.adj_pd, sizeof(double) * 4 * n},
         {(void **)&P.adj_pot, sizeof(double) * n},
-        {&P.gemm_part, esz * 8 * kSplitTargets * (size_t)(P.ns + 1)},
         {(void **)&P.sys_off_d, sizeof(int64_t) * (P.sys_cap + 1)},
         {(void **)&P.lo_side, sizeof(double) * 4 * P.sys_cap},
         {(void **)&P.key_scale, sizeof(double) * P.sys_cap},

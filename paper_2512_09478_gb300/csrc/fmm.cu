@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "gemm_rows.cuh"
 #include "internal.h"
 
 namespace kifmm {
@@ -279,164 +280,95 @@ __global__ void __launch_bounds__(1024, 1)
 }
 
 // ---------------------------------------------------------------------------
-// Gathered, class-tiled GEMM on SIMT cores:
-//   out[t] (=|+=) sum_{s < nslots} Op_s  in[src(t, s)]
-// for a list of targets.  A block owns 64 targets and all outputs (padded to
-// 160); each thread keeps an 8 x 5 register tile (targets 8 ty .. 8 ty + 7,
-// outputs tx + 32 c).  Operators are stored transposed ([k][j]); k advances in
-// chunks of 8 through shared memory with the next chunk prefetched into
-// registers.  Used for M2M (8 child octants), L2L (parent) and the two factors
-// of the leaf pseudo-inverses.
+// Gathered row products in FP64 (FP32: gemm_rows.cuh), out[t] (=|+=) Op
+// in[src(t)]: a block owns NTY RT rows of one class and 32 RC outputs; thread
+// (tx, ty) keeps rows RT ty .. RT ty + RT - 1 by outputs tx + 32 c.  Operators
+// are stored transposed ([k][n]); k advances in chunks of 16 through shared
+// memory with the next chunk prefetched into registers.  Bound by the FP64
+// unit (two lanes per clock and SM).
 // ---------------------------------------------------------------------------
 constexpr int kGK = 16;
 
-// Target ranges of up to 8 classes (blockIdx.y = class) in one launch.
-struct ClassRanges {
-    int64_t b[9];
-};
-
-// Operator blocks are [k][ld]: ld = n_s, or n_s + 1 when column n_s holds the
-// mean row of a mean-free check-to-check block (FP32-based modes).
-template <typename T>
-struct GatherChild {
-    const int32_t *child8;
-    const T *ops;
-    int ns;
-    __device__ int src(int t, int s, int) const { return child8[(size_t)t * 8 + s]; }
-    __device__ const T *op(int s, int) const { return ops + (size_t)s * ns * ns; }
-    __device__ double mean_base(int, const double *) const { return 0.0; }
-};
-// One operator per class (L2L: the octant of the child); the child inherits
-// the parent's mean.
-template <typename T>
-struct GatherParent {
-    const int32_t *parent;
-    const T *ops;
-    int ns, ld;
-    __device__ int src(int t, int, int) const { return parent[t]; }
-    __device__ const T *op(int, int cls) const { return ops + (size_t)cls * ns * ld; }
-    __device__ double mean_base(int t, const double *dbar) const { return dbar[parent[t]]; }
-};
-template <typename T>
-struct GatherSelf {
-    const T *op0;
-    __device__ int src(int t, int, int) const { return t; }
-    __device__ const T *op(int, int) const { return op0; }
-    __device__ double mean_base(int, const double *) const { return 0.0; }
-};
-
-// With dbar: output column n_s (operator column n_s, the mean row) goes to
-// dbar[t] (FP64, plus the functor's mean_base) instead of out.
-// Tile: NTY warps; thread (tx, ty) owns targets RT ty .. RT ty + RT-1 and
-// outputs tx + 32 c (c < RC): TT = NTY RT targets by TJ = 32 RC outputs.
-// SPLIT: blockIdx.z = slot * ncb + column block; the block writes that
-// slot's partial product to part ([slot][target position][ld]) and
-// k_ggemm_sum adds the slots in order (the same arithmetic as the unsplit
-// form; used for the small-tile M2M levels, whose latency is otherwise
-// 8 slots x n_s / 16 dependent steps per block).
-// MULTI: more than one slot per block (FP32 then keeps per-slot partials and
-// running sums); single-slot launches need half the accumulator registers
-// and run two 256-thread blocks per SM.
-template <typename T, class G, int NTY, int RT, int RC, bool SPLIT, bool MULTI>
-__global__ void __launch_bounds__(32 * NTY, (sizeof(T) == 4 && NTY == 8 && !MULTI) ? 2 : 1) k_ggemm(G g, const int32_t *__restrict__ targets, ClassRanges cr,
-                                                    int nslots, int ns, int ld, const T *__restrict__ in,
-                                                    T *__restrict__ out, int accumulate, double *dbar, int ncb,
-                                                    T *__restrict__ part) {
+template <int NTY, int RT, int RC>
+__global__ void __launch_bounds__(32 * NTY) k_rows_f64(RowMap<double> g, const int32_t *__restrict__ targets,
+                                                       ClassRanges cr, int n, const double *__restrict__ in,
+                                                       double *out, int accumulate) {
     constexpr int TT = NTY * RT, TJ = 32 * RC, NT = 32 * NTY;
-    __shared__ __align__(16) T Us[kGK][TT];
-    __shared__ __align__(16) T Ms[kGK][TJ];
+    __shared__ __align__(16) double Us[kGK][TT];
+    __shared__ __align__(16) double Ms[kGK][TJ];
     __shared__ int32_t tgt[TT];
     __shared__ int32_t src[TT];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int cls = blockIdx.y;
-    const int j0 = (SPLIT ? (int)blockIdx.z % ncb : (int)blockIdx.z) * TJ;  // output columns [j0, j0 + TJ)
-    const int s_lo = SPLIT ? (int)blockIdx.z / ncb : 0, s_hi = SPLIT ? s_lo + 1 : nslots;
+    const int j0 = (int)blockIdx.z * TJ;  // output columns [j0, j0 + TJ)
     int64_t t_begin = 0, t_end = 0;
 #pragma unroll
     for (int c = 0; c < 8; ++c)
-        if (c == cls) {
-            t_begin = cr.b[c];
-            t_end = cr.b[c + 1];
-        }
+        if (c == cls) t_begin = cr.b[c], t_end = cr.b[c + 1];
     const int64_t t0 = t_begin + (int64_t)blockIdx.x * TT;
     if (t0 >= t_end) return;  // uniform for the block
-    if (threadIdx.x < TT) tgt[threadIdx.x] = (t0 + threadIdx.x < t_end) ? targets[t0 + threadIdx.x] : -1;
-    // FP32: each slot sums into a fresh partial that is then added to the
-    // running total, so no rounding chain is longer than one slot's n_s terms.
-    constexpr bool kTwoLevel = sizeof(T) == 4 && MULTI;
-    T acc[RT][RC], run[RT][RC];
+    if (threadIdx.x < TT) {
+        const int32_t t = (t0 + threadIdx.x < t_end) ? targets[t0 + threadIdx.x] : -1;
+        tgt[threadIdx.x] = t;
+        src[threadIdx.x] = t >= 0 ? g.src(t) : -1;
+    }
+    double acc[RT][RC];
 #pragma unroll
     for (int a = 0; a < RT; ++a)
 #pragma unroll
-        for (int c = 0; c < RC; ++c) acc[a][c] = run[a][c] = T(0);
-    const int nk = (ns + kGK - 1) / kGK;
+        for (int c = 0; c < RC; ++c) acc[a][c] = 0.0;
+    const int nk = (n + kGK - 1) / kGK;
+    const double *M = g.op(cls);
     __syncthreads();
-    for (int s = s_lo; s < s_hi; ++s) {
-        if (threadIdx.x < TT) {
-            const int32_t t = tgt[threadIdx.x];
-            src[threadIdx.x] = (t >= 0) ? g.src(t, s, cls) : -1;
+    constexpr int kRU = (TT * kGK + NT - 1) / NT, kRM = (kGK * TJ + NT - 1) / NT;
+    double ru[kRU], rm[kRM];
+    auto load = [&](int kc) {
+        const int k0 = kc * kGK;
+#pragma unroll
+        for (int r = 0; r < kRU; ++r) {
+            const int e = threadIdx.x + NT * r;
+            const int t = e / kGK, k = e % kGK;
+            ru[r] = 0.0;
+            if (t < TT) {
+                const int32_t sb = src[t];
+                if (sb >= 0 && k0 + k < n) ru[r] = in[(size_t)sb * n + k0 + k];
+            }
         }
-        const T *M = g.op(s, cls);
+#pragma unroll
+        for (int r = 0; r < kRM; ++r) {
+            const int e = threadIdx.x + NT * r;
+            const int k = e / TJ, j = e - k * TJ;
+            rm[r] = (k < kGK && k0 + k < n && j0 + j < n) ? M[(size_t)(k0 + k) * n + j0 + j] : 0.0;
+        }
+    };
+    load(0);
+    for (int kc = 0; kc < nk; ++kc) {
+#pragma unroll
+        for (int r = 0; r < kRU; ++r) {
+            const int e = threadIdx.x + NT * r;
+            if (e < TT * kGK) Us[e % kGK][e / kGK] = ru[r];
+        }
+#pragma unroll
+        for (int r = 0; r < kRM; ++r) {
+            const int e = threadIdx.x + NT * r;
+            const int k = e / TJ;
+            if (k < kGK) Ms[k][e - k * TJ] = rm[r];
+        }
         __syncthreads();
-        constexpr int kRU = (TT * kGK + NT - 1) / NT, kRM = (kGK * TJ + NT - 1) / NT;
-        T ru[kRU], rm[kRM];
-        auto load = [&](int kc) {
-            const int k0 = kc * kGK;
+        if (kc + 1 < nk) load(kc + 1);
 #pragma unroll
-            for (int r = 0; r < kRU; ++r) {
-                const int e = threadIdx.x + NT * r;
-                const int t = e / kGK, k = e % kGK;
-                ru[r] = T(0);
-                if (t < TT) {
-                    const int32_t sb = src[t];
-                    if (sb >= 0 && k0 + k < ns) ru[r] = in[(size_t)sb * ns + k0 + k];
-                }
-            }
+        for (int k = 0; k < kGK; ++k) {
+            double uv[RT], mv[RC];
 #pragma unroll
-            for (int r = 0; r < kRM; ++r) {
-                const int e = threadIdx.x + NT * r;
-                const int k = e / TJ, j = e - k * TJ;
-                rm[r] = (k < kGK && k0 + k < ns && j0 + j < ld) ? M[(size_t)(k0 + k) * ld + j0 + j] : T(0);
-            }
-        };
-        load(0);
-        for (int kc = 0; kc < nk; ++kc) {
+            for (int a = 0; a < RT; ++a) uv[a] = Us[k][RT * ty + a];
 #pragma unroll
-            for (int r = 0; r < kRU; ++r) {
-                const int e = threadIdx.x + NT * r;
-                if (e < TT * kGK) Us[e % kGK][e / kGK] = ru[r];
-            }
-#pragma unroll
-            for (int r = 0; r < kRM; ++r) {
-                const int e = threadIdx.x + NT * r;
-                const int k = e / TJ;
-                if (k < kGK) Ms[k][e - k * TJ] = rm[r];
-            }
-            __syncthreads();
-            if (kc + 1 < nk) load(kc + 1);
-#pragma unroll
-            for (int k = 0; k < kGK; ++k) {
-                T uv[RT], mv[RC];
-#pragma unroll
-                for (int a = 0; a < RT; ++a) uv[a] = Us[k][RT * ty + a];
-#pragma unroll
-                for (int c = 0; c < RC; ++c) mv[c] = Ms[k][tx + 32 * c];
-#pragma unroll
-                for (int a = 0; a < RT; ++a)
-#pragma unroll
-                    for (int c = 0; c < RC; ++c) acc[a][c] += uv[a] * mv[c];
-            }
-            __syncthreads();
-        }
-        if constexpr (kTwoLevel) {
+            for (int c = 0; c < RC; ++c) mv[c] = Ms[k][tx + 32 * c];
 #pragma unroll
             for (int a = 0; a < RT; ++a)
 #pragma unroll
-                for (int c = 0; c < RC; ++c) {
-                    run[a][c] += acc[a][c];
-                    acc[a][c] = T(0);
-                }
+                for (int c = 0; c < RC; ++c) acc[a][c] += uv[a] * mv[c];
         }
+        __syncthreads();
     }
 #pragma unroll
     for (int a = 0; a < RT; ++a) {
@@ -445,181 +377,33 @@ __global__ void __launch_bounds__(32 * NTY, (sizeof(T) == 4 && NTY == 8 && !MULT
 #pragma unroll
         for (int c = 0; c < RC; ++c) {
             const int j = j0 + tx + 32 * c;
-            const T v = kTwoLevel ? run[a][c] : acc[a][c];
-            if constexpr (SPLIT) {
-                if (j < ld)
-                    part[((size_t)s_lo * (size_t)(cr.b[gridDim.y] - cr.b[0]) + (size_t)(t0 + RT * ty + a - cr.b[0])) * ld +
-                         j] = v;
-            } else if (j < ns) {
-                T *o = out + (size_t)t * ns + j;
-                *o = accumulate ? *o + v : v;
-            } else if (j == ns && dbar) {
-                dbar[t] = (accumulate ? dbar[t] : 0.0) + (double)v + g.mean_base(t, dbar);
-            }
+            if (j >= n) continue;
+            double *o = out + (size_t)t * n + j;
+            *o = accumulate ? *o + acc[a][c] : acc[a][c];
         }
     }
 }
 
-// FP32 big tiles with vector shared-memory reads: 64 targets x 160 outputs
-// per 320-thread block; thread (tn = t % 40, tm = t / 40) owns outputs
-// 4 tn .. 4 tn + 3 and targets 8 tm .. 8 tm + 7, so each k step reads one
-// float4 of the operator and two of the gathered inputs for 32 FMAs (the
-// scalar tile above reads 13 values for 40).  The sums run over k in the same
-// order, one fresh partial per slot, so the results equal the scalar form's
-// bit for bit.  VEC: the input rows are 16-byte aligned (n_s a multiple of 4)
-// and are read as float4.
-constexpr int kV4Threads = 320;
-// SPLIT: blockIdx.z = slot * ncb + column block, the slot's partial product
-// to part ([slot][target position][ld]) as in the scalar tile's split form.
-template <class G, bool MULTI, bool VEC, bool SPLIT = false>
-__global__ void __launch_bounds__(kV4Threads, 2) k_ggemm_v4(G g, const int32_t *__restrict__ targets,
-                                                            ClassRanges cr, int nslots, int ns, int ld,
-                                                            const float *__restrict__ in, float *__restrict__ out,
-                                                            int accumulate, double *dbar, int ncb = 1,
-                                                            float *__restrict__ part = nullptr) {
-    constexpr int TT = 64, TJ = 160;
-    __shared__ __align__(16) float Us[kGK][TT];
-    __shared__ __align__(16) float Ms[kGK][TJ];
-    __shared__ int32_t tgt[TT];
-    __shared__ int32_t src[TT];
-    const int tid = threadIdx.x;
-    const int tn = tid % 40, tm = tid / 40;
-    const int cls = blockIdx.y;
-    const int j0 = (SPLIT ? (int)blockIdx.z % ncb : (int)blockIdx.z) * TJ;
-    const int s_lo = SPLIT ? (int)blockIdx.z / ncb : 0, s_hi = SPLIT ? s_lo + 1 : nslots;
-    int64_t t_begin = 0, t_end = 0;
-#pragma unroll
-    for (int c = 0; c < 8; ++c)
-        if (c == cls) {
-            t_begin = cr.b[c];
-            t_end = cr.b[c + 1];
-        }
-    const int64_t t0 = t_begin + (int64_t)blockIdx.x * TT;
-    if (t0 >= t_end) return;  // uniform for the block
-    if (tid < TT) tgt[tid] = (t0 + tid < t_end) ? targets[t0 + tid] : -1;
-    float acc[8][4], run[8][4];
-#pragma unroll
-    for (int a = 0; a < 8; ++a)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc[a][c] = run[a][c] = 0.f;
-    const int nk = (ns + kGK - 1) / kGK;
-    __syncthreads();
-    for (int s = s_lo; s < s_hi; ++s) {
-        if (tid < TT) {
-            const int32_t t = tgt[tid];
-            src[tid] = (t >= 0) ? g.src(t, s, cls) : -1;
-        }
-        const float *M = g.op(s, cls);
-        __syncthreads();
-        // staged values: inputs as (target = e % 64, k quad = e / 64), four
-        // k values each; operator rows as (k, j) with j fastest
-        constexpr int kRM = kGK * TJ / kV4Threads;  // 8
-        float4 ru = make_float4(0.f, 0.f, 0.f, 0.f);
-        float rm[kRM];
-        auto load = [&](int kc) {
-            const int k0 = kc * kGK;
-            if (tid < TT * (kGK / 4)) {
-                const int t = tid % TT, k = 4 * (tid / TT);
-                const int32_t sb = src[t];
-                ru = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (sb >= 0) {
-                    const float *row = in + (size_t)sb * ns + k0 + k;
-                    if (VEC && k0 + k + 3 < ns) {
-                        ru = *reinterpret_cast<const float4 *>(row);
-                    } else {
-                        if (k0 + k < ns) ru.x = row[0];
-                        if (k0 + k + 1 < ns) ru.y = row[1];
-                        if (k0 + k + 2 < ns) ru.z = row[2];
-                        if (k0 + k + 3 < ns) ru.w = row[3];
-                    }
-                }
-            }
-#pragma unroll
-            for (int r = 0; r < kRM; ++r) {
-                const int e = tid + kV4Threads * r;
-                const int k = e / TJ, j = e - k * TJ;
-                rm[r] = (k0 + k < ns && j0 + j < ld) ? M[(size_t)(k0 + k) * ld + j0 + j] : 0.f;
-            }
-        };
-        load(0);
-        for (int kc = 0; kc < nk; ++kc) {
-            if (tid < TT * (kGK / 4)) {
-                const int t = tid % TT, k = 4 * (tid / TT);
-                Us[k][t] = ru.x;
-                Us[k + 1][t] = ru.y;
-                Us[k + 2][t] = ru.z;
-                Us[k + 3][t] = ru.w;
-            }
-#pragma unroll
-            for (int r = 0; r < kRM; ++r) {
-                const int e = tid + kV4Threads * r;
-                Ms[e / TJ][e % TJ] = rm[r];
-            }
-            __syncthreads();
-            if (kc + 1 < nk) load(kc + 1);
-#pragma unroll
-            for (int k = 0; k < kGK; ++k) {
-                const float4 u0 = *reinterpret_cast<const float4 *>(&Us[k][8 * tm]);
-                const float4 u1 = *reinterpret_cast<const float4 *>(&Us[k][8 * tm + 4]);
-                const float4 m = *reinterpret_cast<const float4 *>(&Ms[k][4 * tn]);
-                const float uv[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
-                const float mv[4] = {m.x, m.y, m.z, m.w};
-#pragma unroll
-                for (int a = 0; a < 8; ++a)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) acc[a][c] += uv[a] * mv[c];
-            }
-            __syncthreads();
-        }
-        if constexpr (MULTI) {
-#pragma unroll
-            for (int a = 0; a < 8; ++a)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    run[a][c] += acc[a][c];
-                    acc[a][c] = 0.f;
-                }
-        }
-    }
-#pragma unroll
-    for (int a = 0; a < 8; ++a) {
-        const int32_t t = tgt[8 * tm + a];
-        if (t < 0) continue;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int j = j0 + 4 * tn + c;
-            const float v = MULTI ? run[a][c] : acc[a][c];
-            if constexpr (SPLIT) {
-                if (j < ld)
-                    part[((size_t)s_lo * (size_t)(cr.b[gridDim.y] - cr.b[0]) + (size_t)(t0 + 8 * tm + a - cr.b[0])) *
-                             ld + j] = v;
-            } else if (j < ns) {
-                float *o = out + (size_t)t * ns + j;
-                *o = accumulate ? *o + v : v;
-            } else if (j == ns && dbar) {
-                dbar[t] = (accumulate ? dbar[t] : 0.0) + (double)v + g.mean_base(t, dbar);
-            }
-        }
-    }
-}
-
-// Slot-split form: out = the in-order sum of the slots' partial products.
-template <typename T, class G>
-__global__ void k_ggemm_sum(G g, const int32_t *__restrict__ targets, int64_t t_first, int64_t n_t, int nslots, int ns,
-                            int ld, const T *__restrict__ part, T *__restrict__ out, int accumulate, double *dbar) {
+// out[parent] (=|+=) the sum of its children's rows, in octant order (M2M and
+// the adjoint of L2L: the children's products come from one row product over
+// all children of a level, grouped by octant, so that absent children cost
+// nothing).
+template <typename T>
+__global__ void k_child_sum(const int32_t *__restrict__ parents, int64_t n_p, int n, const int32_t *__restrict__ child8,
+                            const T *__restrict__ prod, T *__restrict__ out, int accumulate) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n_t * ld) return;
-    const int64_t i = idx / ld;
-    const int j = (int)(idx - i * ld);
+    if (idx >= n_p * n) return;
+    const int64_t i = idx / n;
+    const int j = (int)(idx - i * n);
+    const int32_t t = parents[i];
     T v = T(0);
-    for (int s = 0; s < nslots; ++s) v += part[((size_t)s * n_t + i) * ld + j];
-    const int32_t t = targets[t_first + i];
-    if (j < ns) {
-        T *o = out + (size_t)t * ns + j;
-        *o = accumulate ? *o + v : v;
-    } else if (j == ns && dbar) {
-        dbar[t] = (accumulate ? dbar[t] : 0.0) + (double)v + g.mean_base(t, dbar);
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+        const int32_t c = child8[(size_t)t * 8 + s];
+        if (c >= 0) v += prod[(size_t)c * n + j];
     }
+    T *o = out + (size_t)t * n + j;
+    *o = accumulate ? *o + v : v;
 }
 
 // ---------------------------------------------------------------------------
@@ -1311,94 +1095,91 @@ inline int p2l_threads(const Plan &P) {
 template <typename T>
 inline size_t p2m_smem(const Plan &P) { return 7 * sizeof(T) * (size_t)p2m_threads(P); }
 
-// Classes c < ncls own targets [starts[c], starts[c + 1]); one launch.
-template <typename T, class G>
-void ggemm_classes(Plan &P, const G &g, const int32_t *targets, const int64_t *starts, int ncls, int nslots,
-                   const T *in, T *out, int accumulate, cudaStream_t s, int ld = 0, double *dbar = nullptr) {
+// FP32 operator block of n inputs and ld outputs (padded), FP64 [n][n].
+template <typename T>
+inline int64_t op_block(int n, int ld) {
+    return sizeof(T) == 4 ? (int64_t)gemm_nkp(n) * gemm_ldp(ld) : (int64_t)n * n;
+}
+
+template <bool VEC>
+void rows_launch_f32(const RowMap<float> &g, const int32_t *targets, const ClassRanges &cr, int64_t most, int ncls,
+                     bool big, int n, int ld, const float *in, float *out, int accumulate, double *dbar,
+                     cudaStream_t s) {
+    const int nkp = gemm_nkp(n), ldp = gemm_ldp(ld), nc = gemm_nc(ld);
+    if (!big) {
+        const dim3 grid(grid_for(most, kSmallRows), ncls, grid_for(ld, kSmallCols));
+        ++g_launches, k_rows_small<VEC><<<grid, kRThreads, rows_small_smem(nkp), s>>>(g, targets, cr, n, nkp, ldp, in,
+                                                                                     out, accumulate, dbar);
+        return;
+    }
+    const dim3 grid(grid_for(most, 64), ncls, ldp / (32 * nc));
+    switch (nc) {
+        case 1: ++g_launches, k_rows_big<1, VEC><<<grid, kRThreads, 0, s>>>(g, targets, cr, n, nkp, ldp, in, out, accumulate, dbar); break;
+        case 2: ++g_launches, k_rows_big<2, VEC><<<grid, kRThreads, 0, s>>>(g, targets, cr, n, nkp, ldp, in, out, accumulate, dbar); break;
+        case 3: ++g_launches, k_rows_big<3, VEC><<<grid, kRThreads, 0, s>>>(g, targets, cr, n, nkp, ldp, in, out, accumulate, dbar); break;
+        case 4: ++g_launches, k_rows_big<4, VEC><<<grid, kRThreads, 0, s>>>(g, targets, cr, n, nkp, ldp, in, out, accumulate, dbar); break;
+        default: ++g_launches, k_rows_big<5, VEC><<<grid, kRThreads, 0, s>>>(g, targets, cr, n, nkp, ldp, in, out, accumulate, dbar); break;
+    }
+}
+
+// out[t] (=|+=) Op in[src(t)] for the rows targets[starts[c] .. starts[c + 1])
+// of class c < ncls; ld = n, or n + 1 with the mean row (FP32-based modes).
+// The big tile once its blocks fill the GPU, the small one below (a level of
+// few boxes is latency-bound).
+template <typename T>
+void rows(Plan &P, const RowMap<T> &g, const int32_t *targets, const int64_t *starts, int ncls, const T *in, T *out,
+          int accumulate, cudaStream_t s, int ld = 0, double *dbar = nullptr) {
     ClassRanges cr;
     int64_t most = 0, total = 0;
-    for (int c = 0; c <= ncls; ++c) cr.b[c] = starts[c];
+    for (int c = 0; c <= 8; ++c) cr.b[c] = starts[std::min(c, ncls)];
     for (int c = 0; c < ncls; ++c) {
         most = std::max<int64_t>(most, starts[c + 1] - starts[c]);
         total += starts[c + 1] - starts[c];
     }
     if (most <= 0) return;
-    if (ld == 0) ld = P.ns;
-    // 64 x 160 tiles while they fill the GPU twice over; else 16 x 32 tiles
-    // (the coarse levels of M2M / L2L and small trees are latency-bound),
-    // with up to 8 slots split over blocks for up to kSplitTargets targets.
-    const int64_t big_blocks = grid_for(total, 64) * grid_for(ld, 160);
-    if (big_blocks >= 2 * P.num_sms) {
-        dim3 grid(grid_for(most, 64), ncls, grid_for(ld, 160));
-        if constexpr (sizeof(T) == 4) {
-            const bool vec = P.ns % 4 == 0;
-            if (nslots > 1 && vec)
-                ++g_launches, k_ggemm_v4<G, true, true><<<grid, kV4Threads, 0, s>>>(g, targets, cr, nslots, P.ns, ld,
-                                                                                   in, out, accumulate, dbar);
-            else if (nslots > 1)
-                ++g_launches, k_ggemm_v4<G, true, false><<<grid, kV4Threads, 0, s>>>(g, targets, cr, nslots, P.ns,
-                                                                                    ld, in, out, accumulate, dbar);
-            else if (vec)
-                ++g_launches, k_ggemm_v4<G, false, true><<<grid, kV4Threads, 0, s>>>(g, targets, cr, nslots, P.ns,
-                                                                                    ld, in, out, accumulate, dbar);
-            else
-                ++g_launches, k_ggemm_v4<G, false, false><<<grid, kV4Threads, 0, s>>>(g, targets, cr, nslots, P.ns,
-                                                                                     ld, in, out, accumulate, dbar);
-            return;
-        }
-        if (nslots > 1)
-            ++g_launches, k_ggemm<T, G, 8, 8, 5, false, true><<<grid, 256, 0, s>>>(g, targets, cr, nslots, P.ns, ld,
-                                                                                  in, out, accumulate, dbar, 1, nullptr);
+    const int n = P.ns;
+    if (ld == 0) ld = n;
+    if constexpr (sizeof(T) == 4) {
+        const bool big = (int64_t)grid_for(total, 64) * (gemm_ldp(ld) / (32 * gemm_nc(ld))) >= P.num_sms;
+        if (n % 4 == 0)
+            rows_launch_f32<true>(g, targets, cr, most, ncls, big, n, ld, in, out, accumulate, dbar, s);
         else
-            ++g_launches, k_ggemm<T, G, 8, 8, 5, false, false><<<grid, 256, 0, s>>>(g, targets, cr, nslots, P.ns, ld,
-                                                                                   in, out, accumulate, dbar, 1, nullptr);
-        return;
+            rows_launch_f32<false>(g, targets, cr, most, ncls, big, n, ld, in, out, accumulate, dbar, s);
+    } else if ((int64_t)grid_for(total, 64) * grid_for(n, 160) >= 2 * P.num_sms) {
+        const dim3 grid(grid_for(most, 64), ncls, grid_for(n, 160));
+        ++g_launches, k_rows_f64<8, 8, 5><<<grid, 256, 0, s>>>(g, targets, cr, n, in, out, accumulate);
+    } else {
+        const dim3 grid(grid_for(most, 16), ncls, grid_for(n, 32));
+        ++g_launches, k_rows_f64<4, 4, 1><<<grid, 128, 0, s>>>(g, targets, cr, n, in, out, accumulate);
     }
-    const bool splittable = nslots > 1 && nslots <= 8 && total <= kSplitTargets;
-    if (splittable && big_blocks * nslots >= 2 * P.num_sms) {
-        // big tiles, one slot per block (single-slot registers: two blocks per SM)
-        T *part = (T *)P.gemm_part;
-        const int ncb_big = (int)grid_for(ld, 160);
-        dim3 grid(grid_for(most, 64), ncls, ncb_big * nslots);
-        if constexpr (sizeof(T) == 4) {
-            if (P.ns % 4 == 0)
-                ++g_launches, k_ggemm_v4<G, false, true, true><<<grid, kV4Threads, 0, s>>>(
-                                  g, targets, cr, nslots, P.ns, ld, in, out, accumulate, dbar, ncb_big, part);
-            else
-                ++g_launches, k_ggemm_v4<G, false, false, true><<<grid, kV4Threads, 0, s>>>(
-                                  g, targets, cr, nslots, P.ns, ld, in, out, accumulate, dbar, ncb_big, part);
-        } else {
-            ++g_launches, k_ggemm<T, G, 8, 8, 5, true, false><<<grid, 256, 0, s>>>(g, targets, cr, nslots, P.ns, ld,
-                                                                                    in, out, accumulate, dbar,
-                                                                                    ncb_big, part);
-        }
-        ++g_launches, k_ggemm_sum<T, G><<<grid_for(total * ld, 256), 256, 0, s>>>(
-                          g, targets, cr.b[0], total, nslots, P.ns, ld, part, out, accumulate, dbar);
-        return;
-    }
-    const int ncb = (int)grid_for(ld, 32);
-    int64_t small_blocks = 0;
-    for (int c = 0; c < ncls; ++c) small_blocks += grid_for(starts[c + 1] - starts[c], 16);
-    small_blocks *= ncb;
-    if (splittable && small_blocks < 16 * P.num_sms) {
-        T *part = (T *)P.gemm_part;
-        dim3 grid(grid_for(most, 16), ncls, ncb * nslots);
-        ++g_launches, k_ggemm<T, G, 4, 4, 1, true, false><<<grid, 128, 0, s>>>(g, targets, cr, nslots, P.ns, ld, in,
-                                                                                out, accumulate, dbar, ncb, part);
-        ++g_launches, k_ggemm_sum<T, G><<<grid_for(total * ld, 256), 256, 0, s>>>(
-                          g, targets, cr.b[0], total, nslots, P.ns, ld, part, out, accumulate, dbar);
-        return;
-    }
-    dim3 grid(grid_for(most, 16), ncls, ncb);
-    ++g_launches, k_ggemm<T, G, 4, 4, 1, false, true><<<grid, 128, 0, s>>>(g, targets, cr, nslots, P.ns, ld, in,
-                                                                            out, accumulate, dbar, ncb, nullptr);
 }
 
-template <typename T, class G>
-void ggemm(Plan &P, const G &g, const int32_t *targets, int64_t a, int64_t e, int nslots, const T *in, T *out,
-           int accumulate, cudaStream_t s) {
+// The same operator for the rows targets[a .. e).
+template <typename T>
+void rows_one(Plan &P, const T *op, const int32_t *targets, int64_t a, int64_t e, const T *in, T *out,
+              cudaStream_t s) {
     const int64_t st[2] = {a, e};
-    ggemm_classes<T, G>(P, g, targets, st, 1, nslots, in, out, accumulate, s);
+    rows<T>(P, RowMap<T>{nullptr, op, 0, false}, targets, st, 1, in, out, 0, s);
+}
+
+// out[b] (=|+=) sum over the children c of b of Op_{octant(c)} in[c], for the
+// boxes b of level l that have children; prod: scratch rows.
+template <typename T>
+void rows_children(Plan &P, int l, const T *ops, const T *in, T *prod, T *out, int accumulate, cudaStream_t s) {
+    rows<T>(P, RowMap<T>{nullptr, ops, op_block<T>(P.ns, P.ns), true}, P.part_list[3],
+            P.part_start[3].data() + 8 * (l + 1), 8, in, prod, 0, s);
+    const int64_t a = P.part_start[1][1 + l], np = P.part_start[1][2 + l] - a;
+    if (np > 0)
+        ++g_launches, k_child_sum<T><<<grid_for(np * P.ns, 256), 256, 0, s>>>(P.part_list[1] + a, np, P.ns, P.child8,
+                                                                              prod, out, accumulate);
+}
+
+// out[b] += Op_{octant(b)} in[parent(b)] for the boxes b of level l.
+template <typename T>
+void rows_parent(Plan &P, int l, const T *ops, const T *in, T *out, cudaStream_t s, int ld = 0,
+                 double *dbar = nullptr) {
+    rows<T>(P, RowMap<T>{P.parent, ops, op_block<T>(P.ns, ld ? ld : P.ns), true}, P.part_list[3],
+            P.part_start[3].data() + 8 * l, 8, in, out, 1, s, ld, dbar);
 }
 
 // Periodic cell (Sec. 2.4): the images beyond the 26 nearest act on the
@@ -1512,7 +1293,6 @@ template <typename T>
 cudaError_t evaluate_t(Plan &P, void *pot, void *grad, double *energy, cudaStream_t s) {
     using V4 = typename Vec4<T>::type;
     const int ns = P.ns;
-    const size_t nn = (size_t)ns * ns;
     const T *surf = P.f64 ? (const T *)P.surf64 : (const T *)P.surf32;
     T *u = (T *)P.u_chk, *d = (T *)P.d_chk, *tmp = (T *)P.tmp_chk;
     const V4 *pts = (const V4 *)P.pts;
@@ -1529,8 +1309,7 @@ cudaError_t evaluate_t(Plan &P, void *pot, void *grad, double *energy, cudaStrea
     stage_end(P, KIFMM_STAGE_P2M, s);
     stage_begin(P, KIFMM_STAGE_M2M, s);
     for (int l = P.max_level - 1; l >= 0; --l)
-        ggemm<T>(P, GatherChild<T>{P.child8, (const T *)P.m2m_t, ns}, P.part_list[1],
-                 P.part_start[1][1 + l], P.part_start[1][2 + l], 8, u, u, 0, s);
+        rows_children<T>(P, l, (const T *)P.m2m_t, u, tmp, u, 0, s);
     stage_end(P, KIFMM_STAGE_M2M, s);
     KIFMM_CUDA_TRY(cudaGetLastError());
     // interactions
@@ -1572,19 +1351,17 @@ cudaError_t evaluate_t(Plan &P, void *pot, void *grad, double *energy, cudaStrea
     // downward pass: per level, per octant class of the child
     stage_begin(P, KIFMM_STAGE_L2L, s);
     for (int l = 1; l <= P.max_level; ++l)
-        ggemm_classes<T>(P, GatherParent<T>{P.parent, (const T *)P.l2l_t, ns, P.op_ld}, P.part_list[3],
-                         P.part_start[3].data() + 8 * l, 8, 1, d, d, 1, s, P.op_ld, split_mean ? P.dbar : nullptr);
+        rows_parent<T>(P, l, (const T *)P.l2l_t, d, d, s, P.op_ld, split_mean ? P.dbar : nullptr);
     stage_end(P, KIFMM_STAGE_L2L, s);
     KIFMM_CUDA_TRY(cudaGetLastError());
     // leaves: equivalent densities (two-step pseudo-inverse), then L2P + M2P + P2P
     stage_begin(P, KIFMM_STAGE_LEAF, s);
     if (P.n_w > 0) {
-        ggemm<T>(P, GatherSelf<T>{(const T *)P.up_w_t}, P.part_list[2], 0, P.part_start[2][1], 1, u, tmp, 0, s);
-        ggemm<T>(P, GatherSelf<T>{(const T *)P.up_v_t}, P.part_list[2], 0, P.part_start[2][1], 1, tmp,
-                 (T *)P.up_dens, 0, s);
+        rows_one<T>(P, (const T *)P.up_w_t, P.part_list[2], 0, P.part_start[2][1], u, tmp, s);
+        rows_one<T>(P, (const T *)P.up_v_t, P.part_list[2], 0, P.part_start[2][1], tmp, (T *)P.up_dens, s);
     }
-    ggemm<T>(P, GatherSelf<T>{(const T *)P.dn_w_t}, P.leaves, 0, P.n_leaves, 1, d, tmp, 0, s);
-    ggemm<T>(P, GatherSelf<T>{(const T *)P.dn_v_t}, P.leaves, 0, P.n_leaves, 1, tmp, (T *)P.dn_dens, 0, s);
+    rows_one<T>(P, (const T *)P.dn_w_t, P.leaves, 0, P.n_leaves, d, tmp, s);
+    rows_one<T>(P, (const T *)P.dn_v_t, P.leaves, 0, P.n_leaves, tmp, (T *)P.dn_dens, s);
     stage_end(P, KIFMM_STAGE_LEAF, s);
     stage_begin(P, KIFMM_STAGE_P2P, s);
     LeafCtx C{P.lvl, P.cx, P.cy, P.cz, P.first, P.cnt, P.u_ptr, P.w_ptr, P.u_idx, P.w_idx, ns,
@@ -2031,8 +1808,7 @@ cudaError_t evaluate_stokes_t(Plan &P, void *vel, cudaStream_t s) {
     stage_end(P, KIFMM_STAGE_P2M, s);
     stage_begin(P, KIFMM_STAGE_M2M, s);
     for (int l = P.max_level - 1; l >= 0; --l)
-        ggemm<T>(P, GatherChild<T>{P.child8, (const T *)P.m2m_t, ns}, P.part_list[1],
-                 P.part_start[1][1 + l], P.part_start[1][2 + l], 8, u, u, 0, s);
+        rows_children<T>(P, l, (const T *)P.m2m_t, u, tmp, u, 0, s);
     stage_end(P, KIFMM_STAGE_M2M, s);
     stage_begin(P, KIFMM_STAGE_M2L, s);
     KIFMM_CUDA_TRY(cudaMemsetAsync(d, 0, sizeof(T) * (size_t)P.nb * ns, s));
@@ -2047,18 +1823,16 @@ cudaError_t evaluate_stokes_t(Plan &P, void *vel, cudaStream_t s) {
     }
     stage_begin(P, KIFMM_STAGE_L2L, s);
     for (int l = 1; l <= P.max_level; ++l)
-        ggemm_classes<T>(P, GatherParent<T>{P.parent, (const T *)P.l2l_t, ns, P.op_ld}, P.part_list[3],
-                         P.part_start[3].data() + 8 * l, 8, 1, d, d, 1, s, P.op_ld, nullptr);
+        rows_parent<T>(P, l, (const T *)P.l2l_t, d, d, s);
     stage_end(P, KIFMM_STAGE_L2L, s);
     KIFMM_CUDA_TRY(cudaGetLastError());
     stage_begin(P, KIFMM_STAGE_LEAF, s);
     if (P.n_w > 0) {
-        ggemm<T>(P, GatherSelf<T>{(const T *)P.up_w_t}, P.part_list[2], 0, P.part_start[2][1], 1, u, tmp, 0, s);
-        ggemm<T>(P, GatherSelf<T>{(const T *)P.up_v_t}, P.part_list[2], 0, P.part_start[2][1], 1, tmp,
-                 (T *)P.up_dens, 0, s);
+        rows_one<T>(P, (const T *)P.up_w_t, P.part_list[2], 0, P.part_start[2][1], u, tmp, s);
+        rows_one<T>(P, (const T *)P.up_v_t, P.part_list[2], 0, P.part_start[2][1], tmp, (T *)P.up_dens, s);
     }
-    ggemm<T>(P, GatherSelf<T>{(const T *)P.dn_w_t}, P.leaves, 0, P.n_leaves, 1, d, tmp, 0, s);
-    ggemm<T>(P, GatherSelf<T>{(const T *)P.dn_v_t}, P.leaves, 0, P.n_leaves, 1, tmp, (T *)P.dn_dens, 0, s);
+    rows_one<T>(P, (const T *)P.dn_w_t, P.leaves, 0, P.n_leaves, d, tmp, s);
+    rows_one<T>(P, (const T *)P.dn_v_t, P.leaves, 0, P.n_leaves, tmp, (T *)P.dn_dens, s);
     stage_end(P, KIFMM_STAGE_LEAF, s);
     stage_begin(P, KIFMM_STAGE_P2P, s);
     LeafCtx C{P.lvl, P.cx, P.cy, P.cz, P.first, P.cnt, P.u_ptr, P.w_ptr, P.u_idx, P.w_idx, ns, nullptr,
@@ -2236,7 +2010,7 @@ cudaError_t backward_t(Plan &P, const void *w_user, const void *g_user, const do
                        void *dq, void *dx, cudaStream_t s) {
     using V4 = typename Vec4<T>::type;
     const int ns = P.ns;
-    const size_t nn = (size_t)ns * ns;
+    const int64_t blk = op_block<T>(ns, ns);
     const T *surf = P.f64 ? (const T *)P.surf64 : (const T *)P.surf32;
     T *ub = (T *)P.u_chk, *db = (T *)P.d_chk, *tmp = (T *)P.tmp_chk;
     // scratch of their own: the forward's equivalent densities stay intact
@@ -2273,27 +2047,25 @@ cudaError_t backward_t(Plan &P, const void *w_user, const void *g_user, const do
     KIFMM_CUDA_TRY(cudaMemsetAsync(ub, 0, sizeof(T) * (size_t)P.nb * ns, s));
     ++g_launches, k_p2m<T><<<(unsigned)P.n_leaves, p2m_threads(P), p2m_smem<T>(P), s>>>(P.leaves, P.lvl, P.first, P.cnt, pts, surf,
                                                                         ns, e1, ws, 1, gs);
-    ggemm<T>(P, GatherSelf<T>{adjp + 3 * nn}, P.leaves, 0, P.n_leaves, 1, e1, tmp, 0, s);
-    ggemm<T>(P, GatherSelf<T>{adjp + 2 * nn}, P.leaves, 0, P.n_leaves, 1, tmp, db, 0, s);
+    rows_one<T>(P, adjp + 3 * blk, P.leaves, 0, P.n_leaves, e1, tmp, s);
+    rows_one<T>(P, adjp + 2 * blk, P.leaves, 0, P.n_leaves, tmp, db, s);
     // M2P^T: W-list sources a receive h_a * sum w / |UE_a - x| (+ dipoles) from the leaves of X(a)
     if (P.n_x > 0) {
         KIFMM_CUDA_TRY(cudaMemsetAsync(e2, 0, sizeof(T) * (size_t)P.nb * ns, s));
         ++g_launches, k_p2l<T><<<(unsigned)P.nb, p2l_threads<T>(P), 0, s>>>(
                           p2m_threads(P), P.nx, P.xdense, P.lvl, P.cx, P.cy, P.cz, P.first, P.cnt, pts, surf, ns, e2,
                           ws, 1, nullptr, gs);
-        ggemm<T>(P, GatherSelf<T>{adjp + 1 * nn}, P.part_list[2], 0, P.part_start[2][1], 1, e2, tmp, 0, s);
-        ggemm<T>(P, GatherSelf<T>{adjp}, P.part_list[2], 0, P.part_start[2][1], 1, tmp, ub, 0, s);
+        rows_one<T>(P, adjp + 1 * blk, P.part_list[2], 0, P.part_start[2][1], e2, tmp, s);
+        rows_one<T>(P, adjp, P.part_list[2], 0, P.part_start[2][1], tmp, ub, s);
     }
     // L2L^T, bottom-up
     for (int l = P.max_level - 1; l >= 0; --l)
-        ggemm<T>(P, GatherChild<T>{P.child8, (const T *)P.adj_l2l, ns}, P.part_list[1], P.part_start[1][1 + l],
-                 P.part_start[1][2 + l], 8, db, db, 1, s);
+        rows_children<T>(P, l, (const T *)P.adj_l2l, db, tmp, db, 1, s);
     // M2L^T (V lists are symmetric; operator at the negated offset, transposed)
     KIFMM_CUDA_TRY(m2l_exact(P, 1, db, ub, 1, nullptr, s));
     // M2M^T, top-down
     for (int l = 1; l <= P.max_level; ++l)
-        ggemm_classes<T>(P, GatherParent<T>{P.parent, (const T *)P.adj_m2m, ns, ns}, P.part_list[3],
-                         P.part_start[3].data() + 8 * l, 8, 1, ub, ub, 1, s);
+        rows_parent<T>(P, l, (const T *)P.adj_m2m, ub, ub, s);
     // P2M^T (own UC surface, u-bar), P2L^T (W boxes' DC surfaces, d-bar), P2P^T (weights w)
     const LeafW<T> W{ub, 0, db, 0, ws};
     leaf_launch<T>(P, C, pts, surf, W, res, s);
@@ -2310,6 +2082,13 @@ cudaError_t backward_t(Plan &P, const void *w_user, const void *g_user, const do
 }
 
 }  // namespace
+
+cudaError_t rows_setup() {
+    const auto dyn = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const int most = (int)rows_small_smem(gemm_nkp(3 * (6 * 7 * 7 + 2)));  // the longest rows: Stokeslet, p = 8
+    KIFMM_CUDA_TRY(cudaFuncSetAttribute(k_rows_small<true>, dyn, most));
+    return cudaFuncSetAttribute(k_rows_small<false>, dyn, most);
+}
 
 cudaError_t run_backward(Plan &P, const void *w, const void *g, const double *dLdU, const void *grad, void *dq,
                          void *dx, cudaStream_t s) {

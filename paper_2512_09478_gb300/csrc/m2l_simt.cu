@@ -14,9 +14,9 @@
 // targets of one octant class by 160 outputs, a thread RT targets by five
 // pairs of outputs, on packed f32x2 FMAs (each half rounds as a scalar FMA;
 // packed they reach 111 lanes per clock and SM, three-operand scalar ones 82):
-// at RT = 8, 40 of them per input for nine shared-memory reads.  The inputs
-// are staged in pairs (u, u), so that no register moves are spent on forming
-// them; the operators, padded to whole blocks of 16 inputs x 160 outputs at
+// at RT = 8, 40 of them per input for seven shared-memory reads.  The inputs
+// are staged once and paired (u, u) in registers (the loop alone: 95 lanes per
+// clock and SM, 86 with staged pairs); the operators, padded to whole blocks of 16 inputs x 160 outputs at
 // plan time, come by 16-byte asynchronous copies without bounds tests.  One
 // barrier per 16 inputs (two buffers).  Stokeslet, 60k points, p = 6 (4672
 // targets, n = 456): 27.1 ms with 16 x 32 tiles of scalar FMAs, 11.7 here,
@@ -36,7 +36,7 @@ constexpr int kSThreads = 128;  // 16 threads across the outputs, 8 across the t
 
 template <int RT>
 struct SimtSmem {
-    float2 u[2][kSK][8 * RT];  // (u, u)
+    float u[2][kSK][8 * RT];
     float m[2][kSK][kSCols];
 };
 
@@ -129,10 +129,10 @@ __global__ void __launch_bounds__(kSThreads, RT == 8 ? 2 : (RT == 4 ? 3 : 4))
             for (int r = 0; r < kQ; ++r) {
                 const int e = tid + kSThreads * r, t = e % TT, k = 4 * (e / TT);
                 if (!kAll && e >= TT * (kSK / 4)) continue;
-                S.u[b][k][t] = make_float2(ru[r].x, ru[r].x);
-                S.u[b][k + 1][t] = make_float2(ru[r].y, ru[r].y);
-                S.u[b][k + 2][t] = make_float2(ru[r].z, ru[r].z);
-                S.u[b][k + 3][t] = make_float2(ru[r].w, ru[r].w);
+                S.u[b][k][t] = ru[r].x;
+                S.u[b][k + 1][t] = ru[r].y;
+                S.u[b][k + 2][t] = ru[r].z;
+                S.u[b][k + 3][t] = ru[r].w;
             }
             cp_wait_all();
         };
@@ -142,23 +142,28 @@ __global__ void __launch_bounds__(kSThreads, RT == 8 ? 2 : (RT == 4 ? 3 : 4))
         for (int kc = 0; kc < nk; ++kc) {
             const int b = kc & 1;
             if (kc + 1 < nk) load(kc + 1, b ^ 1);  // last read before the previous barrier
-            const float2 *su = &S.u[b][0][RT * ty];
+            const float *su = &S.u[b][0][RT * ty];
             const float *sm = &S.m[b][0][2 * tx];
 #pragma unroll 4
             for (int k = 0; k < kSK; ++k) {
-                float2 uv[RT], mv[5];
+                float uv[RT];
+                float2 mv[5];
 #pragma unroll
-                for (int a = 0; a < RT; a += 2) {
-                    const float4 w = *reinterpret_cast<const float4 *>(su + k * TT + a);
-                    uv[a] = make_float2(w.x, w.y);
-                    uv[a + 1] = make_float2(w.z, w.w);
+                for (int a = 0; a < RT; a += 4) {
+                    if constexpr (RT >= 4) {
+                        const float4 w = *reinterpret_cast<const float4 *>(su + k * TT + a);
+                        uv[a] = w.x, uv[a + 1] = w.y, uv[a + 2] = w.z, uv[a + 3] = w.w;
+                    } else {
+                        const float2 w = *reinterpret_cast<const float2 *>(su + k * TT);
+                        uv[0] = w.x, uv[1] = w.y;
+                    }
                 }
 #pragma unroll
                 for (int c = 0; c < 5; ++c) mv[c] = *reinterpret_cast<const float2 *>(sm + k * kSCols + 32 * c);
 #pragma unroll
                 for (int a = 0; a < RT; ++a)
 #pragma unroll
-                    for (int c = 0; c < 5; ++c) acc[a][c] = __ffma2_rn(uv[a], mv[c], acc[a][c]);
+                    for (int c = 0; c < 5; ++c) acc[a][c] = __ffma2_rn(make_float2(uv[a], uv[a]), mv[c], acc[a][c]);
             }
             if (kc + 1 < nk) {
                 store(b ^ 1);
