@@ -176,15 +176,16 @@ __global__ void k_p2m_f32(const int32_t *__restrict__ leaves, int64_t n_leaves, 
 }
 
 // P2L: d(b)_j += (1/h_b) sum_{a in X(b)} sum_i q_i / |1.05 S_j - (x_i - c_b)/h_b|
-// One block per box, few of which have an X list, but those up to 26 leaves of
-// it: a block's length is the launch's.  A thread per check point (tpg of them:
+// One block per box with an X list (the X lists are the transposed W lists, so
+// these are the boxes of part_list[2]), up to 26 leaves of it: a block's length
+// is the launch's.  A thread per check point (tpg of them:
 // n_s rounded up to a warp; with 128 threads, two rounds over the sources, the
 // second for the last 24 points of n_s = 152).  FP64, bound by the FP64 unit,
 // also cuts the sources into blockDim / tpg interleaved groups, whose sums are
 // added in group order.  60k Plummer, FP64: 1.18 -> 0.44 ms.
 template <typename T>
 __global__ void __launch_bounds__(1024, 1)
-    k_p2l(int tpg, const int32_t *__restrict__ nx, const int32_t *__restrict__ xdense, const int32_t *__restrict__ lvl,
+    k_p2l(int tpg, const int32_t *__restrict__ boxes, const int32_t *__restrict__ nx, const int32_t *__restrict__ xdense, const int32_t *__restrict__ lvl,
           const int32_t *__restrict__ cx, const int32_t *__restrict__ cy, const int32_t *__restrict__ cz,
           const int32_t *__restrict__ first, const int32_t *__restrict__ cnt,
           const typename Vec4<T>::type *__restrict__ pts, const T *__restrict__ surf, int ns, T *__restrict__ d,
@@ -197,8 +198,7 @@ __global__ void __launch_bounds__(1024, 1)
     __shared__ T gx[kLeafThreads], gy[kLeafThreads], gz[kLeafThreads];
     __shared__ T cv[kMaxNs];
     __shared__ double red[32];
-    const int b = blockIdx.x;
-    if (nx[b] == 0) return;
+    const int b = boxes[blockIdx.x];
     const int lb = lvl[b];
     const T hb = box_half<T>(lb), hinv = T(1) / hb;
     const T cbx = box_center<T>(cx[b], lb), cby = box_center<T>(cy[b], lb), cbz = box_center<T>(cz[b], lb);
@@ -1331,8 +1331,8 @@ cudaError_t evaluate_t(Plan &P, void *pot, void *grad, double *energy, cudaStrea
     stage_end(P, KIFMM_STAGE_M2L, s);
     if (P.n_x > 0) {
         stage_begin(P, KIFMM_STAGE_P2L, s);
-        ++g_launches, k_p2l<T><<<(unsigned)P.nb, p2l_threads<T>(P), 0, s>>>(
-                          p2m_threads(P), P.nx, P.xdense, P.lvl, P.cx, P.cy, P.cz, P.first, P.cnt, pts, surf, ns, d,
+        ++g_launches, k_p2l<T><<<(unsigned)P.part_start[2][1], p2l_threads<T>(P), 0, s>>>(
+                          p2m_threads(P), P.part_list[2], P.nx, P.xdense, P.lvl, P.cx, P.cy, P.cz, P.first, P.cnt, pts, surf, ns, d,
                           nullptr, 0, split_mean ? P.dbar : nullptr, nullptr, P.periodic ? P.x_sh : nullptr);
         stage_end(P, KIFMM_STAGE_P2L, s);
     }
@@ -1627,7 +1627,7 @@ __global__ void k_p2m_stokes(const int32_t *__restrict__ leaves, const int32_t *
 
 // P2L: d(b) += the forces of the leaves of X(b) on b's downward check surface.
 template <typename T>
-__global__ void k_p2l_stokes(const int32_t *__restrict__ nx, const int32_t *__restrict__ xdense,
+__global__ void k_p2l_stokes(const int32_t *__restrict__ boxes, const int32_t *__restrict__ nx, const int32_t *__restrict__ xdense,
                              const int32_t *__restrict__ lvl, const int32_t *__restrict__ cx,
                              const int32_t *__restrict__ cy, const int32_t *__restrict__ cz,
                              const int32_t *__restrict__ first, const int32_t *__restrict__ cnt,
@@ -1635,8 +1635,7 @@ __global__ void k_p2l_stokes(const int32_t *__restrict__ nx, const int32_t *__re
                              const T *__restrict__ surf, int npt, T *__restrict__ d) {
     __shared__ T sx[kLeafThreads], sy[kLeafThreads], sz[kLeafThreads], sfx[kLeafThreads], sfy[kLeafThreads],
         sfz[kLeafThreads];
-    const int b = blockIdx.x;
-    if (nx[b] == 0) return;
+    const int b = boxes[blockIdx.x];
     const int lb = lvl[b];
     const T hb = box_half<T>(lb), hinv = T(1) / hb;
     const T al = (T)kAlphaInner;
@@ -1817,7 +1816,7 @@ cudaError_t evaluate_stokes_t(Plan &P, void *vel, cudaStream_t s) {
     stage_end(P, KIFMM_STAGE_M2L, s);
     if (P.n_x > 0) {
         stage_begin(P, KIFMM_STAGE_P2L, s);
-        ++g_launches, k_p2l_stokes<T><<<(unsigned)P.nb, thr, 0, s>>>(P.nx, P.xdense, P.lvl, P.cx, P.cy, P.cz,
+        ++g_launches, k_p2l_stokes<T><<<(unsigned)P.part_start[2][1], thr, 0, s>>>(P.part_list[2], P.nx, P.xdense, P.lvl, P.cx, P.cy, P.cz,
                                                                        P.first, P.cnt, pts, frc, surf, npt, d);
         stage_end(P, KIFMM_STAGE_P2L, s);
     }
@@ -2052,8 +2051,8 @@ cudaError_t backward_t(Plan &P, const void *w_user, const void *g_user, const do
     // M2P^T: W-list sources a receive h_a * sum w / |UE_a - x| (+ dipoles) from the leaves of X(a)
     if (P.n_x > 0) {
         KIFMM_CUDA_TRY(cudaMemsetAsync(e2, 0, sizeof(T) * (size_t)P.nb * ns, s));
-        ++g_launches, k_p2l<T><<<(unsigned)P.nb, p2l_threads<T>(P), 0, s>>>(
-                          p2m_threads(P), P.nx, P.xdense, P.lvl, P.cx, P.cy, P.cz, P.first, P.cnt, pts, surf, ns, e2,
+        ++g_launches, k_p2l<T><<<(unsigned)P.part_start[2][1], p2l_threads<T>(P), 0, s>>>(
+                          p2m_threads(P), P.part_list[2], P.nx, P.xdense, P.lvl, P.cx, P.cy, P.cz, P.first, P.cnt, pts, surf, ns, e2,
                           ws, 1, nullptr, gs);
         rows_one<T>(P, adjp + 1 * blk, P.part_list[2], 0, P.part_start[2][1], e2, tmp, s);
         rows_one<T>(P, adjp, P.part_list[2], 0, P.part_start[2][1], tmp, ub, s);

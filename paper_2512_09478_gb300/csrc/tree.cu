@@ -1062,7 +1062,13 @@ __device__ __forceinline__ void dev_x(int64_t b, int lane, int level, int thr, i
 // direct-sum leaf.  When b itself is a direct-sum leaf, its X list (coarser
 // leaves adjacent to the parent, not to b) goes to U as well.  Pass 0 counts,
 // pass 1 fills.
-__global__ void k_uw(int64_t nb, int pass, int thr, const int32_t *__restrict__ parent,
+//
+// One warp per box: a lane per coarse leaf, then a lane per colleague, each
+// descending its own (the entries keep the order of a single thread's scan: a
+// lane's places come from a prefix sum of the lanes' counts, for which pass 1
+// descends once more).  A clustered tree's time is the longest descent of one
+// leaf: a thread per box took all 26 in a row (60k Plummer: 130 us a pass).
+__global__ void __launch_bounds__(128) k_uw(int64_t nb, int pass, int thr, const int32_t *__restrict__ parent,
                      const int32_t *__restrict__ cnt, const int32_t *__restrict__ child_first,
                      const int32_t *__restrict__ nchild, const int32_t *__restrict__ lvl,
                      const int32_t *__restrict__ cx, const int32_t *__restrict__ cy,
@@ -1071,69 +1077,92 @@ __global__ void k_uw(int64_t nb, int pass, int thr, const int32_t *__restrict__ 
                      uint32_t *u_cnt, uint32_t *w_cnt, const uint32_t *__restrict__ u_ptr,
                      const uint32_t *__restrict__ w_ptr, int32_t *u_idx, int32_t *w_idx, int64_t u_cap,
                      int64_t w_cap, int *status, ListShifts sh) {
-    int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nb) return;
+    const int64_t b = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (b >= nb) return;  // uniform for the warp
     if (nchild[b] != 0) {
-        if (pass == 0) u_cnt[b] = w_cnt[b] = 0;
+        if (pass == 0 && lane == 0) u_cnt[b] = w_cnt[b] = 0;
         return;
     }
     const int lb = lvl[b], bx = cx[b], by = cy[b], bz = cz[b];
-    uint32_t nu = 0, nw = 0;
     const uint32_t u0 = pass ? u_ptr[b] : 0, w0 = pass ? w_ptr[b] : 0;
     // pass 1 writes only inside the storage; the host sees a list that
     // outgrew it from the totals and builds the lists again
-    auto put_u = [&](int32_t a, int sa) {
-        if (pass && (int64_t)u0 + nu < u_cap) {
-            u_idx[u0 + nu] = a;
-            if (sh.u) sh.u[u0 + nu] = (int8_t)sa;
+    auto put_u = [&](uint32_t pos, int32_t a, int sa) {
+        if (pass && (int64_t)u0 + pos < u_cap) {
+            u_idx[u0 + pos] = a;
+            if (sh.u) sh.u[u0 + pos] = (int8_t)sa;
         }
-        ++nu;
     };
-    auto put_w = [&](int32_t a, int sa) {
-        if (pass && (int64_t)w0 + nw < w_cap) {
-            w_idx[w0 + nw] = a;
-            if (sh.w) sh.w[w0 + nw] = (int8_t)sa;
+    auto put_w = [&](uint32_t pos, int32_t a, int sa) {
+        if (pass && (int64_t)w0 + pos < w_cap) {
+            w_idx[w0 + pos] = a;
+            if (sh.w) sh.w[w0 + pos] = (int8_t)sa;
         }
-        ++nw;
     };
-    put_u((int32_t)b, 13);
-    for (int k = 0; k < ncoarse[b]; ++k) put_u(coarse[b * kMaxCoarse + k], shift_of(sh.coarse, b * kMaxCoarse + k));
+    const int nc = ncoarse[b];  // <= kMaxCoarse < 32
+    if (lane == 0) put_u(0, (int32_t)b, 13);
+    if (lane < nc) put_u(1 + lane, coarse[b * kMaxCoarse + lane], shift_of(sh.coarse, b * kMaxCoarse + lane));
+    uint32_t nu = 1 + (uint32_t)nc, nw = 0;
     if (lb > 0 && direct_box(nchild, cnt, thr, (int32_t)b)) {
         const int32_t P = parent[b];
-        for (int k = 0; k < ncoarse[P]; ++k) {
-            const int32_t a = coarse[(int64_t)P * kMaxCoarse + k];
-            const int sa = shift_of(sh.coarse, (int64_t)P * kMaxCoarse + k);
-            if (adjacent_img(lvl[a], cx[a], cy[a], cz[a], sa, lb, bx, by, bz)) continue;
-            put_u(a, sa);
+        int32_t a = -1;
+        int sa = 13;
+        bool keep = false;
+        if (lane < ncoarse[P]) {
+            a = coarse[(int64_t)P * kMaxCoarse + lane];
+            sa = shift_of(sh.coarse, (int64_t)P * kMaxCoarse + lane);
+            keep = !adjacent_img(lvl[a], cx[a], cy[a], cz[a], sa, lb, bx, by, bz);
         }
+        const unsigned m = __ballot_sync(0xffffffffu, keep);
+        if (keep) put_u(nu + __popc(m & ((1u << lane) - 1u)), a, sa);
+        nu += __popc(m);
     }
-    int32_t stack[8 * (kMaxLevel + 1)];
-    for (int k = 0; k < kColl; ++k) {
-        const int32_t c = coll[b * kColl + k];
-        if (k == 13 || c < 0 || nchild[c] == 0) continue;
-        const int sc = shift_of(sh.coll, b * kColl + k);  // every descendant is taken in this image
+    // lane k descends colleague k; every descendant is taken in its image
+    const int32_t c = (lane < kColl && lane != 13) ? coll[b * kColl + lane] : -1;
+    const bool mine = c >= 0 && nchild[c] != 0;
+    const int sc = mine ? shift_of(sh.coll, b * kColl + lane) : 13;
+    auto descend = [&](auto &&to_u, auto &&to_w) {
+        int32_t stack[8 * (kMaxLevel + 1)];
         int sp = 0;
         for (int32_t ch = child_first[c]; ch < child_first[c] + nchild[c]; ++ch) stack[sp++] = ch;
         while (sp > 0) {
             const int32_t a = stack[--sp];
+            const int na = nchild[a];
             if (adjacent_img(lvl[a], cx[a], cy[a], cz[a], sc, lb, bx, by, bz)) {
-                if (nchild[a] == 0) {
-                    put_u(a, sc);
+                if (na == 0) {
+                    to_u(a);
                 } else {
-                    if (sp + nchild[a] > 8 * (kMaxLevel + 1)) {
+                    if (sp + na > 8 * (kMaxLevel + 1)) {
                         set_status(status, KIFMM_ERR_CAPACITY);
                         return;
                     }
-                    for (int32_t ch = child_first[a]; ch < child_first[a] + nchild[a]; ++ch) stack[sp++] = ch;
+                    for (int32_t ch = child_first[a]; ch < child_first[a] + na; ++ch) stack[sp++] = ch;
                 }
             } else if (direct_box(nchild, cnt, thr, a)) {
-                put_u(a, sc);
+                to_u(a);
             } else {
-                put_w(a, sc);
+                to_w(a);
             }
         }
+    };
+    if (__any_sync(0xffffffffu, mine)) {
+        uint32_t cu = 0, cw = 0;
+        if (mine) descend([&](int32_t) { ++cu; }, [&](int32_t) { ++cw; });
+        uint32_t iu = cu, iw = cw;  // inclusive sums over the lanes
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t yu = __shfl_up_sync(0xffffffffu, iu, o), yw = __shfl_up_sync(0xffffffffu, iw, o);
+            if (lane >= o) iu += yu, iw += yw;
+        }
+        if (pass && mine) {
+            uint32_t pu = nu + iu - cu, pw = nw + iw - cw;
+            descend([&](int32_t a) { put_u(pu++, a, sc); }, [&](int32_t a) { put_w(pw++, a, sc); });
+        }
+        nu += __shfl_sync(0xffffffffu, iu, 31);
+        nw += __shfl_sync(0xffffffffu, iw, 31);
     }
-    if (pass == 0) {
+    if (pass == 0 && lane == 0) {
         u_cnt[b] = nu;
         w_cnt[b] = nw;
     }
@@ -1741,7 +1770,7 @@ cudaError_t build_lists(Plan &P, cudaStream_t s) {
                                                       list_shifts(P));
         KIFMM_CUDA_TRY(cudaGetLastError());
     }
-    const unsigned g = grid_for(nb, 128);
+    const unsigned g = grid_for(nb, 4);  // a warp per box, 4 per block
     ++g_launches, k_uw<<<g, 128, 0, s>>>(nb, 0, P.direct_thr, P.parent, P.cnt, P.child_first, P.nchild, P.lvl,
                                          P.cx, P.cy, P.cz, P.coll, P.coarse, P.ncoarse, P.u_cnt, P.w_cnt, nullptr,
                                          nullptr, nullptr, nullptr, 0, 0, P.status, list_shifts(P));
