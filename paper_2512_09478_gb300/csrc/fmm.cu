@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(1024, 1)
     }
     __syncthreads();
     double tot = 0.0;
-    for (int w = 0; w < kLeafThreads / 32; ++w) tot += red[w];
+    for (int w = 0; w < min((int)blockDim.x, kLeafThreads) / 32; ++w) tot += red[w];  // (p <= 4: two warps)
     const double mean = tot / ns;
     for (int k = threadIdx.x; k < ns; k += blockDim.x) d[(size_t)b * ns + k] += (T)((double)cv[k] - mean);
     if (threadIdx.x == 0) dbar[b] += mean;

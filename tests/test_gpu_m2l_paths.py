@@ -98,3 +98,23 @@ def test_one_system_alone_equals_its_copies(precision, kernel, copies):
         assert torch.equal(outs[1][0][n * i:n * (i + 1)], outs[0][0])
         if outs[0][1] is not None:
             assert torch.equal(outs[1][1][n * i:n * (i + 1)], outs[0][1])
+
+
+@pytest.mark.parametrize("precision,p", [("fp64", 3), ("fp64", 6), ("fp32", 3), ("fp32", 4), ("mixed_fp16", 4),
+                                         ("mixed_fp16", 5)])
+def test_x_lists_at_every_block_width(precision, p):
+    """P2L's block is n_s rounded up to a warp (32 to 160 threads here): a
+    clustered cloud with W/X lists kept (direct_max = -1) against the direct
+    sum, within the method's own error (10% and the FP32 budget)."""
+    x = G.plummer(3000, 46)[0]
+    q = np.random.default_rng(46).normal(size=len(x))
+    x, q = x.astype(np.float32).astype(np.float64), q.astype(np.float32).astype(np.float64)
+    pd, gd = O.direct(x, q)
+    po, go, _ = O.kifmm(x, q, p=p, leaf_cap=16, direct_max=-1)
+    plan = _plan(len(x), precision, p, 16, direct_max=-1)
+    plan.set_sources(_dev(x, plan.dtype), _dev(q, plan.dtype))
+    assert plan.tree_info()["n_x"] > 0
+    pot, grad, _ = plan.evaluate()
+    assert plan.device_status() == 0
+    assert O.rel_l2(pot.double().cpu().numpy(), pd) <= 1.1 * O.rel_l2(po, pd) + 5e-6
+    assert O.rel_l2(grad.double().cpu().numpy(), gd) <= 1.1 * O.rel_l2(go, gd) + 5e-6
