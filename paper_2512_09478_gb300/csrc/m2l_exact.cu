@@ -36,7 +36,7 @@
 // Measured, M2L alone: FP64, 60k Plummer, p = 6: 30.7 -> 2.4 ms; FP32, 200k
 // packing, p = 6: 3.30 -> 0.28 ms (the gathered SIMT product before).
 //
-// Pipeline and bounded waits as in m2l_tc.cu: four producer warps (cp.async
+// Pipeline and bounded waits as in m2l_tc.cu: producer warps (cp.async
 // of the gathered rows, one bulk copy of the operator block per stage), one
 // MMA warp, eight drain warps; one CTA per SM.
 #include <cuda_bf16.h>
@@ -56,9 +56,7 @@ namespace {
 
 constexpr int kKB = 32;             // 16-bit elements per stage row (64 bytes)
 constexpr int kRowB = 64;
-constexpr int kProd = 4;            // producer warps
 constexpr int kDrain = 8;           // drain warps
-constexpr int kExThreads = 32 * (kProd + 1 + kDrain);
 constexpr long long kExDrainPolls = 1LL << 18;  // bound of the clean-up wait on the last bulk copy
 
 template <typename T>
@@ -66,6 +64,7 @@ struct Slicing;
 template <>
 struct Slicing<float> {
     static constexpr int kSlices = 3, kGroups = 2, kCols = 160, kChunkBlocks = 8;  // 8 x 32 x 2^16 = 2^24
+    static constexpr int kProd = 4;                                                // producer warps
     static constexpr uint32_t kFmt = 0;                                            // FP16
     __host__ __device__ static constexpr bool used(int i, int j) { return i + j <= 2; }
     __host__ __device__ static constexpr int group(int i, int j) { return i + j == 0 ? 0 : 1; }
@@ -73,10 +72,16 @@ struct Slicing<float> {
 template <>
 struct Slicing<double> {
     static constexpr int kSlices = 8, kGroups = 7, kCols = 64, kChunkBlocks = 5;  // K <= 160 per accumulation
+    static constexpr int kProd = 2;  // producer warps: with 12 or fewer warps the drain's 160 registers fit
     static constexpr uint32_t kFmt = 1;                                           // BF16
     __host__ __device__ static constexpr bool used(int i, int j) { return i + j <= 7; }
     __host__ __device__ static constexpr int group(int i, int j) { return i + j < 6 ? i + j : 6; }
 };
+
+template <typename T>
+constexpr int ex_threads() {
+    return 32 * (Slicing<T>::kProd + 1 + kDrain);
+}
 
 // Scale exponent: the least e with m <= 2^e (m > 0).
 __device__ __forceinline__ int ceil_exp(float m) {
@@ -214,13 +219,19 @@ struct ExArgs {
     int *status;
 };
 
+// An accumulator value as an integer of units 2^-E.
+template <int E>
+__device__ __forceinline__ int unit_int(uint32_t bits) {
+    return __float2int_rn(__uint_as_float(bits) * __int_as_float((127 + E) << 23));
+}
+
 // Byte offset of 16-byte chunk c of row r inside a 64-byte-swizzled tile.
 __device__ __forceinline__ uint32_t swz(int r, int c) { return (uint32_t)(r * kRowB + ((c ^ ((r >> 1) & 3)) << 4)); }
 
 template <typename T>
-__global__ void __launch_bounds__(kExThreads, 1) k_m2l_exact(ExArgs<T> a) {
+__global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
     using SL = Slicing<T>;
-    constexpr int NS = SL::kSlices, NG = SL::kGroups;
+    constexpr int NS = SL::kSlices, NG = SL::kGroups, kProd = SL::kProd;
     constexpr uint32_t kTileB = kTcRows * kRowB;  // one slice of the gathered rows
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -444,28 +455,42 @@ __global__ void __launch_bounds__(kExThreads, 1) k_m2l_exact(ExArgs<T> a) {
                     if (col >= nt) continue;  // uniform
 #pragma unroll
                     for (int half = 0; half < 2; ++half) {
-                        uint32_t v[8 * NG];
+                        const uint32_t at = base + (uint32_t)(col + 8 * half);
+                        if constexpr (sizeof(T) == 4) {
+                            uint32_t v[16];
 #pragma unroll
-                        for (int e = 0; e < NG; ++e)
-                            tmem_ld8_nowait(base + (uint32_t)(e * a.nt + col + 8 * half), v + 8 * e);
-                        tmem_wait_ld(v);
+                            for (int e = 0; e < 2; ++e) tmem_ld8_nowait(at + (uint32_t)(e * a.nt), v + 8 * e);
+                            tmem_wait_ld(v);
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            if constexpr (sizeof(T) == 4) {
+                            for (int j = 0; j < 8; ++j) {
                                 const float p = __uint_as_float(v[j]) + __uint_as_float(v[8 + j]);
                                 acc[g][8 * half + j] = fmaf(p, sc, acc[g][8 * half + j]);
-                            } else {
-                                // group e is an integer times 2^-8e: the sum in units of 2^-42
-                                int n[7];
+                            }
+                        } else {
+                            // group e is an integer times 2^-8e: the sum in units
+                            // of 2^-42, groups 0 .. 2 first
+                            long long hi[8];
+                            {
+                                uint32_t v[24];
 #pragma unroll
-                                for (int e = 0; e < 6; ++e)
-                                    n[e] = __float2int_rn(__uint_as_float(v[8 * e + j]) *
-                                                          __int_as_float((127 + 8 * e) << 23));
-                                n[6] = __float2int_rn(__uint_as_float(v[48 + j]) * 0x1p42f);
-                                const long long hi = (long long)n[0] * 65536 + (long long)(n[1] * 256LL + n[2]);
-                                const long long lo =
-                                    (long long)n[3] * (1 << 18) + (long long)n[4] * 1024 + (long long)n[5] * 4 + n[6];
-                                acc[g][8 * half + j] = fma((double)(hi * (1LL << 26) + lo), sc, acc[g][8 * half + j]);
+                                for (int e = 0; e < 3; ++e) tmem_ld8_nowait(at + (uint32_t)(e * a.nt), v + 8 * e);
+                                tmem_wait_ld(v);
+#pragma unroll
+                                for (int j = 0; j < 8; ++j)
+                                    hi[j] = (long long)unit_int<0>(v[j]) * 65536 +
+                                            (unit_int<8>(v[8 + j]) * 256LL + unit_int<16>(v[16 + j]));
+                            }
+                            uint32_t v[32];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) tmem_ld8_nowait(at + (uint32_t)((e + 3) * a.nt), v + 8 * e);
+                            tmem_wait_ld(v);
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) {
+                                const long long lo = (long long)unit_int<24>(v[j]) * (1 << 18) +
+                                                     (long long)unit_int<32>(v[8 + j]) * 1024 +
+                                                     (long long)unit_int<40>(v[16 + j]) * 4 + unit_int<42>(v[24 + j]);
+                                acc[g][8 * half + j] =
+                                    fma((double)(hi[j] * (1LL << 26) + lo), sc, acc[g][8 * half + j]);
                             }
                         }
                     }
@@ -680,7 +705,8 @@ static cudaError_t ex_run(Plan &P, int dir, const T *u, T *d, int accumulate, do
     const int z = m2l_slot_split((int64_t)ntiles * S.ncb[dir], P.num_sms);
     a.part = z > 1 ? (T *)P.m2l_part : nullptr;
     const size_t smem = (size_t)a.nstages * SL::kSlices * (kTcRows + a.nt) * kRowB + 1024;
-    ++g_launches, k_m2l_exact<T><<<dim3((unsigned)ntiles, (unsigned)S.ncb[dir], (unsigned)z), kExThreads, smem, s>>>(a);
+    ++g_launches, k_m2l_exact<T><<<dim3((unsigned)ntiles, (unsigned)S.ncb[dir], (unsigned)z), ex_threads<T>(),
+                                 smem, s>>>(a);
     if (z > 1) part_sum<T>(P, a.n_targets, z, a.ns, a.ld, a.part, d, accumulate, dbar, s);
     return cudaGetLastError();
 }

@@ -747,27 +747,27 @@ cudaError_t m2l_tiles_build(Plan &P, cudaStream_t s) {
 }
 
 // Slot split z and tiles per CTA (of 128 targets) of an untuned launch: the
-// pair with the shortest estimated time.  A stage takes 0.53 us with one tile
-// per CTA, 0.82 with two (measured: 12k and 1M packings); a CTA costs about
-// four slots of set-up and fill beside its 189 / z; a split writes and reads
-// every slot's partial products (about 5 TB/s).  So trees of up to some 6 k
-// targets split and larger ones run unsplit.  Measured, both sides: 12k
-// particles (585 boxes) 957 -> 537 us a step; 120k in a periodic cell (4681
-// boxes) 1885 -> 1171 (with the root's own kernels); 1M (150 CTAs of two
-// tiles) runs unsplit as before, 2531 us.
-static void tc_shape(int n1, int n2, int64_t n_t, int ncb, int np, int kblocks, int num_sms, int *z_out,
+// pair with the shortest estimated time.  An SM takes in a stage's bytes at
+// about 33 per clock, 68 KB per us (p = 6: 36 KB in 0.53 us with one tile per
+// CTA, 52 KB in 0.82 with two); a CTA costs about four slots of set-up and fill
+// beside its 189 / z.  A split stores every slot's partial products (2.6 TB/s
+// beside the products) and reads them back (5.4 TB/s).  Measured, both sides:
+// 12k particles (585 boxes) 957 -> 537 us a step; 120k in a periodic cell (4681
+// boxes) 1885 -> 1171 (with the root's own kernels); 1M (150 CTAs of two tiles)
+// runs unsplit as before, 2531 us.
+static void tc_shape(int n1, int n2, int ncb, int np, int kblocks, int num_sms, int *z_out,
                      int *tl_out) {
     double least = 1e30;
     *z_out = 1;
     *tl_out = 1;
-    const double traffic_us = 2.0 * kVSlots * (double)n_t * np * 4.0 / 5e6 + 4.0;
+    const double part_bytes = 4.0 * kVSlots * kTcRows * (double)n1 * np;
     for (int z = 1; z <= 63 && (z == 1 || (int64_t)n1 * ncb * z <= 8 * (int64_t)num_sms); ++z)
         for (int tl = 1; tl <= 2; ++tl) {
             if (tl == 2 && n2 == n1) continue;
             const int64_t ctas = (int64_t)(tl == 1 ? n1 : n2) * ncb * z;
-            const double t = (double)((ctas + num_sms - 1) / num_sms) * ((kVSlots + z - 1) / z + 4.0) * kblocks *
-                                 (tl == 1 ? 0.53 : 0.82) +
-                             (z > 1 ? traffic_us : 0.0);
+            const double stage_us = (tl * 2.0 * kTcRows + 2.0 * np / ncb) * kRowBytes / 68e3;
+            double t = (double)((ctas + num_sms - 1) / num_sms) * ((kVSlots + z - 1) / z + 4.0) * kblocks * stage_us;
+            if (z > 1) t = std::max(t, part_bytes / 2.6e6) + part_bytes / 5.4e6 + 6.0;
             if (t < 0.98 * least) {
                 least = t;
                 *z_out = z;
@@ -785,7 +785,7 @@ cudaError_t m2l_tensor_prepare(Plan &P) {
     }
     const M2lTiles &TS = tile_state(P);
     int z, tl;
-    tc_shape(TS.n_tiles[0], TS.n_tiles[1], P.m2l_class_start[8], S.ncb, S.np, S.kp / kKBlock, P.num_sms, &z, &tl);
+    tc_shape(TS.n_tiles[0], TS.n_tiles[1], S.ncb, S.np, S.kp / kKBlock, P.num_sms, &z, &tl);
     return m2l_part_reserve(P, z > 1 ? sizeof(float) * kVSlots * (size_t)TS.n_tiles[0] * kTcRows * S.np : 0);
 }
 
@@ -825,7 +825,7 @@ cudaError_t m2l_tensor(Plan &P, cudaStream_t s) {
     a.np = S.np;
     a.status = P.status;
     int z, tl_default;
-    tc_shape(TS.n_tiles[0], TS.n_tiles[1], P.m2l_class_start[8], S.ncb, S.np, S.kp / kKBlock, P.num_sms, &z,
+    tc_shape(TS.n_tiles[0], TS.n_tiles[1], S.ncb, S.np, S.kp / kKBlock, P.num_sms, &z,
              &tl_default);
     a.part = z > 1 ? (float *)P.m2l_part : nullptr;
     a.n_tiles = TS.n_tiles[0];
