@@ -14,9 +14,13 @@
 //     h l, l h, l l, h l2, l2 h, 2^-9 and less of it, in a second one.
 //   FP64 (eight BF16 slices): x = 2^-6 sum_i 2^-8i d_i, balanced base-256
 //     digits (|d_0| <= 64, |d_i| <= 128).  The products d_i d_j with i + j = g
-//     <= 5 go to the accumulator of g, where at most 160 (g + 1) of them sum
-//     to an integer below 2^24 (times 2^-8g), exactly; g = 6 and 7 share a
-//     seventh (2^-48 and 2^-56 of the first: rounding there is below 2^-60).
+//     <= 7 go to the accumulator of g, where (up to g = 6) at most 160 (g + 1)
+//     of them sum to an integer below 2^24 (times 2^-8g), exactly; at g = 7,
+//     2^-56 of the first, a rounding would be below 2^-79.
+//     The accumulators of g and the slices of the operator lie side by side,
+//     so one MMA of up to 256 columns multiplies slice i of the rows with four
+//     slices j of the operator: 24 MMAs per stage for the 72 products, whose
+//     issue one by one took longer than the tensor core does.
 //     The split scheme is Ozaki, Ogita, Oishi & Rump (Numer. Algorithms 59,
 //     2012) for error-free matrix products, with the digits of a fixed-point
 //     expansion.
@@ -66,16 +70,12 @@ struct Slicing<float> {
     static constexpr int kSlices = 3, kGroups = 2, kCols = 160, kChunkBlocks = 8;  // 8 x 32 x 2^16 = 2^24
     static constexpr int kProd = 4;                                                // producer warps
     static constexpr uint32_t kFmt = 0;                                            // FP16
-    __host__ __device__ static constexpr bool used(int i, int j) { return i + j <= 2; }
-    __host__ __device__ static constexpr int group(int i, int j) { return i + j == 0 ? 0 : 1; }
 };
 template <>
 struct Slicing<double> {
-    static constexpr int kSlices = 8, kGroups = 7, kCols = 64, kChunkBlocks = 5;  // K <= 160 per accumulation
+    static constexpr int kSlices = 8, kGroups = 8, kCols = 64, kChunkBlocks = 5;  // K <= 160 per accumulation
     static constexpr int kProd = 2;  // producer warps: with 12 or fewer warps the drain's 160 registers fit
     static constexpr uint32_t kFmt = 1;                                           // BF16
-    __host__ __device__ static constexpr bool used(int i, int j) { return i + j <= 7; }
-    __host__ __device__ static constexpr int group(int i, int j) { return i + j < 6 ? i + j : 6; }
 };
 
 template <typename T>
@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    const uint32_t buf_cols = (uint32_t)(NG * a.nt);
+    const uint32_t buf_cols = (uint32_t)(NG * nt);
     const uint32_t want_cols = buf_cols * a.nbuf;
     const uint32_t tmem_cols = want_cols <= 128 ? 128u : (want_cols <= 256 ? 256u : 512u);
     if (warp == kProd) {
@@ -348,7 +348,8 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
         // ---------------- MMA issuer ----------------
         // One accumulation per (slot, K chunk), in accumulator set w % nbuf.
         if (lane == 0) {
-            const uint32_t id = idesc_f16(nt, SL::kFmt);
+            const uint32_t id = idesc_f16(nt, SL::kFmt);  // (FP32)
+            const int wide = min(NS, 256 / nt);             // (FP64) operator slices per MMA, 256 columns at most
             int it = 0, w = 0;
             for (int s = s_lo; s < s_hi && !abort_s; ++s) {
                 for (int c = 0; c < a.nchunks && !abort_s; ++c, ++w) {
@@ -374,28 +375,34 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
                         const uint32_t sA = smem_u32(smem + (size_t)stage * stage_bytes);
                         // descriptors differ in the address field only
                         const uint64_t dA0 = sdesc_sw64(sA), dB0 = sdesc_sw64(sA + NS * kTileB);
-#pragma unroll
-                        for (int kk = 0; kk < 2; ++kk) {
-                            const uint32_t on = (kb > c * a.chunk_blocks || kk > 0) ? 1u : 0u;
-#pragma unroll
-                            for (int i = 0; i < NS; ++i) {
-                                const uint64_t dA = dA0 + (uint64_t)((i * kTileB + 32 * kk) >> 4);
-                                int last = -1;
-#pragma unroll
-                                for (int j = 0; j < NS; ++j)
-                                    if (SL::used(i, j)) last = j;
-#pragma unroll
-                                for (int j = 0; j < NS; ++j) {
-                                    if (!SL::used(i, j)) continue;
-                                    const uint64_t dB = dB0 + (uint64_t)((j * b_slice + 32 * kk) >> 4);
-                                    const uint32_t acc = acc0 + (uint32_t)(SL::group(i, j) * a.nt);
-                                    // the first product of a group is d_0 d_g
-                                    const uint32_t add = (i == 0 && SL::group(i, j) == j) ? on : 1u;
-                                    if (last == 0) mma_f16(acc, dA, dB, id, add);
-                                    else if (j == 0) mma_f16_fill(acc, dA, dB, id, add);
-                                    else if (j == last) mma_f16_lastuse(acc, dA, dB, id, add);
-                                    else mma_f16_use(acc, dA, dB, id, add);
+                        if constexpr (sizeof(T) == 8) {
+                            // rows' slice i with operator slices j .. j + m - 1,
+                            // into the accumulators i + j .. i + j + m - 1
+                            for (int kk = 0; kk < 2; ++kk) {
+                                const uint32_t on = (kb > c * a.chunk_blocks || kk > 0) ? 1u : 0u;
+                                for (int i = 0; i < NS; ++i) {
+                                    const uint64_t dA = dA0 + (uint64_t)((i * kTileB + 32 * kk) >> 4);
+                                    for (int j = 0; j < NS - i; j += wide) {
+                                        const int m = min(wide, NS - i - j);
+                                        const uint64_t dB = dB0 + (uint64_t)((j * b_slice + 32 * kk) >> 4);
+                                        mma_f16(acc0 + (uint32_t)((i + j) * nt), dA, dB, idesc_f16(m * nt, SL::kFmt),
+                                                i == 0 ? on : 1u);  // d_0 meets every accumulator first
+                                    }
                                 }
+                            }
+                        } else {
+#pragma unroll
+                            for (int kk = 0; kk < 2; ++kk) {
+                                const uint32_t on = (kb > c * a.chunk_blocks || kk > 0) ? 1u : 0u;
+                                const uint64_t dA = dA0 + (uint64_t)(2 * kk), dB = dB0 + (uint64_t)(2 * kk);
+                                const uint32_t a_step = kTileB >> 4, b_step = b_slice >> 4;
+                                const uint32_t acc1 = acc0 + (uint32_t)nt;
+                                mma_f16_fill(acc0, dA, dB, id, on);                           // h h
+                                mma_f16_use(acc1, dA, dB + b_step, id, on);                   // h l
+                                mma_f16_lastuse(acc1, dA, dB + 2 * b_step, id, 1u);           // h l2
+                                mma_f16_fill(acc1, dA + a_step, dB, id, 1u);                  // l h
+                                mma_f16_lastuse(acc1, dA + a_step, dB + b_step, id, 1u);      // l l
+                                mma_f16(acc1, dA + 2 * a_step, dB, id, 1u);                   // l2 h
                             }
                         }
                         mma_commit(smem_u32(&empty_bar[stage]));
@@ -459,7 +466,7 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
                         if constexpr (sizeof(T) == 4) {
                             uint32_t v[16];
 #pragma unroll
-                            for (int e = 0; e < 2; ++e) tmem_ld8_nowait(at + (uint32_t)(e * a.nt), v + 8 * e);
+                            for (int e = 0; e < 2; ++e) tmem_ld8_nowait(at + (uint32_t)(e * nt), v + 8 * e);
                             tmem_wait_ld(v);
 #pragma unroll
                             for (int j = 0; j < 8; ++j) {
@@ -468,29 +475,39 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
                             }
                         } else {
                             // group e is an integer times 2^-8e: the sum in units
-                            // of 2^-42, groups 0 .. 2 first
-                            long long hi[8];
+                            // of 2^-42, three batches of groups
+                            long long sum[8];
                             {
                                 uint32_t v[24];
 #pragma unroll
-                                for (int e = 0; e < 3; ++e) tmem_ld8_nowait(at + (uint32_t)(e * a.nt), v + 8 * e);
+                                for (int e = 0; e < 3; ++e) tmem_ld8_nowait(at + (uint32_t)(e * nt), v + 8 * e);
                                 tmem_wait_ld(v);
 #pragma unroll
                                 for (int j = 0; j < 8; ++j)
-                                    hi[j] = (long long)unit_int<0>(v[j]) * 65536 +
-                                            (unit_int<8>(v[8 + j]) * 256LL + unit_int<16>(v[16 + j]));
+                                    sum[j] = ((long long)unit_int<0>(v[j]) * 65536 +
+                                              (unit_int<8>(v[8 + j]) * 256LL + unit_int<16>(v[16 + j])))
+                                             * (1LL << 26);
                             }
-                            uint32_t v[32];
+                            {
+                                uint32_t v[24];
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) tmem_ld8_nowait(at + (uint32_t)((e + 3) * a.nt), v + 8 * e);
+                                for (int e = 0; e < 3; ++e) tmem_ld8_nowait(at + (uint32_t)((e + 3) * nt), v + 8 * e);
+                                tmem_wait_ld(v);
+#pragma unroll
+                                for (int j = 0; j < 8; ++j)
+                                    sum[j] += (long long)unit_int<24>(v[j]) * (1 << 18) +
+                                              (long long)unit_int<32>(v[8 + j]) * 1024 +
+                                              (long long)unit_int<40>(v[16 + j]) * 4;
+                            }
+                            uint32_t v[16];
+#pragma unroll
+                            for (int e = 0; e < 2; ++e) tmem_ld8_nowait(at + (uint32_t)((e + 6) * nt), v + 8 * e);
                             tmem_wait_ld(v);
 #pragma unroll
                             for (int j = 0; j < 8; ++j) {
-                                const long long lo = (long long)unit_int<24>(v[j]) * (1 << 18) +
-                                                     (long long)unit_int<32>(v[8 + j]) * 1024 +
-                                                     (long long)unit_int<40>(v[16 + j]) * 4 + unit_int<42>(v[24 + j]);
-                                acc[g][8 * half + j] =
-                                    fma((double)(hi[j] * (1LL << 26) + lo), sc, acc[g][8 * half + j]);
+                                sum[j] += unit_int<42>(
+                                    __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(v[8 + j])));
+                                acc[g][8 * half + j] = fma((double)sum[j], sc, acc[g][8 * half + j]);
                             }
                         }
                     }
