@@ -329,12 +329,9 @@ kifmm_status kifmm_plan_create(const kifmm_plan_desc *desc, kifmm_plan **out) {
         {(void **)&P.out_scale, sizeof(double) * 2 * P.sys_cap},
         {(void **)&P.bbox_ord, sizeof(unsigned long long) * 6 * P.sys_cap},
         {(void **)&P.hist, sizeof(uint32_t) * P.hist_elems},
-        {(void **)&P.status, sizeof(int)},
+        {(void **)&P.rb_dev, sizeof(Plan::Counts)},
         {(void **)&P.moved, sizeof(int)},
         {(void **)&P.spec_buf, sizeof(int64_t) * 32},
-        {(void **)&P.spec_fail, sizeof(int)},
-        {(void **)&P.part_counts, sizeof(uint32_t) * 4 * 256},
-        {(void **)&P.list_totals, sizeof(unsigned long long) * 4},
         {(void **)&P.energy_chunk_start, sizeof(int32_t) * (P.sys_cap + 1)},
         {(void **)&P.qsum, sizeof(double) * 2},
         {&P.frc, P.stokes ? esz * 3 * n : 8},
@@ -353,6 +350,9 @@ kifmm_status kifmm_plan_create(const kifmm_plan_desc *desc, kifmm_plan **out) {
     P.scan_tmp_elems = std::max(P.scan_tmp_elems, scan_tmp_needed((int64_t)256 * nblk) + 8);
     if (plan_alloc(P, (void **)&P.scan_tmp, sizeof(uint32_t) * P.scan_tmp_elems) != cudaSuccess)
         return fail(KIFMM_ERR_CUDA);
+    P.status = &P.rb_dev->status;
+    P.list_totals = P.rb_dev->vx;
+    P.part_counts = &P.rb_dev->part_counts[0][0];
     if (cudaMemset(P.status, 0, sizeof(int)) != cudaSuccess) return fail(KIFMM_ERR_CUDA);
     if (cudaMallocHost((void **)&P.rb, sizeof(Plan::Readback)) != cudaSuccess) return fail(KIFMM_ERR_CUDA);
     if (cudaDeviceSynchronize() != cudaSuccess) return fail(KIFMM_ERR_CUDA);
@@ -452,7 +452,8 @@ static kifmm_status set_sources_impl(Plan &P, const void *xyz, const void *q, cu
     }
     // the one synchronisation after the octree levels: the status word and,
     // for new lists, their sizes and the partition counts
-    API_CUDA(cudaMemcpyAsync(&P.rb->status, P.status, sizeof(int), cudaMemcpyDeviceToHost, s));
+    API_CUDA(cudaMemcpyAsync(static_cast<Plan::Counts *>(P.rb), P.rb_dev, sizeof(Plan::Counts), cudaMemcpyDeviceToHost,
+                             s));
     API_CUDA(cudaStreamSynchronize(s));
     const int st = P.rb->status;
     if (!P.lists_reused) {

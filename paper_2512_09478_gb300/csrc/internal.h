@@ -12,6 +12,7 @@
 
 namespace kifmm {
 
+constexpr int kSpecFail = 31;       // word of the all-levels build's flag behind the level boundaries
 constexpr int kMaxLevel = 20;       // 21-bit quantisation per axis
 constexpr int kNumM2L = 316;        // offsets in {-3..3}^3 minus {-1..1}^3
 constexpr int kVSlots = 189;        // V-list slots per octant class (6^3 - 3^3)
@@ -137,6 +138,7 @@ struct Plan {
     uint32_t *vals[2] = {nullptr, nullptr};
     uint64_t *keys_user = nullptr;  // keys in caller order (introspection)
     uint32_t *perm = nullptr;       // sorted -> caller index
+    uint64_t *keys_sorted = nullptr;  // the sorted keys (one of keys[])
     void *pts = nullptr;            // [N] {dx, dy, dz, q} leaf-relative, compute type
     double *near_pot = nullptr;     // scratch accumulators (FP64 final sums)
     int64_t *sys_off_d = nullptr;   // [S+1]
@@ -204,12 +206,19 @@ struct Plan {
     uint32_t *part_counts = nullptr; // [4][256]
     // What set_sources reads back at its final synchronisation (pinned host
     // memory): the status word, the list sizes and the partition counts.
-    struct Readback {
+    // The device holds the first part in the same layout (rb_dev), so that one
+    // copy brings it; status, list_totals and part_counts point into it.
+    struct Counts {
         int status;
         uint32_t uw[2];                 // U and W list entries
         unsigned long long vx[4];       // V and X list entries
-        uint32_t part_counts[4][256];
+        uint32_t part_counts[4][256];   // (directly after vx: zeroed together)
+    };
+    struct Readback : Counts {
+        int64_t levels[32];             // the all-levels build: level boundaries, [kSpecFail]: it gave up
+        uint32_t level_total;           // level-by-level build: children of one level
     } *rb = nullptr;
+    Counts *rb_dev = nullptr;
     unsigned long long *list_totals = nullptr;  // [4] V and X list sizes
     // Box lists grouped by a small key (stable, canonical order within a key):
     //   0: octant class of boxes with a V list (8 = none)
@@ -248,8 +257,7 @@ struct Plan {
     // ---- status ----
     int *status = nullptr;   // device status word
     int *moved = nullptr;    // device flag of the tree reuse test
-    int64_t *spec_buf = nullptr;  // [32] all-levels octree build: level boundaries
-    int *spec_fail = nullptr;     // the all-levels build outgrew the box arrays
+    int64_t *spec_buf = nullptr;  // [32] all-levels octree build: level boundaries; [kSpecFail]: outgrew the box arrays
     uint32_t *os_cnt = nullptr;   // [levels][particle tiles] box counts, then box offsets
     size_t os_cnt_elems = 0;
     cudaStream_t last_stream = nullptr;

@@ -328,7 +328,9 @@ constexpr int kScanBlock = 512;
 constexpr int kScanItems = 4;
 constexpr int kScanTile = kScanBlock * kScanItems;
 
-__global__ void k_scan_tiles(const uint32_t *__restrict__ in, uint32_t *out, int64_t n, uint32_t *sums) {
+// One tile (blockIdx.x) of an exclusive scan; its total to *sum.
+__device__ __forceinline__ void scan_tile(const uint32_t *__restrict__ in, uint32_t *out, int64_t n,
+                                                 uint32_t *sum) {
     __shared__ uint32_t ws[kScanBlock / 32];
     const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
     uint32_t v[kScanItems];
@@ -340,7 +342,7 @@ __global__ void k_scan_tiles(const uint32_t *__restrict__ in, uint32_t *out, int
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t x = t;
     for (int o = 1; o < 32; o <<= 1) {
-        uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= o) x += y;
     }
     if (lane == 31) ws[warp] = x;
@@ -348,7 +350,7 @@ __global__ void k_scan_tiles(const uint32_t *__restrict__ in, uint32_t *out, int
     if (warp == 0) {
         uint32_t w = (lane < kScanBlock / 32) ? ws[lane] : 0u;
         for (int o = 1; o < 32; o <<= 1) {
-            uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
+            const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
             if (lane >= o) w += y;
         }
         if (lane < kScanBlock / 32) ws[lane] = w;
@@ -359,7 +361,10 @@ __global__ void k_scan_tiles(const uint32_t *__restrict__ in, uint32_t *out, int
         if (base + k < n) out[base + k] = run;
         run += v[k];
     }
-    if (threadIdx.x == kScanBlock - 1) sums[blockIdx.x] = run;
+    if (threadIdx.x == kScanBlock - 1) *sum = run;
+}
+__global__ void k_scan_tiles(const uint32_t *__restrict__ in, uint32_t *out, int64_t n, uint32_t *sums) {
+    scan_tile(in, out, n, sums + blockIdx.x);
 }
 
 __global__ void k_scan_add(uint32_t *out, int64_t n, const uint32_t *__restrict__ sums_scanned) {
@@ -547,12 +552,16 @@ __device__ __forceinline__ uint32_t os_box_levels(const OsPoint &p, const uint64
     return f;
 }
 
-// Pass 1: boxes of levels 1 .. L per particle tile -> cnt[(l - 1) ntiles + tile].
+// Pass 1: boxes of levels 1 .. L per particle tile -> cnt[(l - 1) ntiles + tile],
+// and each particle's levels -> flags (the emit pass searched the keys again:
+// 41 of 66 us of the two passes at 1M).
 __global__ void __launch_bounds__(kOsTile) k_os_count(int64_t n, const uint64_t *__restrict__ keys,
                                                       const int64_t *__restrict__ off, int S, int L, int M,
-                                                      int max_depth, int ntiles, uint32_t *cnt) {
+                                                      int max_depth, int ntiles, uint32_t *cnt,
+                                                      uint32_t *__restrict__ flags) {
     const OsPoint p = os_point(n, keys, off, S);
     const uint32_t f = os_box_levels(p, keys, L, M, max_depth);
+    if (p.valid) flags[p.i] = f;
     for (int l = 1; l <= L; ++l) {
         const int c = __syncthreads_count((f >> (l - 1)) & 1u);
         if (threadIdx.x == 0) cnt[(size_t)(l - 1) * ntiles + blockIdx.x] = (uint32_t)c;
@@ -567,7 +576,7 @@ __global__ void __launch_bounds__(kOsTile) k_os_count(int64_t n, const uint64_t 
 // set when the boxes outgrow the arrays (then nothing else is written).
 __global__ void __launch_bounds__(1024) k_os_scan(int L, int ntiles, int S, int64_t cap,
                                                   const uint32_t *__restrict__ cnt, uint32_t *__restrict__ first_idx,
-                                                  int64_t *lb, int *fail) {
+                                                  int64_t *lb, int64_t *fail) {
     __shared__ uint32_t ws[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t len = (int64_t)L * ntiles;
@@ -645,15 +654,15 @@ __device__ __forceinline__ int64_t warp_segment_end(const uint64_t *__restrict__
 // index is the tile's first box of the level plus the boxes of the level
 // before it in the tile (ballots, then the warps' counts).
 __global__ void __launch_bounds__(kOsTile) k_os_emit(int64_t n, const uint64_t *__restrict__ keys,
-                                                     const int64_t *__restrict__ off, int S, int L, int M,
-                                                     int max_depth, int ntiles, const uint32_t *__restrict__ base_idx,
-                                                     const int *fail, int32_t *lvl, int32_t *cx, int32_t *cy,
+                                                     const int64_t *__restrict__ off, int S, int L, int ntiles,
+                                                     const uint32_t *__restrict__ flags,
+                                                     const uint32_t *__restrict__ base_idx, const int64_t *fail, int32_t *lvl, int32_t *cx, int32_t *cy,
                                                      int32_t *cz, int32_t *first, int32_t *cnt, int32_t *sys) {
     __shared__ uint32_t wc[kOsTile / 32];
     if (*fail) return;
     const OsPoint p = os_point(n, keys, off, S);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t f = os_box_levels(p, keys, L, M, max_depth);
+    const uint32_t f = p.valid ? flags[p.i] : 0u;
     for (int l = 1; l <= L; ++l) {
         const bool box = (f >> (l - 1)) & 1u;
         const unsigned m = __ballot_sync(0xffffffffu, box);
@@ -698,7 +707,7 @@ __device__ __forceinline__ int64_t last_le(const int32_t *__restrict__ a, int64_
 // at or before the box's) and child ranges (the boxes of the level below
 // whose first particle lies in the box's range); the boxes of level L get
 // none here (the level-by-level build continues from them if one splits).
-__global__ void k_os_link(const int64_t *__restrict__ lb, int L, int M, int max_depth, const int *fail,
+__global__ void k_os_link(const int64_t *__restrict__ lb, int L, int M, int max_depth, const int64_t *fail,
                           const int32_t *__restrict__ lvl, const int32_t *__restrict__ first,
                           const int32_t *__restrict__ cnt, int32_t *parent, int32_t *child_first, int32_t *nchild) {
     if (*fail) return;
@@ -911,7 +920,10 @@ __device__ __forceinline__ int dev_colleagues_v(int64_t b, int lane, int level, 
                                                 const int32_t *__restrict__ cy, const int32_t *__restrict__ cz,
                                                 int32_t *coll, int32_t *vdense, const ListShifts &sh) {
     int32_t *cb = coll + b * kColl;
-    // cb and the V table were set to -1 by memsets of the whole arrays
+    // empty slots first (the warp's own rows)
+    for (int k = lane; k < kColl; k += 32) cb[k] = -1;
+    for (int k = lane; k < kVSlots; k += 32) vdense[b * kVSlots + k] = -1;
+    __syncwarp();
     if (level == 0) {
         if (sh.coll) {
             if (lane < kColl) {
@@ -1076,10 +1088,12 @@ __global__ void __launch_bounds__(128) k_uw(int64_t nb, int pass, int thr, const
                      const int32_t *__restrict__ coarse, const int32_t *__restrict__ ncoarse,
                      uint32_t *u_cnt, uint32_t *w_cnt, const uint32_t *__restrict__ u_ptr,
                      const uint32_t *__restrict__ w_ptr, int32_t *u_idx, int32_t *w_idx, int64_t u_cap,
-                     int64_t w_cap, int *status, ListShifts sh) {
+                     int64_t w_cap, int *status, ListShifts sh, int32_t *wsrc_flag, uint32_t *uw_total) {
     const int64_t b = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (b >= nb) return;  // uniform for the warp
+    if (pass == 0 && lane == 0) wsrc_flag[b] = 0;  // (marked after pass 1)
+    if (pass == 1 && b == 0 && lane < 2) uw_total[lane] = lane == 0 ? u_ptr[nb] : w_ptr[nb];
     if (nchild[b] != 0) {
         if (pass == 0 && lane == 0) u_cnt[b] = w_cnt[b] = 0;
         return;
@@ -1179,6 +1193,45 @@ __global__ void k_mark_w(int64_t cap, const uint32_t *__restrict__ w_total, cons
 inline unsigned grid_for(int64_t n, int block) { return (unsigned)((n + block - 1) / block); }
 
 }  // namespace
+
+// Two scans of n entries each (blockIdx.y: which), their totals at out[n].
+static __global__ void k_scan_pair(const uint32_t *__restrict__ in0, uint32_t *out0, const uint32_t *__restrict__ in1,
+                                   uint32_t *out1, int64_t n, uint32_t *sums) {
+    if (gridDim.x == 1) {  // one tile: its sum is the total
+        if (blockIdx.y == 0) scan_tile(in0, out0, n, out0 + n);
+        else scan_tile(in1, out1, n, out1 + n);
+    } else if (blockIdx.y == 0) {
+        scan_tile(in0, out0, n, sums + blockIdx.x);
+    } else {
+        scan_tile(in1, out1, n, sums + gridDim.x + blockIdx.x);
+    }
+}
+// The tiles' offsets: every block sums the tile totals before its own (at most
+// a few hundred) and adds them; the last tile also writes the total.
+static __global__ void k_scan_pair_add(uint32_t *out0, uint32_t *out1, int64_t n, const uint32_t *__restrict__ sums) {
+    __shared__ uint32_t red[kScanBlock / 32];
+    const uint32_t *sm = sums + (blockIdx.y ? gridDim.x : 0);
+    uint32_t *out = blockIdx.y ? out1 : out0;
+    uint32_t t = 0;
+    for (unsigned i = threadIdx.x; i < blockIdx.x; i += blockDim.x) t += sm[i];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
+    __syncthreads();
+    uint32_t add = 0;
+    for (int w = 0; w < kScanBlock / 32; ++w) add += red[w];
+    const int64_t base = (int64_t)blockIdx.x * kScanTile;
+    for (int k = threadIdx.x; k < kScanTile; k += kScanBlock)
+        if (base + k < n) out[base + k] += add;
+    if (blockIdx.x + 1 == gridDim.x && threadIdx.x == 0) out[n] = add + sm[blockIdx.x];
+}
+static cudaError_t exclusive_scan_pair(const uint32_t *in0, uint32_t *out0, const uint32_t *in1, uint32_t *out1,
+                                       int64_t n, uint32_t *tmp, size_t tmp_elems, cudaStream_t s) {
+    const int64_t nblk = std::max<int64_t>(1, (n + kScanTile - 1) / kScanTile);
+    if ((size_t)(2 * nblk) > tmp_elems) return cudaErrorInvalidValue;
+    ++g_launches, k_scan_pair<<<dim3((unsigned)nblk, 2), kScanBlock, 0, s>>>(in0, out0, in1, out1, n, tmp);
+    if (nblk > 1) ++g_launches, k_scan_pair_add<<<dim3((unsigned)nblk, 2), kScanBlock, 0, s>>>(out0, out1, n, tmp);
+    return cudaGetLastError();
+}
 
 size_t scan_tmp_needed(int64_t n) {
     size_t total = 0;
@@ -1330,7 +1383,6 @@ cudaError_t partition_boxes(Plan &P, cudaStream_t s) {
         KIFMM_CUDA_TRY(plan_alloc(P, (void **)&P.scan_tmp, sizeof(uint32_t) * P.scan_tmp_elems));
     }
     ++g_launches, k_child8<<<grid_for(nb, 256), 256, 0, s>>>(nb, P.child_first, P.nchild, P.cx, P.cy, P.cz, P.child8);
-    KIFMM_CUDA_TRY(cudaMemsetAsync(P.part_counts, 0, sizeof(uint32_t) * 4 * 256, s));
     const dim3 grid((unsigned)nblk, 4);
     ++g_launches, k_part_hist<<<grid, kBlock, 0, s>>>(nb, nblk, P.nv, P.nchild, P.lvl, P.wsrc_flag, P.cx, P.cy, P.cz,
                                                       P.hist, P.part_counts);
@@ -1338,10 +1390,8 @@ cudaError_t partition_boxes(Plan &P, cudaStream_t s) {
     ++g_launches, k_part_scatter<<<grid, kBlock, 0, s>>>(nb, nblk, P.nv, P.nchild, P.lvl, P.wsrc_flag, P.cx, P.cy,
                                                          P.cz, P.hist + nh, P.part_list[0], P.part_list[1],
                                                          P.part_list[2], P.part_list[3]);
-    // the four key histograms come back with set_sources' final
-    // synchronisation (the gather reads the leaf count on the device)
-    KIFMM_CUDA_TRY(cudaMemcpyAsync(P.rb->part_counts, P.part_counts, sizeof(P.rb->part_counts),
-                                   cudaMemcpyDeviceToHost, s));
+    // (the four key histograms come back with set_sources' final
+    // synchronisation; the gather reads the leaf count on the device)
     P.m2l_targets = P.part_list[0];
     P.leaves = P.part_list[1];
     return cudaGetLastError();
@@ -1421,19 +1471,21 @@ static int levels_sorted(int npass) { return (8 * npass - 1) / 3; }
 
 // Stable LSD sort on the top `npass` key digits (then the system id, for
 // batched sorts): equal top digits keep the incoming order.
-static cudaError_t radix_sort(Plan &P, int64_t n, cudaStream_t s, int &cur, int npass) {
-    const int nblk = (int)((n + kTile - 1) / kTile);
+// The keys start in keys[cur], the values in vin; the values of the last pass
+// go to P.perm, the keys to keys[cur] (cur updated).
+static cudaError_t radix_sort(Plan &P, int64_t n, cudaStream_t s, int &cur, const uint32_t *vin, int npass) {
     struct Pass { int mode, shift; };
     std::vector<Pass> passes;
     for (int sh = 64 - 8 * npass; sh < 64; sh += 8) passes.push_back({0, sh});
     if (P.n_sys > 1) {
         for (int sh = 0; (1LL << sh) < P.n_sys; sh += 8) passes.push_back({1, sh});
     }
-    (void)nblk;
-    for (const Pass &ps : passes) {
+    for (size_t i = 0; i < passes.size(); ++i) {
         const int nxt = cur ^ 1;
-        KIFMM_CUDA_TRY(radix_pass(P, P.keys[cur], P.vals[cur], P.keys[nxt], P.vals[nxt], n, ps.mode, ps.shift, s));
+        uint32_t *vout = i + 1 == passes.size() ? P.perm : P.vals[nxt];
+        KIFMM_CUDA_TRY(radix_pass(P, P.keys[cur], vin, P.keys[nxt], vout, n, passes[i].mode, passes[i].shift, s));
         cur = nxt;
+        vin = vout;
     }
     return cudaSuccess;
 }
@@ -1489,13 +1541,12 @@ cudaError_t build_tree(Plan &P, const void *xyz, const void *q, cudaStream_t s) 
     want = std::max(1, std::min(want, P.desc.max_depth));
     int npass = 1;
     while (npass < 8 && levels_sorted(npass) < want) ++npass;
+    int cur = 0;
+    const uint32_t *vin = P.vals[0];
     for (;;) {
-        int cur = 0;
-        KIFMM_CUDA_TRY(radix_sort(P, n, s, cur, npass));
-        if (cur != 0) {
-            KIFMM_CUDA_TRY(cudaMemcpyAsync(P.keys[0], P.keys[1], sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, s));
-            KIFMM_CUDA_TRY(cudaMemcpyAsync(P.vals[0], P.vals[1], sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, s));
-        }
+        KIFMM_CUDA_TRY(radix_sort(P, n, s, cur, vin, npass));
+        P.keys_sorted = P.keys[cur];
+        vin = P.perm;  // a second sort (eight passes or more) starts from this order
         cudaError_t e = build_levels(P, s, npass < 8 ? levels_sorted(npass) : kMaxLevel + 1);
         if (e == cudaErrorNotReady) {  // a node below the sorted levels must split
             npass = 8;
@@ -1505,7 +1556,6 @@ cudaError_t build_tree(Plan &P, const void *xyz, const void *q, cudaStream_t s) 
         break;
     }
     P.sort_passes = npass;
-    KIFMM_CUDA_TRY(cudaMemcpyAsync(P.perm, P.vals[0], sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, s));
     return cudaGetLastError();  // the particle records follow once the leaves are listed
 }
 
@@ -1553,30 +1603,29 @@ static cudaError_t build_levels(Plan &P, cudaStream_t s, int lsort) {
         }
         const int M = P.desc.leaf_cap, D = P.desc.max_depth;
         if (ntiles > 0)
-            ++g_launches, k_os_count<<<ntiles, kOsTile, 0, s>>>(n, P.keys[0], P.sys_off_d, S, lspec, M, D, ntiles,
-                                                               P.os_cnt);
+            ++g_launches, k_os_count<<<ntiles, kOsTile, 0, s>>>(n, P.keys_sorted, P.sys_off_d, S, lspec, M, D, ntiles,
+                                                               P.os_cnt, P.vals[0]);
         uint32_t *first_idx = P.os_cnt + (size_t)lspec * std::max(ntiles, 1);
         ++g_launches, k_os_scan<<<1, 1024, 0, s>>>(lspec, ntiles, S, P.box_cap, P.os_cnt, first_idx, lsd,
-                                                   P.spec_fail);
+                                                   lsd + kSpecFail);
         if (ntiles > 0)
-            ++g_launches, k_os_emit<<<ntiles, kOsTile, 0, s>>>(n, P.keys[0], P.sys_off_d, S, lspec, M, D, ntiles,
-                                                              first_idx, P.spec_fail, P.lvl, P.cx, P.cy, P.cz,
+            ++g_launches, k_os_emit<<<ntiles, kOsTile, 0, s>>>(n, P.keys_sorted, P.sys_off_d, S, lspec, ntiles, P.vals[0],
+                                                              first_idx, lsd + kSpecFail, P.lvl, P.cx, P.cy, P.cz,
                                                               P.first, P.cnt, P.sys);
         ++g_launches, k_os_link<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(grid_for(need, 256),
                                                                                     (int64_t)P.num_sms * 8)),
-                                  256, 0, s>>>(lsd, lspec, M, D, P.spec_fail, P.lvl, P.first, P.cnt, P.parent,
+                                  256, 0, s>>>(lsd, lspec, M, D, lsd + kSpecFail, P.lvl, P.first, P.cnt, P.parent,
                                                P.child_first, P.nchild);
         KIFMM_CUDA_TRY(cudaGetLastError());
-        std::vector<int64_t> lsh(lspec + 2);
-        int fail = 0;
-        KIFMM_CUDA_TRY(cudaMemcpyAsync(lsh.data(), lsd, sizeof(int64_t) * lsh.size(), cudaMemcpyDeviceToHost, s));
-        KIFMM_CUDA_TRY(cudaMemcpyAsync(&fail, P.spec_fail, sizeof(int), cudaMemcpyDeviceToHost, s));
+        int64_t *lsh = P.rb->levels;
+        KIFMM_CUDA_TRY(cudaMemcpyAsync(lsh, lsd, sizeof(P.rb->levels), cudaMemcpyDeviceToHost, s));
         KIFMM_CUDA_TRY(cudaStreamSynchronize(s));
+        const bool fail = lsh[kSpecFail] != 0;
         if (!fail) {
             // keep the non-empty levels; an empty one ends the tree
             int last = 0;
             while (last + 1 <= lspec && lsh[last + 2] > lsh[last + 1]) ++last;
-            P.level_start.assign(lsh.begin(), lsh.begin() + last + 2);
+            P.level_start.assign(lsh, lsh + last + 2);
             level = last;
             ls = lsh[last];
             le = lsh[last + 1];
@@ -1602,14 +1651,14 @@ static cudaError_t build_levels(Plan &P, cudaStream_t s, int lsort) {
     while (true) {
         const int64_t m = le - ls;
         ++g_launches, k_split<<<grid_for(m, 4), 128, 0, s>>>(ls, le, level, P.desc.leaf_cap, P.desc.max_depth,
-                                                             P.keys[0], P.first, P.cnt, P.tmp_nchild,
+                                                             P.keys_sorted, P.first, P.cnt, P.tmp_nchild,
                                                              P.child_rng);
         uint32_t *scan_out = P.tmp_nchild + P.box_cap;
         KIFMM_CUDA_TRY(exclusive_scan_u32(P.tmp_nchild, scan_out, m, total_dev, P.scan_tmp,
                                           P.scan_tmp_elems - 1, s));
-        uint32_t total = 0;
-        KIFMM_CUDA_TRY(cudaMemcpyAsync(&total, total_dev, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        KIFMM_CUDA_TRY(cudaMemcpyAsync(&P.rb->level_total, total_dev, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
         KIFMM_CUDA_TRY(cudaStreamSynchronize(s));
+        const uint32_t total = P.rb->level_total;
         if (level >= lsort && total > 0) return cudaErrorNotReady;
         if (le + (int64_t)total > P.box_cap) {
             KIFMM_CUDA_TRY(grow_tree_arrays(P, 2 * (le + (int64_t)total) + 1024, le));
@@ -1758,9 +1807,8 @@ static ListShifts list_shifts(const Plan &P) {
 
 cudaError_t build_lists(Plan &P, cudaStream_t s) {
     const int64_t nb = P.nb;
-    KIFMM_CUDA_TRY(cudaMemsetAsync(P.coll, 0xFF, sizeof(int32_t) * kColl * nb, s));
-    KIFMM_CUDA_TRY(cudaMemsetAsync(P.vdense, 0xFF, sizeof(int32_t) * kVSlots * nb, s));
-    KIFMM_CUDA_TRY(cudaMemsetAsync(P.list_totals, 0, sizeof(unsigned long long) * 4, s));
+    // the list totals and (for partition_boxes) the key counts
+    KIFMM_CUDA_TRY(cudaMemsetAsync(&P.rb_dev->vx, 0, sizeof(P.rb_dev->vx) + sizeof(P.rb_dev->part_counts), s));
     for (int l = 0; l <= P.max_level; ++l) {
         const int64_t ls = P.level_start[l], le = P.level_start[l + 1];
         const unsigned g = grid_for(le - ls, 8);  // warp per box, 8 per block
@@ -1773,23 +1821,17 @@ cudaError_t build_lists(Plan &P, cudaStream_t s) {
     const unsigned g = grid_for(nb, 4);  // a warp per box, 4 per block
     ++g_launches, k_uw<<<g, 128, 0, s>>>(nb, 0, P.direct_thr, P.parent, P.cnt, P.child_first, P.nchild, P.lvl,
                                          P.cx, P.cy, P.cz, P.coll, P.coarse, P.ncoarse, P.u_cnt, P.w_cnt, nullptr,
-                                         nullptr, nullptr, nullptr, 0, 0, P.status, list_shifts(P));
-    // two scans, totals in the last two scratch words, then appended to the
-    // offsets; the sizes come back to the host with set_sources' final
-    // synchronisation (no round trip here: the fill pass writes only inside
-    // the storage and flags a list that outgrew it)
-    uint32_t *tot_u = P.scan_tmp + P.scan_tmp_elems - 1, *tot_w = P.scan_tmp + P.scan_tmp_elems - 2;
-    KIFMM_CUDA_TRY(exclusive_scan_u32(P.u_cnt, P.u_ptr, nb, tot_u, P.scan_tmp, P.scan_tmp_elems - 2, s));
-    KIFMM_CUDA_TRY(exclusive_scan_u32(P.w_cnt, P.w_ptr, nb, tot_w, P.scan_tmp, P.scan_tmp_elems - 2, s));
-    KIFMM_CUDA_TRY(cudaMemcpyAsync(P.u_ptr + nb, tot_u, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
-    KIFMM_CUDA_TRY(cudaMemcpyAsync(P.w_ptr + nb, tot_w, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
-    KIFMM_CUDA_TRY(cudaMemcpyAsync(&P.rb->uw[0], tot_u, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    KIFMM_CUDA_TRY(cudaMemcpyAsync(&P.rb->uw[1], tot_w, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    KIFMM_CUDA_TRY(cudaMemcpyAsync(P.rb->vx, P.list_totals, sizeof(P.rb->vx), cudaMemcpyDeviceToHost, s));
+                                         nullptr, nullptr, nullptr, 0, 0, P.status, list_shifts(P), P.wsrc_flag,
+                                         nullptr);
+    // both scans in one set of launches, the totals appended to the offsets;
+    // the sizes come back to the host with set_sources' final synchronisation
+    // (no round trip here: the fill pass writes only inside the storage, and
+    // the host sees a list that outgrew it)
+    KIFMM_CUDA_TRY(exclusive_scan_pair(P.u_cnt, P.u_ptr, P.w_cnt, P.w_ptr, nb, P.scan_tmp, P.scan_tmp_elems - 2, s));
     ++g_launches, k_uw<<<g, 128, 0, s>>>(nb, 1, P.direct_thr, P.parent, P.cnt, P.child_first, P.nchild, P.lvl,
                                          P.cx, P.cy, P.cz, P.coll, P.coarse, P.ncoarse, P.u_cnt, P.w_cnt, P.u_ptr,
-                                         P.w_ptr, P.u_idx, P.w_idx, P.u_cap, P.w_cap, P.status, list_shifts(P));
-    KIFMM_CUDA_TRY(cudaMemsetAsync(P.wsrc_flag, 0, sizeof(int32_t) * nb, s));
+                                         P.w_ptr, P.u_idx, P.w_idx, P.u_cap, P.w_cap, P.status, list_shifts(P),
+                                         P.wsrc_flag, P.rb_dev->uw);
     if (P.w_cap > 0)
         ++g_launches, k_mark_w<<<grid_for(P.w_cap, 256), 256, 0, s>>>(P.w_cap, P.w_ptr + nb, P.w_idx, P.wsrc_flag);
     KIFMM_CUDA_TRY(cudaGetLastError());
