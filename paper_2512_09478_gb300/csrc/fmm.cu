@@ -280,19 +280,19 @@ __global__ void __launch_bounds__(1024, 1)
 }
 
 // ---------------------------------------------------------------------------
-// Gathered row products in FP64 (FP32: gemm_rows.cuh), out[t] (=|+=) Op
-// in[src(t)]: a block owns NTY RT rows of one class and 32 RC outputs; thread
-// (tx, ty) keeps rows RT ty .. RT ty + RT - 1 by outputs tx + 32 c.  Operators
-// are stored transposed ([k][n]); k advances in chunks of 16 through shared
+// Gathered row products of many rows in FP64 (FP32 and few rows:
+// gemm_rows.cuh), out[t] (=|+=) Op in[src(t)]: a block owns NTY RT rows of one
+// class and 32 RC outputs; thread (tx, ty) keeps rows RT ty .. RT ty + RT - 1
+// by outputs tx + 32 c.  Operators [k][ldp]; k advances in chunks of 16 through shared
 // memory with the next chunk prefetched into registers.  Bound by the FP64
 // unit (two lanes per clock and SM).
 // ---------------------------------------------------------------------------
 constexpr int kGK = 16;
 
-template <int NTY, int RT, int RC>
-__global__ void __launch_bounds__(32 * NTY) k_rows_f64(RowMap<double> g, const int32_t *__restrict__ targets,
-                                                       ClassRanges cr, int n, const double *__restrict__ in,
-                                                       double *out, int accumulate) {
+__global__ void __launch_bounds__(256) k_rows_f64(RowMap<double> g, const int32_t *__restrict__ targets,
+                                                  ClassRanges cr, int n, int ldp, const double *__restrict__ in,
+                                                  double *out, int accumulate) {
+    constexpr int NTY = 8, RT = 8, RC = 5;
     constexpr int TT = NTY * RT, TJ = 32 * RC, NT = 32 * NTY;
     __shared__ __align__(16) double Us[kGK][TT];
     __shared__ __align__(16) double Ms[kGK][TJ];
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(32 * NTY) k_rows_f64(RowMap<double> g, const i
         for (int r = 0; r < kRM; ++r) {
             const int e = threadIdx.x + NT * r;
             const int k = e / TJ, j = e - k * TJ;
-            rm[r] = (k < kGK && k0 + k < n && j0 + j < n) ? M[(size_t)(k0 + k) * n + j0 + j] : 0.0;
+            rm[r] = (k < kGK && k0 + k < n && j0 + j < n) ? M[(size_t)(k0 + k) * ldp + j0 + j] : 0.0;
         }
     };
     load(0);
@@ -905,20 +905,40 @@ __global__ void k_leaf_partition(int64_t n_leaves, const int32_t *__restrict__ l
     const bool valid = i < n_leaves;
     const int b = valid ? leaves[i] : -1;
     const int n = valid ? cnt[b] : 0;
-    int t0 = 0;
-    while (__any_sync(0xffffffffu, t0 < n)) {
-        const int v = (t0 < n) ? leaf_variant(tile, n - t0) : -1;
+    // places for all of a leaf's passes at once: leaves stay in order in every
+    // list (coarse leaves, with the longest source lists, first), where places
+    // taken pass by pass put a coarse leaf's last passes at the end
+    int mine[kLeafTiles];
 #pragma unroll
-        for (int u = 0; u < kLeafTiles; ++u) {
-            const unsigned m = __ballot_sync(0xffffffffu, v == u);
-            if (m == 0) continue;
-            const int leader = __ffs(m) - 1;
-            int base = 0;
-            if (lane == leader) base = atomicAdd(&counts[u], __popc(m));
-            base = __shfl_sync(0xffffffffu, base, leader);
-            if (v == u) lists[(int64_t)u * cap + base + __popc(m & ((1u << lane) - 1))] = make_int2(b, t0);
+    for (int u = 0; u < kLeafTiles; ++u) mine[u] = 0;
+    for (int t0 = 0; t0 < n;) {
+        const int v = leaf_variant(tile, n - t0);
+#pragma unroll
+        for (int u = 0; u < kLeafTiles; ++u) mine[u] += u == v ? 1 : 0;
+        t0 += (32 / leaf_tile_groups(v)) * leaf_tile_tpl(v);
+    }
+    __syncwarp();
+    int at[kLeafTiles];
+#pragma unroll
+    for (int u = 0; u < kLeafTiles; ++u) {
+        at[u] = 0;
+        if (!__any_sync(0xffffffffu, mine[u] > 0)) continue;
+        int incl = mine[u];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
         }
-        if (v >= 0) t0 += (32 / leaf_tile_groups(v)) * leaf_tile_tpl(v);
+        int base = 0;
+        if (lane == 31) base = atomicAdd(&counts[u], incl);
+        at[u] = __shfl_sync(0xffffffffu, base, 31) + incl - mine[u];
+    }
+    for (int t0 = 0; t0 < n;) {
+        const int v = leaf_variant(tile, n - t0);
+#pragma unroll
+        for (int u = 0; u < kLeafTiles; ++u)
+            if (u == v) lists[(int64_t)u * cap + at[u]++] = make_int2(b, t0);
+        t0 += (32 / leaf_tile_groups(v)) * leaf_tile_tpl(v);
     }
 }
 
@@ -1095,23 +1115,31 @@ inline int p2l_threads(const Plan &P) {
 template <typename T>
 inline size_t p2m_smem(const Plan &P) { return 7 * sizeof(T) * (size_t)p2m_threads(P); }
 
-// FP32 operator block of n inputs and ld outputs (padded), FP64 [n][n].
-template <typename T>
-inline int64_t op_block(int n, int ld) {
-    return sizeof(T) == 4 ? (int64_t)gemm_nkp(n) * gemm_ldp(ld) : (int64_t)n * n;
+constexpr int kRowsSmallMax = 200 * 1024;  // shared memory of a small tile (FP64: n_s up to 512)
+
+// Elements of an operator block of n inputs and ld outputs (padded).
+inline int64_t op_block(int n, int ld) { return (int64_t)gemm_nkp(n) * gemm_ldp(ld); }
+
+template <typename T, bool VEC>
+void rows_small_launch(const RowMap<T> &g, const int32_t *targets, const ClassRanges &cr, int64_t most, int ncls,
+                       bool few, int n, int ld, const T *in, T *out, int accumulate, double *dbar, cudaStream_t s) {
+    const int nkp = gemm_nkp(n), ldp = gemm_ldp(ld), rw = few ? 1 : 4;
+    const dim3 grid(grid_for(most, 4 * rw), ncls, grid_for(ld, kSmallCols));
+    const size_t smem = rows_small_smem<T>(nkp, rw);
+    if (few)
+        ++g_launches, k_rows_small<T, VEC, 1><<<grid, kRThreads, smem, s>>>(g, targets, cr, n, nkp, ldp, in, out,
+                                                                           accumulate, dbar);
+    else
+        ++g_launches, k_rows_small<T, VEC, 4><<<grid, kRThreads, smem, s>>>(g, targets, cr, n, nkp, ldp, in, out,
+                                                                           accumulate, dbar);
 }
 
 template <bool VEC>
 void rows_launch_f32(const RowMap<float> &g, const int32_t *targets, const ClassRanges &cr, int64_t most, int ncls,
-                     bool big, int n, int ld, const float *in, float *out, int accumulate, double *dbar,
+                     bool big, bool few, int n, int ld, const float *in, float *out, int accumulate, double *dbar,
                      cudaStream_t s) {
     const int nkp = gemm_nkp(n), ldp = gemm_ldp(ld), nc = gemm_nc(ld);
-    if (!big) {
-        const dim3 grid(grid_for(most, kSmallRows), ncls, grid_for(ld, kSmallCols));
-        ++g_launches, k_rows_small<VEC><<<grid, kRThreads, rows_small_smem(nkp), s>>>(g, targets, cr, n, nkp, ldp, in,
-                                                                                     out, accumulate, dbar);
-        return;
-    }
+    if (!big) return rows_small_launch<float, VEC>(g, targets, cr, most, ncls, few, n, ld, in, out, accumulate, dbar, s);
     const dim3 grid(grid_for(most, 64), ncls, ldp / (32 * nc));
     switch (nc) {
         case 1: ++g_launches, k_rows_big<1, VEC><<<grid, kRThreads, 0, s>>>(g, targets, cr, n, nkp, ldp, in, out, accumulate, dbar); break;
@@ -1139,18 +1167,21 @@ void rows(Plan &P, const RowMap<T> &g, const int32_t *targets, const int64_t *st
     if (most <= 0) return;
     const int n = P.ns;
     if (ld == 0) ld = n;
+    // blocks of 16 rows by 32 outputs
+    const int64_t small_blocks = (int64_t)grid_for(total, 16) * grid_for(ld, kSmallCols);
+    const bool few = small_blocks < (sizeof(T) == 4 ? 1 : 4) * (int64_t)P.num_sms;
     if constexpr (sizeof(T) == 4) {
         const bool big = (int64_t)grid_for(total, 64) * (gemm_ldp(ld) / (32 * gemm_nc(ld))) >= P.num_sms;
         if (n % 4 == 0)
-            rows_launch_f32<true>(g, targets, cr, most, ncls, big, n, ld, in, out, accumulate, dbar, s);
+            rows_launch_f32<true>(g, targets, cr, most, ncls, big, few, n, ld, in, out, accumulate, dbar, s);
         else
-            rows_launch_f32<false>(g, targets, cr, most, ncls, big, n, ld, in, out, accumulate, dbar, s);
-    } else if ((int64_t)grid_for(total, 64) * grid_for(n, 160) >= 2 * P.num_sms) {
+            rows_launch_f32<false>(g, targets, cr, most, ncls, big, few, n, ld, in, out, accumulate, dbar, s);
+    } else if ((int64_t)grid_for(total, 64) * grid_for(n, 160) >= 2 * P.num_sms ||
+               rows_small_smem<double>(gemm_nkp(n)) > (size_t)kRowsSmallMax) {
         const dim3 grid(grid_for(most, 64), ncls, grid_for(n, 160));
-        ++g_launches, k_rows_f64<8, 8, 5><<<grid, 256, 0, s>>>(g, targets, cr, n, in, out, accumulate);
+        ++g_launches, k_rows_f64<<<grid, 256, 0, s>>>(g, targets, cr, n, gemm_ldp(n), in, out, accumulate);
     } else {
-        const dim3 grid(grid_for(most, 16), ncls, grid_for(n, 32));
-        ++g_launches, k_rows_f64<4, 4, 1><<<grid, 128, 0, s>>>(g, targets, cr, n, in, out, accumulate);
+        rows_small_launch<double, true>(g, targets, cr, most, ncls, few, n, n, in, out, accumulate, nullptr, s);
     }
 }
 
@@ -1166,7 +1197,7 @@ void rows_one(Plan &P, const T *op, const int32_t *targets, int64_t a, int64_t e
 // boxes b of level l that have children; prod: scratch rows.
 template <typename T>
 void rows_children(Plan &P, int l, const T *ops, const T *in, T *prod, T *out, int accumulate, cudaStream_t s) {
-    rows<T>(P, RowMap<T>{nullptr, ops, op_block<T>(P.ns, P.ns), true}, P.part_list[3],
+    rows<T>(P, RowMap<T>{nullptr, ops, op_block(P.ns, P.ns), true}, P.part_list[3],
             P.part_start[3].data() + 8 * (l + 1), 8, in, prod, 0, s);
     const int64_t a = P.part_start[1][1 + l], np = P.part_start[1][2 + l] - a;
     if (np > 0)
@@ -1178,7 +1209,7 @@ void rows_children(Plan &P, int l, const T *ops, const T *in, T *prod, T *out, i
 template <typename T>
 void rows_parent(Plan &P, int l, const T *ops, const T *in, T *out, cudaStream_t s, int ld = 0,
                  double *dbar = nullptr) {
-    rows<T>(P, RowMap<T>{P.parent, ops, op_block<T>(P.ns, ld ? ld : P.ns), true}, P.part_list[3],
+    rows<T>(P, RowMap<T>{P.parent, ops, op_block(P.ns, ld ? ld : P.ns), true}, P.part_list[3],
             P.part_start[3].data() + 8 * l, 8, in, out, 1, s, ld, dbar);
 }
 
@@ -2009,7 +2040,7 @@ cudaError_t backward_t(Plan &P, const void *w_user, const void *g_user, const do
                        void *dq, void *dx, cudaStream_t s) {
     using V4 = typename Vec4<T>::type;
     const int ns = P.ns;
-    const int64_t blk = op_block<T>(ns, ns);
+    const int64_t blk = op_block(ns, ns);
     const T *surf = P.f64 ? (const T *)P.surf64 : (const T *)P.surf32;
     T *ub = (T *)P.u_chk, *db = (T *)P.d_chk, *tmp = (T *)P.tmp_chk;
     // scratch of their own: the forward's equivalent densities stay intact
@@ -2084,9 +2115,14 @@ cudaError_t backward_t(Plan &P, const void *w_user, const void *g_user, const do
 
 cudaError_t rows_setup() {
     const auto dyn = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    const int most = (int)rows_small_smem(gemm_nkp(3 * (6 * 7 * 7 + 2)));  // the longest rows: Stokeslet, p = 8
-    KIFMM_CUDA_TRY(cudaFuncSetAttribute(k_rows_small<true>, dyn, most));
-    return cudaFuncSetAttribute(k_rows_small<false>, dyn, most);
+    // the longest rows: FP32 the Stokeslet's at p = 8; FP64 those whose tile fits
+    const int f32 = (int)rows_small_smem<float>(gemm_nkp(3 * (6 * 7 * 7 + 2)));
+    KIFMM_CUDA_TRY(cudaFuncSetAttribute(k_rows_small<double, true, 4>, dyn, kRowsSmallMax));
+    KIFMM_CUDA_TRY(cudaFuncSetAttribute(k_rows_small<double, true, 1>, dyn, kRowsSmallMax));
+    KIFMM_CUDA_TRY(cudaFuncSetAttribute(k_rows_small<float, true, 4>, dyn, f32));
+    KIFMM_CUDA_TRY(cudaFuncSetAttribute(k_rows_small<float, true, 1>, dyn, f32));
+    KIFMM_CUDA_TRY(cudaFuncSetAttribute(k_rows_small<float, false, 4>, dyn, f32));
+    return cudaFuncSetAttribute(k_rows_small<float, false, 1>, dyn, f32);
 }
 
 cudaError_t run_backward(Plan &P, const void *w, const void *g, const double *dLdU, const void *grad, void *dq,

@@ -1,4 +1,4 @@
-// Gathered row products in FP32: out[t] (=|+=) Op in[src(t)], one operator per
+// Gathered row products: out[t] (=|+=) Op in[src(t)], one operator per
 // class of rows (M2M over the children's octants, L2L, the factors of the leaf
 // pseudo-inverses and their adjoints), one FMA per product in input order.
 //
@@ -6,13 +6,13 @@
 // multiple of 16 and the outputs to a multiple of the kernels' column block
 // (gemm_ldp), so that they come by 16-byte asynchronous copies without bounds
 // tests.  Two tiles:
-//  k_rows_big    64 rows by 32 NC outputs per 128 threads, a thread 8 rows by
+//  k_rows_big    (FP32; k_rows_f64 in fmm.cu) 64 rows by 32 NC outputs per 128 threads, a thread 8 rows by
 //                NC pairs of outputs on packed f32x2 FMAs.  FMA-bound: with
 //                operands from shared memory the loop alone reaches 95 FMA
 //                lanes per clock and SM (the inputs unduplicated, their pairs
 //                formed in registers: 95 against 86), a scalar three-operand
 //                FMA 82.
-//  k_rows_small  16 rows by 32 outputs, the whole input staged by four groups
+//  k_rows_small  (FP32 and FP64) 16 or 4 rows by 32 outputs, the whole input staged by four groups
 //                of asynchronous copies at once: a coarse level's time is the
 //                latency of its loads, which the big tile's chunks (and the
 //                16-input chunks of its predecessor) take one after the other.
@@ -55,10 +55,11 @@ __device__ __forceinline__ void row_cp_wait_all() { asm volatile("cp.async.wait_
 
 // With dbar: output column n (the operators' mean row) goes to dbar[t] (FP64,
 // plus the map's mean_base) instead of out.
-__device__ __forceinline__ void row_store(float v, int t, int j, int n, float *out, int accumulate, double *dbar,
-                                          const RowMap<float> &g) {
+template <typename T>
+__device__ __forceinline__ void row_store(T v, int t, int j, int n, T *out, int accumulate, double *dbar,
+                                          const RowMap<T> &g) {
     if (j < n) {
-        float *o = out + (size_t)t * n + j;
+        T *o = out + (size_t)t * n + j;
         *o = accumulate ? *o + v : v;
     } else if (j == n && dbar) {
         dbar[t] = (accumulate ? dbar[t] : 0.0) + (double)v + g.mean_base(t, dbar);
@@ -160,77 +161,91 @@ __global__ void __launch_bounds__(kRThreads, 3)
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
             const int j = j0 + 2 * tx + 32 * c;
-            row_store(acc[a][c].x, t, j, n, out, accumulate, dbar, g);
-            row_store(acc[a][c].y, t, j + 1, n, out, accumulate, dbar, g);
+            row_store<float>(acc[a][c].x, t, j, n, out, accumulate, dbar, g);
+            row_store<float>(acc[a][c].y, t, j + 1, n, out, accumulate, dbar, g);
         }
     }
 }
 
-// 16 rows by 32 outputs: warp w rows 4 w .. 4 w + 3, a lane per output.
-constexpr int kSmallRows = 16, kSmallCols = 32;
-inline size_t rows_small_smem(int nkp) {
-    return sizeof(float) * ((size_t)nkp * kSmallCols + (size_t)kSmallRows * (nkp + 4));
+// 4 RW rows by 32 outputs: warp w rows RW w .. RW w + RW - 1, a lane per
+// output.  RW = 4, or 1 for levels of so few rows that their blocks leave SMs
+// idle (a tile's sums take 2 us in FP32, 7 on one SM's FP64 lanes at n_s = 56).
+// VEC: the input rows are 16-byte aligned (FP32: n a multiple of 4; FP64: n
+// even, as every n_s is).
+constexpr int kSmallCols = 32;
+template <typename T>
+inline size_t rows_small_smem(int nkp, int rw = 4) {
+    return sizeof(T) * ((size_t)nkp * kSmallCols + (size_t)(4 * rw) * (nkp + 4));
 }
-template <bool VEC>
+template <typename T, bool VEC, int RW>
 __global__ void __launch_bounds__(kRThreads)
-    k_rows_small(RowMap<float> g, const int32_t *__restrict__ targets, ClassRanges cr, int n, int nkp, int ldp,
-                 const float *__restrict__ in, float *out, int accumulate, double *dbar) {
+    k_rows_small(RowMap<T> g, const int32_t *__restrict__ targets, ClassRanges cr, int n, int nkp, int ldp,
+                 const T *__restrict__ in, T *out, int accumulate, double *dbar) {
+    constexpr int kV = 16 / sizeof(T);                   // values per 16-byte copy
+    constexpr int kRows = 4 * RW, kPer = kRThreads / kRows;  // rows, staging threads per row
     extern __shared__ __align__(16) unsigned char rows_sm[];
-    float *Ms = reinterpret_cast<float *>(rows_sm);      // [nkp][32]
+    T *Ms = reinterpret_cast<T *>(rows_sm);              // [nkp][32]
     const int ldu = nkp + 4;                             // rows on other banks, 16-byte aligned
-    float *Us = Ms + (size_t)nkp * kSmallCols;           // [16][ldu]
+    T *Us = Ms + (size_t)nkp * kSmallCols;               // [kRows][ldu]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int cls = blockIdx.y, j0 = blockIdx.z * kSmallCols;
     int64_t t_begin = 0, t_end = 0;
 #pragma unroll
     for (int c = 0; c < 8; ++c)
         if (c == cls) t_begin = cr.b[c], t_end = cr.b[c + 1];
-    const int64_t t0 = t_begin + (int64_t)blockIdx.x * kSmallRows;
+    const int64_t t0 = t_begin + (int64_t)blockIdx.x * kRows;
     if (t0 >= t_end) return;  // uniform for the block
-    const float *M = g.op(cls) + j0;
-    // rows: thread t stages row t / 8, quads t % 8, t % 8 + 8, ...
-    const int64_t tr = t0 + tid / 8;
+    const T *M = g.op(cls) + j0;
+    // rows: thread t stages row t / kPer, 16-byte pieces t % kPer, + kPer, ...
+    const int64_t tr = t0 + tid / kPer;
     const int row = tr < t_end ? g.src(targets[tr]) : -1;
-    const float *src = in + (size_t)(row >= 0 ? row : 0) * n;
-    float *du = Us + (tid / 8) * ldu;
+    const T *src = in + (size_t)(row >= 0 ? row : 0) * n;
+    T *du = Us + (tid / kPer) * ldu;
     const int step = (nkp / 4 + 15) / 16 * 16;           // inputs per group of copies (four groups)
     for (int q = 0; q < 4; ++q) {
         const int k0 = min(nkp, q * step), k1 = min(nkp, k0 + step);
-        for (int e = tid; e < (k1 - k0) * (kSmallCols / 4); e += kRThreads) {
-            const int k = k0 + e / (kSmallCols / 4), c = 4 * (e % (kSmallCols / 4));
+        constexpr int kPieces = kSmallCols / kV;
+        for (int e = tid; e < (k1 - k0) * kPieces; e += kRThreads) {
+            const int k = k0 + e / kPieces, c = kV * (e % kPieces);
             row_cp16(Ms + (size_t)k * kSmallCols + c, M + (size_t)k * ldp + c);
         }
-        for (int k = k0 + 4 * (tid % 8); k < k1; k += 32) {
-            if (VEC) {
-                if (row >= 0 && k < n) row_cp16(du + k, src + k);
-                else *reinterpret_cast<float4 *>(du + k) = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int k = k0 + kV * (tid % kPer); k < k1; k += kPer * kV) {
+            if (VEC && row >= 0 && k < n) {
+                row_cp16(du + k, src + k);
             } else {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) du[k + i] = (row >= 0 && k + i < n) ? src[k + i] : 0.f;
+                for (int i = 0; i < kV; ++i) du[k + i] = (!VEC && row >= 0 && k + i < n) ? src[k + i] : T(0);
             }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    const float *u0 = Us + 4 * warp * ldu, *m0 = Ms + lane;
+    T acc[RW];
+#pragma unroll
+    for (int a = 0; a < RW; ++a) acc[a] = T(0);
+    const T *u0 = Us + RW * warp * ldu, *m0 = Ms + lane;
     auto sum = [&](int q) {
         __syncthreads();
         const int k0 = min(nkp, q * step), k1 = min(nkp, k0 + step);
 #pragma unroll 2
         for (int k = k0; k < k1; k += 4) {
-            float4 u[4];
+            T u[RW][4], m[4];
 #pragma unroll
-            for (int a = 0; a < 4; ++a) u[a] = *reinterpret_cast<const float4 *>(u0 + a * ldu + k);
-            float m[4];
+            for (int a = 0; a < RW; ++a) {
+                if constexpr (sizeof(T) == 4) {
+                    const float4 w = *reinterpret_cast<const float4 *>(u0 + a * ldu + k);
+                    u[a][0] = w.x, u[a][1] = w.y, u[a][2] = w.z, u[a][3] = w.w;
+                } else {
+                    const double2 w = *reinterpret_cast<const double2 *>(u0 + a * ldu + k);
+                    const double2 x = *reinterpret_cast<const double2 *>(u0 + a * ldu + k + 2);
+                    u[a][0] = w.x, u[a][1] = w.y, u[a][2] = x.x, u[a][3] = x.y;
+                }
+            }
 #pragma unroll
             for (int i = 0; i < 4; ++i) m[i] = m0[(k + i) * kSmallCols];
 #pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                acc[a] = fmaf(u[a].x, m[0], acc[a]);
-                acc[a] = fmaf(u[a].y, m[1], acc[a]);
-                acc[a] = fmaf(u[a].z, m[2], acc[a]);
-                acc[a] = fmaf(u[a].w, m[3], acc[a]);
-            }
+            for (int a = 0; a < RW; ++a)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[a] = fma(u[a][i], m[i], acc[a]);
         }
     };
     asm volatile("cp.async.wait_group 3;" ::: "memory");
@@ -242,9 +257,9 @@ __global__ void __launch_bounds__(kRThreads)
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     sum(3);
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const int64_t ti = t0 + 4 * warp + a;
-        if (ti < t_end) row_store(acc[a], targets[ti], j0 + lane, n, out, accumulate, dbar, g);
+    for (int a = 0; a < RW; ++a) {
+        const int64_t ti = t0 + RW * warp + a;
+        if (ti < t_end) row_store<T>(acc[a], targets[ti], j0 + lane, n, out, accumulate, dbar, g);
     }
 }
 

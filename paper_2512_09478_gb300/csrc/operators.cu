@@ -141,13 +141,14 @@ __global__ void k_to_f32(const double *in, float *out, size_t n) {
 }
 
 // [blocks][n][ld] operators to [blocks][nkp][ldp], zero padded.
-__global__ void k_pad_blocks(int64_t total, int n, int ld, int nkp, int ldp, const float *__restrict__ in,
-                             float *__restrict__ out) {
+template <typename T>
+__global__ void k_pad_blocks(int64_t total, int n, int ld, int nkp, int ldp, const T *__restrict__ in,
+                             T *__restrict__ out) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= total) return;
     const int64_t row = i / ldp;
     const int j = (int)(i - row * ldp), k = (int)(row % nkp);
-    out[i] = (k < n && j < ld) ? in[((row / nkp) * n + k) * ld + j] : 0.f;
+    out[i] = (k < n && j < ld) ? in[((row / nkp) * n + k) * ld + j] : T(0);
 }
 
 // W_t[j][m] = sinv[m] * Ut[m][j]
@@ -639,7 +640,7 @@ cudaError_t build_operators(Plan &P, std::string &err) {
         cudaFree(dKfV);
         cudaFree(dF);
     }
-    if (!P.f64) {
+    {
         // the row products' padded form (gemm_rows.cuh)
         struct Op { void **ptr; int blocks, ld; };
         const Op ops[] = {{&P.m2m_t, 8, n},   {&P.l2l_t, 8, P.op_ld}, {&P.up_w_t, 1, n},  {&P.up_v_t, 1, n},
@@ -649,9 +650,14 @@ cudaError_t build_operators(Plan &P, std::string &err) {
             if (!*o.ptr) continue;
             const int64_t total = (int64_t)o.blocks * gemm_nkp(n) * gemm_ldp(o.ld);
             void *padded = nullptr;
-            KIFMM_CUDA_TRY(plan_alloc(P, &padded, sizeof(float) * total));
-            k_pad_blocks<<<(unsigned)((total + 255) / 256), 256>>>(total, n, o.ld, gemm_nkp(n), gemm_ldp(o.ld),
-                                                                  (const float *)*o.ptr, (float *)padded);
+            KIFMM_CUDA_TRY(plan_alloc(P, &padded, esz * total));
+            const unsigned nblk_pad = (unsigned)((total + 255) / 256);
+            if (P.f64)
+                k_pad_blocks<double><<<nblk_pad, 256>>>(total, n, o.ld, gemm_nkp(n), gemm_ldp(o.ld),
+                                                        (const double *)*o.ptr, (double *)padded);
+            else
+                k_pad_blocks<float><<<nblk_pad, 256>>>(total, n, o.ld, gemm_nkp(n), gemm_ldp(o.ld),
+                                                       (const float *)*o.ptr, (float *)padded);
             KIFMM_CUDA_TRY(cudaDeviceSynchronize());
             plan_free(P, o.ptr);
             *o.ptr = padded;
