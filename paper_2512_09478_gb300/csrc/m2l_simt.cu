@@ -243,22 +243,30 @@ cudaError_t m2l_simt_setup(Plan &P) {
     return cudaFuncSetAttribute(k_m2l_simt<8, false>, dyn, (int)sizeof(SimtSmem<8>));
 }
 
-// 64 targets per block while that gives one and a half blocks per SM, else 32
-// or 16: smaller tiles read shared memory more per FMA but fill the GPU.
+// 64, 32 or 16 targets per block, whichever is estimated to finish first: the
+// fullest SM's blocks times their targets, over the FMA rate of the tile (95,
+// 82 and 60 lanes per clock and SM: smaller tiles read shared memory more per
+// FMA, but share out more evenly; 4672 targets of n = 456 are 240 blocks of 64
+// on 152 SMs, or three of 32 on each).
 cudaError_t m2l_simt(Plan &P, const float *u, float *d, double *dbar, cudaStream_t s) {
     int64_t most = 0;
     int64_t blocks[3] = {0, 0, 0};
     for (int c = 0; c < 8; ++c) {
         const int64_t t = P.m2l_class_start[c + 1] - P.m2l_class_start[c];
         most = std::max(most, t);
-        blocks[0] += (t + 63) / 64;
-        blocks[1] += (t + 31) / 32;
+        for (int k = 0; k < 3; ++k) blocks[k] += (t + (64 >> k) - 1) / (64 >> k);
     }
     if (most == 0) return cudaSuccess;  // no V-list targets
-    const int64_t ncb = (P.op_ld + kSCols - 1) / kSCols, want = 3 * (int64_t)P.num_sms / 2;
-    if (blocks[0] * ncb >= want) return simt_launch<8>(P, most, u, d, dbar, s);
-    if (blocks[1] * ncb >= want) return simt_launch<4>(P, most, u, d, dbar, s);
-    return simt_launch<2>(P, most, u, d, dbar, s);
+    const int64_t ncb = (P.op_ld + kSCols - 1) / kSCols;
+    const double rate[3] = {95.0, 82.0, 60.0};
+    int pick = 0;
+    double least = 1e30;
+    for (int k = 0; k < 3; ++k) {
+        const double t = (double)((blocks[k] * ncb + P.num_sms - 1) / P.num_sms) * (64 >> k) / rate[k];
+        if (t < 0.97 * least) least = t, pick = k;
+    }
+    if (pick == 0) return simt_launch<8>(P, most, u, d, dbar, s);
+    return pick == 1 ? simt_launch<4>(P, most, u, d, dbar, s) : simt_launch<2>(P, most, u, d, dbar, s);
 }
 
 }  // namespace kifmm
