@@ -223,9 +223,9 @@ def roofline_for(stage, ms_per_call, work, precision, peaks):
             return {"bound": "tensor", "achieved": ach, "peak": bf16, "unit": "TFLOP/s", "frac": ach / bf16,
                     "traffic": None, "kernel": "k_m2l_tc",
                     "peak_source": f"{kind} bf16 burst (fp16 same rate); 3 split products, 1 counted"}
-        return {"bound": "alu", "achieved": ach, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": ach / FP32_PEAK_TFLOPS, "traffic": None, "kernel": "k_ggemm<GatherM2L>",
-                "peak_source": "152 SMs x 128 FP32 lanes x 2 x 2.07 GHz"}
+        return {"bound": "tensor", "achieved": ach, "peak": bf16, "unit": "TFLOP/s", "frac": ach / bf16,
+                "traffic": None, "kernel": "k_m2l_exact",
+                "peak_source": f"{kind} bf16 burst; {36 if precision == 'fp64' else 6} split products, 1 counted"}
     if stage == "p2p":
         flops = 20.0 * work["leaf_pairs"]
         ach = flops / (ms_per_call * 1e-3) / 1e12
@@ -748,8 +748,8 @@ def accuracy_of(ref, q, coef, pot, grad, force=None, torque=None):
 
 def compare_leg(args, w, prec, xt, qt, offsets, coef, n, value, stream, flush, clumps, cl, ref, q, m2l_eps=0.0,
                 p=None):
-    """The same step with another precision of the library (plain FP32 SIMT
-    M2L for the DEM workload, the FP64 path for gravity), or with the
+    """The same step with another precision of the library (plain FP32 for
+    the DEM workload, the FP64 path for gravity), or with the
     compressed M2L (m2l_eps > 0): its throughput, the speedup of the
     benchmarked configuration over it, and its accuracy."""
     import torch
