@@ -666,6 +666,10 @@ cudaError_t m2l_exact_setup(Plan &P, int dir, const void *ops, int ld) {
     return P.f64 ? ex_setup<double>(P, dir, (const double *)ops, ld) : ex_setup<float>(P, dir, (const float *)ops, ld);
 }
 
+static size_t ex_part_bytes(const Plan &P, const ExState &S, int dir, int z) {
+    return (P.f64 ? sizeof(double) : sizeof(float)) * z * (size_t)P.m2l_class_start[8] * S.ld[dir];
+}
+
 // After set_sources: room for the sliced expansions and the slot splits'
 // partial sums (the adjoint's and the forward's are never live at once).
 cudaError_t m2l_exact_prepare(Plan &P) {
@@ -682,7 +686,7 @@ cudaError_t m2l_exact_prepare(Plan &P) {
     for (int dir = 0; dir < 2; ++dir) {
         if (!S.ops[dir].bs) continue;
         const int z = m2l_slot_split((int64_t)m2l_tiles_128(P) * S.ncb[dir], P.num_sms);
-        if (z > 1) need = std::max(need, esz * z * (size_t)P.m2l_class_start[8] * S.ld[dir]);
+        if (z > 1) need = std::max(need, ex_part_bytes(P, S, dir, z));
     }
     return m2l_part_reserve(P, need);
 }
@@ -719,7 +723,8 @@ static cudaError_t ex_run(Plan &P, int dir, const T *u, T *d, int accumulate, do
     a.accumulate = accumulate;
     a.wait_polls = P.m2l_wait_polls > 0 ? P.m2l_wait_polls : kWaitIters;
     a.status = P.status;
-    const int z = m2l_slot_split((int64_t)ntiles * S.ncb[dir], P.num_sms);
+    int z = m2l_slot_split((int64_t)ntiles * S.ncb[dir], P.num_sms);
+    if (ex_part_bytes(P, S, dir, z) > P.m2l_part_bytes) z = 1;  // no room for the partial sums
     a.part = z > 1 ? (T *)P.m2l_part : nullptr;
     const size_t smem = (size_t)a.nstages * SL::kSlices * (kTcRows + a.nt) * kRowB + 1024;
     ++g_launches, k_m2l_exact<T><<<dim3((unsigned)ntiles, (unsigned)S.ncb[dir], (unsigned)z), ex_threads<T>(),

@@ -625,9 +625,13 @@ const int4 *m2l_tiles_dev(const Plan &P) { return ((const M2lTiles *)P.m2l_tiles
 cudaError_t m2l_part_reserve(Plan &P, size_t bytes) {
     if (bytes <= P.m2l_part_bytes) return cudaSuccess;
     P.m2l_part_bytes = 0;
-    KIFMM_CUDA_TRY(plan_alloc(P, &P.m2l_part, bytes));
-    P.m2l_part_bytes = bytes;
-    return cudaSuccess;
+    const cudaError_t e = plan_alloc(P, &P.m2l_part, bytes);
+    if (e == cudaErrorMemoryAllocation) {  // run unsplit, which needs none
+        cudaGetLastError();
+        return cudaSuccess;
+    }
+    if (e == cudaSuccess) P.m2l_part_bytes = bytes;
+    return e;
 }
 
 static TcState &tc_state(Plan &P) {
@@ -775,7 +779,9 @@ static void tc_shape(int n1, int n2, int ncb, int np, int kblocks, int num_sms, 
             }
         }
 }
-// Room for the split expansions and the slot splits' partial sums.
+static size_t tc_part_bytes(int n1, int np) { return sizeof(float) * kVSlots * (size_t)n1 * kTcRows * np; }
+
+// Room for the split expansions and the slot splits' partial products.
 cudaError_t m2l_tensor_prepare(Plan &P) {
     TcState &S = tc_state(P);
     if (P.nb > S.u_cap) {
@@ -786,7 +792,7 @@ cudaError_t m2l_tensor_prepare(Plan &P) {
     const M2lTiles &TS = tile_state(P);
     int z, tl;
     tc_shape(TS.n_tiles[0], TS.n_tiles[1], S.ncb, S.np, S.kp / kKBlock, P.num_sms, &z, &tl);
-    return m2l_part_reserve(P, z > 1 ? sizeof(float) * kVSlots * (size_t)TS.n_tiles[0] * kTcRows * S.np : 0);
+    return m2l_part_reserve(P, z > 1 ? tc_part_bytes(TS.n_tiles[0], S.np) : 0);
 }
 
 cudaError_t m2l_tensor(Plan &P, cudaStream_t s) {
@@ -827,6 +833,7 @@ cudaError_t m2l_tensor(Plan &P, cudaStream_t s) {
     int z, tl_default;
     tc_shape(TS.n_tiles[0], TS.n_tiles[1], S.ncb, S.np, S.kp / kKBlock, P.num_sms, &z,
              &tl_default);
+    if (tc_part_bytes(TS.n_tiles[0], S.np) > P.m2l_part_bytes) z = 1;  // no room for the partial products
     a.part = z > 1 ? (float *)P.m2l_part : nullptr;
     a.n_tiles = TS.n_tiles[0];
     auto launch_v = [&](auto pwc, auto tlc, auto spl, int nst) -> cudaError_t {
