@@ -61,7 +61,6 @@ namespace {
 constexpr int kKB = 32;             // 16-bit elements per stage row (64 bytes)
 constexpr int kRowB = 64;
 constexpr int kDrain = 8;           // drain warps
-constexpr long long kExDrainPolls = 1LL << 18;  // bound of the clean-up wait on the last bulk copy
 
 template <typename T>
 struct Slicing;
@@ -243,7 +242,7 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
     __shared__ uint32_t tmem_base_s;
     __shared__ int32_t tgt_s[kTcRows];
     __shared__ volatile int abort_s;
-    __shared__ volatile int abort_zero;  // never set: a wait on it runs to its bound
+    __shared__ int last_bulk_s;  // the last stage a bulk copy was issued for, -1: none
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int4 tile = a.tiles[blockIdx.x];
     const int cls = tile.x;
@@ -257,7 +256,7 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
     }
     if (threadIdx.x == 0) {
         abort_s = 0;
-        abort_zero = 0;
+        last_bulk_s = -1;
         for (int s = 0; s < NST; ++s) {
             mbar_init(smem_u32(&full_bar[s]), 32 * kProd + 1);  // producer cp.async arrivals + the bulk-copy leader
             mbar_init(smem_u32(&empty_bar[s]), 1);
@@ -298,7 +297,7 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
         }
         const bool leader = threadIdx.x == 0;
         int o_cur = 0, o_next = leader ? a.slot_off[cls * kVSlots + s_lo] : 0;
-        int it = 0, last_it = -1;
+        int it = 0;
         bool ok = true;
         for (int s = s_lo; s < s_hi && ok; ++s) {
 #pragma unroll
@@ -325,7 +324,7 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
                     const size_t boff = (((size_t)o_cur * kblocks + kb) * a.np + c_first) * (size_t)(NS * kKB);
                     mbar_arrive_expect_tx(fb, NS * b_slice);
                     bulk_g2s(sB, a.bs + boff, NS * b_slice, fb);
-                    last_it = it;
+                    last_bulk_s = it;
                 }
 #pragma unroll
                 for (int i = 0; i < kRows; ++i) {
@@ -340,10 +339,7 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
             }
         }
         cp_async_wait_all();
-        if (leader && abort_s && last_it >= 0) {
-            // the last bulk copy must land before the CTA's shared memory goes away
-            (void)mbar_wait(smem_u32(&full_bar[last_it % NST]), (last_it / NST) & 1, &abort_zero, kExDrainPolls);
-        }
+        wait_bulk_copies(full_bar, NST, 32 * kProd, it, &last_bulk_s, leader);
     } else if (warp == kProd) {
         // ---------------- MMA issuer ----------------
         // One accumulation per (slot, K chunk), in accumulator set w % nbuf.
@@ -541,11 +537,7 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
     tc_fence_before();
     __syncthreads();
     if (warp == kProd) {
-        if (abort_s) {
-            // bounded drain of in-flight MMAs (the done barrier completes when they do)
-            for (long long i = 0; i < kWaitIters; ++i)
-                if (mbar_try_wait(smem_u32(&done_bar), 0) || mbar_try_wait(smem_u32(&done_bar), 1)) break;
-        }
+        if (abort_s) wait_mmas(smem_u32(&done_bar));  // none may touch the memory given back below
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols) : "memory");
     }

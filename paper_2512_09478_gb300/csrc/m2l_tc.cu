@@ -49,11 +49,6 @@ namespace kifmm {
 namespace {
 
 constexpr int kDrainWarps = 8;
-// After a time-out the leader waits this many polls for its last bulk copy
-// to land before the block's shared memory goes away (microseconds are
-// enough; the barrier itself may never complete when other producers
-// stopped before arriving).
-constexpr long long kDrainPolls = 1LL << 18;
 constexpr int kAccBufs = 3;         // per-slot partial accumulators in TMEM
 constexpr int kKBlock = 32;         // FP16 elements per stage row (64 bytes)
 constexpr int kRowBytes = 64;
@@ -76,7 +71,7 @@ struct TileArgs {
     int n_tiles;              // tiles of 128
     int ns, kp, np, nstages;  // np: operator rows (output columns) incl. padding
     int ncb;                  // column blocks (np = ncb NT)
-    long long wait_polls;     // bound of the pipeline's barrier waits (the clean-up waits keep kWaitIters)
+    long long wait_polls;     // bound of the pipeline's barrier waits (the clean-up waits keep their own)
     int *status;
 };
 
@@ -106,7 +101,7 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
     __shared__ int32_t tgt_s[kRows];
 
     __shared__ volatile int abort_s;
-    __shared__ volatile int abort_zero;  // never set: a wait on it runs to its bound
+    __shared__ int last_bulk_s;  // the last stage a bulk copy was issued for, -1: none
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int4 tile = a.tiles[blockIdx.x];
@@ -120,7 +115,7 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
 
     if (threadIdx.x == 0) {
         abort_s = 0;
-        abort_zero = 0;
+        last_bulk_s = -1;
         for (int s = 0; s < NS; ++s) {
             mbar_init(smem_u32(&full_bar[s]), 32 * kProdWarps + 1);  // producer cp.async arrivals + the bulk-copy leader
             mbar_init(smem_u32(&empty_bar[s]), 1);
@@ -168,8 +163,9 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
             src_next[i] = (tg >= 0) ? a.vdense[(size_t)tg * kVSlots + s_lo] : -1;
         }
         const bool leader = threadIdx.x == 0;
-        int o_cur = 0, o_next = leader ? a.slot_off[cls * kVSlots + s_lo] : 0, last_it = -1;
-        for (int it = 0; it < iters; ++it) {
+        int o_cur = 0, o_next = leader ? a.slot_off[cls * kVSlots + s_lo] : 0;
+        int it = 0;
+        for (; it < iters; ++it) {
             const int stage = it % NS;
             const int s = s_lo + it / kblocks, kb = it - (s - s_lo) * kblocks;
             if (kb == 0) {
@@ -198,7 +194,7 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
                 const size_t boff = (((size_t)o_cur * kblocks + kb) * a.ncb + cb) * 2 * (size_t)NT * kKBlock;
                 mbar_arrive_expect_tx(fb, 2 * b_bytes);
                 bulk_g2s(sB, a.bhl + boff, 2 * b_bytes, fb);
-                last_it = it;
+                last_bulk_s = it;
             }
             const size_t koff = (size_t)kb * kKBlock + 8 * ch;
 #pragma unroll
@@ -214,12 +210,7 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
             cp_async_arrive_noinc(fb);
         }
         cp_async_wait_all();
-        if (leader && abort_s && last_it >= 0) {
-            // the last bulk copy must land before the CTA's shared memory
-            // goes away; the bounded wait outlasts it even when other
-            // producers stopped before arriving on that stage
-            (void)mbar_wait(smem_u32(&full_bar[last_it % NS]), (last_it / NS) & 1, &abort_zero, kDrainPolls);
-        }
+        wait_bulk_copies(full_bar, NS, 32 * kProdWarps, it, &last_bulk_s, leader);
     } else if (warp == kMmaWarp) {
         // ---------------- MMA issuer ----------------
         // Partial accumulator u = s ntl + t (slot s, tile t) goes to buffer
@@ -372,11 +363,7 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
     tc_fence_before();
     __syncthreads();
     if (warp == kMmaWarp) {
-        if (abort_s) {
-            // bounded drain of in-flight MMAs (the done barrier completes when they do)
-            for (long long i = 0; i < kWaitIters; ++i)
-                if (mbar_try_wait(smem_u32(&done_bar), 0) || mbar_try_wait(smem_u32(&done_bar), 1)) break;
-        }
+        if (abort_s) wait_mmas(smem_u32(&done_bar));  // none may touch the memory given back below
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols) : "memory");
     }

@@ -40,6 +40,18 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     return false;
 }
 
+// The clean-up waits: copies land and MMAs complete within
+// microseconds, so the bound is never reached unless the GPU itself stalls.
+constexpr int kCleanupPolls = 1 << 18;
+// Waits (bounded) for every MMA issued before the one commit on `done`.  A
+// fresh barrier completes its phase 0 once; a wait on parity 1 would return
+// at once, since the phase before the first counts as complete.
+__device__ __forceinline__ void wait_mmas(uint32_t done) {
+#pragma unroll 1
+    for (int i = 0; i < kCleanupPolls; ++i)
+        if (mbar_try_wait(done, 0)) return;
+}
+
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -65,6 +77,28 @@ __device__ __forceinline__ void cp_async_arrive_noinc(uint32_t bar) {
 }
 
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// The producer threads' end, time-out or not: the bulk copies of the last
+// n_stages stages up to *last (-1: none issued) must land before the CTA's
+// shared memory goes away.  `arrived`: the stages this thread arrived on; the
+// arrivals that a time-out made it stop short of are made up here, so that
+// every stage holding a bulk copy completes.  (The copy of stage k was issued
+// only after stage k - n_stages had been consumed, so no thread is more than
+// n_stages behind and each arrival lands in its own phase.)
+__device__ __forceinline__ void wait_bulk_copies(uint64_t *full, int n_stages, int threads, int arrived,
+                                                 const int *last_s, bool leader) {
+    __syncwarp();
+    asm volatile("barrier.cta.sync 1, %0;" ::"r"(threads) : "memory");  // the leader's *last is final
+    const int last = *last_s;
+#pragma unroll 1
+    for (int k = arrived; k <= last; ++k) mbar_arrive(smem_u32(&full[k % n_stages]));
+    if (!leader) return;
+#pragma unroll 1
+    for (int k = last >= n_stages ? last - n_stages + 1 : 0; k <= last; ++k)
+#pragma unroll 1
+        for (int i = 0; i < kCleanupPolls; ++i)
+            if (mbar_try_wait(smem_u32(&full[k % n_stages]), (uint32_t)(k / n_stages) & 1u)) break;
+}
 
 // Shared-memory matrix descriptor: K-major, 64-byte swizzle, rows of 64 bytes,
 // 8-row groups 512 bytes apart.
