@@ -235,7 +235,9 @@ kifmm_status kifmm_refresh_sources(kifmm_plan *plan, const void *xyz, const void
  * pot (device, [N] or NULL), grad (device, [N, 3] or NULL): outputs in the
  *   caller's particle order, coef applied, self-interaction excluded.
  * energy (device, [n_systems] doubles, or NULL): U_s = 1/2 sum_{i in s} q_i pot_i.
- * Enqueues work only; never allocates; never synchronises.
+ * Enqueues work only; never allocates; never synchronises.  A device wait that
+ * runs out shows in the device status (KIFMM_ERR_TIMEOUT) and as NaN in the
+ * outputs it affects.
  */
 kifmm_status kifmm_evaluate(kifmm_plan *plan, void *pot, void *grad, double *energy,
                             kifmm_stream_t stream);
@@ -423,11 +425,14 @@ kifmm_status kifmm_set_m2l_tuning(kifmm_plan *plan, int producers, int tiles, in
 /* Bound, in polls, of every barrier wait of the tensor-core M2L's pipeline
  * (0: the default, about 2^24).  Every wait of that kernel is bounded: on
  * time-out its blocks record KIFMM_ERR_TIMEOUT in the device status
- * (kifmm_get_device_status), wait for their own copies in flight (with the
- * default bound), free their tensor memory and return, so that the context
- * stays usable; that evaluate's outputs are then not valid.  A tiny bound
+ * (kifmm_get_device_status), wait for their own copies and products in flight
+ * (with a bound of its own), free their tensor memory and return, so that the context
+ * stays usable; the outputs of the particles below a box that timed out are
+ * NaN.  A backward's M2L (exact-split products on the tensor cores in every
+ * mode) is bounded in the same way and takes the same bound.  A tiny bound
  * makes the waits run out on purpose (the time-out path's test).
- * KIFMM_ERR_ARG for a negative bound or a plan without the tensor-core M2L.
+ * KIFMM_ERR_ARG for a negative bound and for FP64 and FP32 plans, whose M2L
+ * keeps the default bound (it ends in the same status and NaN outputs).
  * Host only; no device work. */
 kifmm_status kifmm_set_m2l_wait_bound(kifmm_plan *plan, int64_t polls);
 

@@ -513,7 +513,8 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
                 if (lane == 0) mbar_arrive(smem_u32(&accfree_bar[buf]));
             }
         }
-        if (ok && !abort_s && tb >= 0) {
+        if (tb >= 0) {  // (timed out: NaN, so that no caller takes the row for a result)
+            const bool valid = ok && !abort_s;
             T *out = a.part ? a.part + ((size_t)blockIdx.z * a.n_targets + tile.y + row) * a.ld
                             : a.d + (size_t)tb * a.ns;
 #pragma unroll
@@ -523,12 +524,13 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
                     const int jc = c_first + col + j;
+                    const T v = valid ? acc[g][j] : (T)NAN;
                     if (a.part) {
-                        if (jc < a.ld) out[jc] = acc[g][j];
+                        if (jc < a.ld) out[jc] = v;
                     } else if (jc < a.ns) {
-                        out[jc] = a.accumulate ? out[jc] + acc[g][j] : acc[g][j];
+                        out[jc] = a.accumulate ? out[jc] + v : v;
                     } else if (jc == a.ns && a.dbar) {
-                        a.dbar[tb] = (a.accumulate ? a.dbar[tb] : 0.0) + (double)acc[g][j];
+                        a.dbar[tb] = (a.accumulate ? a.dbar[tb] : 0.0) + (double)v;
                     }
                 }
             }

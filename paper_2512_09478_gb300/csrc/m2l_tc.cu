@@ -289,9 +289,11 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
             if (t < ntl) {
                 float *out = a.part + (((size_t)s_lo * a.n_tiles + tile.w + t) * a.np + cb * NT + c_base) * kTcRows +
                              q * 32 + lane;
+                float *const first = out;
+                bool ok = true;
                 for (int s = 0; s < s_hi - s_lo; ++s, out += (size_t)a.n_tiles * a.np * kTcRows) {
                     const int u = s * ntl + t, buf = u % kAccBufs;
-                    bool ok = mbar_wait(smem_u32(&accfull_bar[buf]), (u / kAccBufs) & 1, &abort_s, a.wait_polls);
+                    ok = mbar_wait(smem_u32(&accfull_bar[buf]), (u / kAccBufs) & 1, &abort_s, a.wait_polls);
                     ok = __all_sync(0xffffffffu, ok);  // warp-uniform: tcgen05.ld is .sync.aligned
                     if (!ok) {
                         set_status(a.status, KIFMM_ERR_TIMEOUT);
@@ -310,6 +312,8 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&accfree_bar[buf]));
                 }
+                if (!ok || abort_s)  // timed out: the sum over the slots carries the NaN on
+                    for (int c = 0; c < NT / 2; ++c) first[c * kTcRows] = NAN;
             }
         } else {
             float acc[NT / 2];
@@ -345,11 +349,10 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
                     if (lane == 0) mbar_arrive(smem_u32(&accfree_bar[buf]));
                 }
             }
-            ok = ok && !abort_s && t < ntl;
             const int row = t * kTcRows + q * 32 + lane;
             const int32_t tb = tgt_s[row];
-            if (ok && tb >= 0) {
-                const float scale = a.level_unscale[a.lvl[tb]];
+            if (tb >= 0) {  // (timed out: NaN, so that no caller takes the row for a result)
+                const float scale = ok && !abort_s ? a.level_unscale[a.lvl[tb]] : NAN;
                 const int col0 = cb * NT + c_base;
                 float *out = a.d + (size_t)tb * a.ns + col0;
 #pragma unroll

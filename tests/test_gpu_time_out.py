@@ -35,10 +35,12 @@ def test_forward_and_adjoint_time_out_and_recover(n):
     assert plan.device_status() == 0
     for _ in range(3):
         plan.set_m2l_wait_bound(1)
-        plan.evaluate()
+        pot1, grad1, _ = plan.evaluate()
         assert plan.device_status() == 5      # KIFMM_ERR_TIMEOUT
-        plan.backward(w, grad)
+        dq1, _ = plan.backward(w, grad)
         assert plan.device_status() == 5
+        # callers that read no status (autograd) see it in the outputs
+        assert torch.isnan(pot1).any() and torch.isnan(grad1).any() and torch.isnan(dq1).any()
         plan.set_m2l_wait_bound(0)
         pot2, grad2, _ = plan.evaluate()
         dq2, dx2 = plan.backward(w, grad2)
