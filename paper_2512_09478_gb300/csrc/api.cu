@@ -131,6 +131,22 @@ cudaError_t plan_grow(Plan &P, void **ptr, size_t bytes, size_t keep_bytes) {
     return cudaSuccess;
 }
 
+cudaError_t plan_replace(Plan &P, int64_t *cap, int64_t new_cap, const std::vector<BufSize> &bufs) {
+    *cap = 0;
+    for (const BufSize &b : bufs) KIFMM_CUDA_TRY(plan_alloc(P, b.ptr, b.bytes));
+    *cap = new_cap;
+    return cudaSuccess;
+}
+
+static cudaError_t words_reserve(Plan &P, uint32_t **buf, size_t *have, size_t elems) {
+    if (elems <= *have) return cudaSuccess;
+    KIFMM_CUDA_TRY(plan_grow(P, (void **)buf, sizeof(uint32_t) * elems, 0));
+    *have = elems;
+    return cudaSuccess;
+}
+cudaError_t scan_tmp_reserve(Plan &P, size_t elems) { return words_reserve(P, &P.scan_tmp, &P.scan_tmp_elems, elems); }
+cudaError_t hist_reserve(Plan &P, size_t elems) { return words_reserve(P, &P.hist, &P.hist_elems, elems); }
+
 // Per-node arrays used while the octree is built.
 cudaError_t grow_tree_arrays(Plan &P, int64_t cap, int64_t keep) {
     KIFMM_CUDA_TRY(cudaDeviceSynchronize());
@@ -139,12 +155,8 @@ cudaError_t grow_tree_arrays(Plan &P, int64_t cap, int64_t keep) {
         KIFMM_CUDA_TRY(plan_grow(P, (void **)a, sizeof(int32_t) * cap, sizeof(int32_t) * keep));
     KIFMM_CUDA_TRY(plan_grow(P, (void **)&P.tmp_nchild, sizeof(uint32_t) * 2 * cap, sizeof(uint32_t) * keep));
     KIFMM_CUDA_TRY(plan_grow(P, (void **)&P.child_rng, sizeof(int32_t) * 16 * cap, sizeof(int32_t) * 16 * keep));
+    KIFMM_CUDA_TRY(scan_tmp_reserve(P, scan_tmp_needed(2 * cap) + 8));
     P.box_cap = cap;
-    const size_t need = scan_tmp_needed(2 * cap) + 8;
-    if (need > P.scan_tmp_elems) {
-        P.scan_tmp_elems = need;
-        KIFMM_CUDA_TRY(plan_alloc(P, (void **)&P.scan_tmp, sizeof(uint32_t) * need));
-    }
     return cudaSuccess;
 }
 
@@ -153,8 +165,8 @@ static cudaError_t ensure_box_arrays(Plan &P) {
     if (P.nb <= P.list_cap) return cudaSuccess;
     const int64_t cap = P.nb + P.nb / 4 + 256;
     const size_t esz = P.f64 ? sizeof(double) : sizeof(float);
-    struct A { void **p; size_t bytes; };
-    const A arrs[] = {
+    P.prev_nb = -1;  // the lists kept for reuse go with the old arrays
+    std::vector<BufSize> arrs = {
         {(void **)&P.coll, sizeof(int32_t) * kColl * cap},
         {(void **)&P.coarse, sizeof(int32_t) * kMaxCoarse * cap},
         {(void **)&P.ncoarse, sizeof(int32_t) * cap},
@@ -186,14 +198,13 @@ static cudaError_t ensure_box_arrays(Plan &P) {
         {(void **)&P.leaf_vlist, sizeof(int2) * kLeafTiles * (cap + P.desc.n_max / 8 + 64)},
         {(void **)&P.leaf_vcnt, sizeof(int32_t) * 16},
     };
-    for (const A &a : arrs) KIFMM_CUDA_TRY(plan_alloc(P, a.p, a.bytes));
     if (P.periodic) {
-        KIFMM_CUDA_TRY(plan_alloc(P, (void **)&P.coll_sh, (size_t)kColl * cap));
-        KIFMM_CUDA_TRY(plan_alloc(P, (void **)&P.coarse_sh, (size_t)kMaxCoarse * cap));
-        KIFMM_CUDA_TRY(plan_alloc(P, (void **)&P.x_sh, (size_t)kMaxCoarse * cap));
-        KIFMM_CUDA_TRY(plan_alloc(P, (void **)&P.leaf_q2, sizeof(double) * cap));
+        arrs.push_back({(void **)&P.coll_sh, (size_t)kColl * cap});
+        arrs.push_back({(void **)&P.coarse_sh, (size_t)kMaxCoarse * cap});
+        arrs.push_back({(void **)&P.x_sh, (size_t)kMaxCoarse * cap});
+        arrs.push_back({(void **)&P.leaf_q2, sizeof(double) * cap});
     }
-    P.list_cap = cap;
+    KIFMM_CUDA_TRY(plan_replace(P, &P.list_cap, cap, arrs));
     P.leaf_item_cap = cap + P.desc.n_max / 8 + 64;
     return cudaSuccess;
 }
@@ -347,9 +358,7 @@ kifmm_status kifmm_plan_create(const kifmm_plan_desc *desc, kifmm_plan **out) {
             return fail(KIFMM_ERR_CUDA);
     const int64_t box0 = 12 * (n / (d.leaf_cap + 1)) + 64LL * P.sys_cap + 1024;
     if (grow_tree_arrays(P, box0, 0) != cudaSuccess) return fail(KIFMM_ERR_CUDA);
-    P.scan_tmp_elems = std::max(P.scan_tmp_elems, scan_tmp_needed((int64_t)256 * nblk) + 8);
-    if (plan_alloc(P, (void **)&P.scan_tmp, sizeof(uint32_t) * P.scan_tmp_elems) != cudaSuccess)
-        return fail(KIFMM_ERR_CUDA);
+    if (scan_tmp_reserve(P, scan_tmp_needed((int64_t)256 * nblk) + 8) != cudaSuccess) return fail(KIFMM_ERR_CUDA);
     P.status = &P.rb_dev->status;
     P.list_totals = P.rb_dev->vx;
     P.part_counts = &P.rb_dev->part_counts[0][0];
@@ -440,10 +449,10 @@ static kifmm_status set_sources_impl(Plan &P, const void *xyz, const void *q, cu
         }
         start[n_systems] = (int32_t)(ch.size() / 2);
         const int64_t nch = (int64_t)ch.size() / 2;
-        if (nch > P.n_energy_chunks) {
-            API_CUDA(plan_alloc(P, (void **)&P.energy_chunks, sizeof(int64_t) * 2 * nch));
-            API_CUDA(plan_alloc(P, (void **)&P.energy_partial, sizeof(double) * nch));
-        }
+        P.energy_off_h.clear();  // (until the new chunks are in place)
+        if (nch > P.energy_cap)
+            API_CUDA(plan_replace(P, &P.energy_cap, nch, {{(void **)&P.energy_chunks, sizeof(int64_t) * 2 * nch},
+                                                          {(void **)&P.energy_partial, sizeof(double) * nch}}));
         P.n_energy_chunks = nch;
         API_CUDA(cudaMemcpyAsync(P.energy_chunks, ch.data(), sizeof(int64_t) * ch.size(), cudaMemcpyHostToDevice, s));
         API_CUDA(cudaMemcpyAsync(P.energy_chunk_start, start.data(), sizeof(int32_t) * start.size(),

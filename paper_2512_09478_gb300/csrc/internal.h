@@ -243,7 +243,7 @@ struct Plan {
     int64_t *energy_chunks = nullptr;     // [n_chunks][2] (begin, end)
     int32_t *energy_chunk_start = nullptr; // [S+1]
     double *energy_partial = nullptr;     // [n_chunks]
-    int64_t n_energy_chunks = 0;
+    int64_t n_energy_chunks = 0, energy_cap = 0;
 
     // ---- profiling ----
     bool prof = false;
@@ -268,9 +268,21 @@ struct Plan {
 
 // allocation helpers (tracked, freed with the plan).  plan_alloc replaces
 // *ptr (freeing a previous tracked buffer); plan_grow keeps the first
-// keep_bytes of the old contents.
+// keep_bytes of the old contents (and the whole buffer when the new one
+// cannot be had).  A buffer's capacity is recorded only once the buffer exists:
+// plan_replace, for buffers too large to hold twice, sets *cap to 0 before it
+// frees the old ones and to new_cap when it has all of the new, so that a
+// failed allocation leaves a plan that asks for the buffers again.
 cudaError_t plan_alloc(Plan &P, void **ptr, size_t bytes);
 cudaError_t plan_grow(Plan &P, void **ptr, size_t bytes, size_t keep_bytes);
+struct BufSize {
+    void **ptr;
+    size_t bytes;
+};
+cudaError_t plan_replace(Plan &P, int64_t *cap, int64_t new_cap, const std::vector<BufSize> &bufs);
+// scratch of at least `elems` words (contents lost)
+cudaError_t scan_tmp_reserve(Plan &P, size_t elems);
+cudaError_t hist_reserve(Plan &P, size_t elems);
 void plan_free(Plan &P, void **ptr);
 cudaError_t grow_tree_arrays(Plan &P, int64_t new_cap, int64_t keep);
 

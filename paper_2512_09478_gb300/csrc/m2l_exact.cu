@@ -672,9 +672,10 @@ cudaError_t m2l_exact_prepare(Plan &P) {
     const size_t esz = P.f64 ? sizeof(double) : sizeof(float);
     const int NS = P.f64 ? Slicing<double>::kSlices : Slicing<float>::kSlices;
     if (P.nb > S.u_cap) {
-        S.u_cap = P.list_cap;
-        KIFMM_CUDA_TRY(plan_alloc(P, (void **)&S.us, sizeof(uint16_t) * S.u_cap * S.kblocks * NS * kKB));
-        KIFMM_CUDA_TRY(plan_alloc(P, &S.rscale, esz * S.u_cap));
+        const int64_t cap = P.list_cap;
+        KIFMM_CUDA_TRY(plan_replace(P, &S.u_cap, cap,
+                                    {{(void **)&S.us, sizeof(uint16_t) * cap * S.kblocks * NS * kKB},
+                                     {&S.rscale, esz * cap}}));
     }
     size_t need = 0;
     for (int dir = 0; dir < 2; ++dir) {

@@ -717,8 +717,8 @@ cudaError_t m2l_tiles_build(Plan &P, cudaStream_t s) {
         S.n_tiles[t - 1] = (int)S.tiles_h.size() - (t == 2 ? S.n_tiles[0] : 0);
     }
     if ((int64_t)S.tiles_h.size() > S.tiles_cap) {
-        S.tiles_cap = (int64_t)S.tiles_h.size() + 64;
-        KIFMM_CUDA_TRY(plan_alloc(P, (void **)&S.tiles, sizeof(int4) * S.tiles_cap));
+        const int64_t cap = (int64_t)S.tiles_h.size() + 64;
+        KIFMM_CUDA_TRY(plan_replace(P, &S.tiles_cap, cap, {{(void **)&S.tiles, sizeof(int4) * cap}}));
     }
     // the staging buffer may still feed the previous upload (set_sources on
     // another stream)
@@ -775,9 +775,9 @@ static size_t tc_part_bytes(int n1, int np) { return sizeof(float) * kVSlots * (
 cudaError_t m2l_tensor_prepare(Plan &P) {
     TcState &S = tc_state(P);
     if (P.nb > S.u_cap) {
-        S.u_cap = P.list_cap;
-        KIFMM_CUDA_TRY(plan_alloc(P, (void **)&S.uh, sizeof(__half) * S.u_cap * S.kp));
-        KIFMM_CUDA_TRY(plan_alloc(P, (void **)&S.ul, sizeof(__half) * S.u_cap * S.kp));
+        const int64_t cap = P.list_cap;
+        KIFMM_CUDA_TRY(plan_replace(P, &S.u_cap, cap, {{(void **)&S.uh, sizeof(__half) * cap * S.kp},
+                                                       {(void **)&S.ul, sizeof(__half) * cap * S.kp}}));
     }
     const M2lTiles &TS = tile_state(P);
     int z, tl;

@@ -1354,14 +1354,8 @@ __global__ void k_child8(int64_t nb, const int32_t *__restrict__ child_first, co
 static cudaError_t radix_pass(Plan &P, const uint64_t *kin, const uint32_t *vin, uint64_t *kout, uint32_t *vout,
                               int64_t n, int mode, int shift, cudaStream_t s) {
     const int nblk = (int)((n + kTile - 1) / kTile);
-    if ((size_t)512 * nblk > P.hist_elems) {
-        P.hist_elems = (size_t)512 * nblk;
-        KIFMM_CUDA_TRY(plan_alloc(P, (void **)&P.hist, sizeof(uint32_t) * P.hist_elems));
-    }
-    if (scan_tmp_needed((int64_t)256 * nblk) + 8 > P.scan_tmp_elems) {
-        P.scan_tmp_elems = scan_tmp_needed((int64_t)256 * nblk) + 8;
-        KIFMM_CUDA_TRY(plan_alloc(P, (void **)&P.scan_tmp, sizeof(uint32_t) * P.scan_tmp_elems));
-    }
+    KIFMM_CUDA_TRY(hist_reserve(P, (size_t)512 * nblk));
+    KIFMM_CUDA_TRY(scan_tmp_reserve(P, scan_tmp_needed((int64_t)256 * nblk) + 8));
     ++g_launches, k_rs_hist<<<nblk, kBlock, 0, s>>>(n, kin, vin, mode, shift, P.sys_off_d, P.n_sys, P.hist, nblk);
     uint32_t *dtot = P.hist + (size_t)256 * nblk;
     ++g_launches, k_rs_dscan<<<256, 256, 0, s>>>(P.hist, nblk, dtot);
@@ -1374,14 +1368,8 @@ cudaError_t partition_boxes(Plan &P, cudaStream_t s) {
     const int64_t nb = P.nb;
     const int nblk = (int)((nb + kTile - 1) / kTile);
     const int64_t nh = (int64_t)4 * 256 * nblk;
-    if ((size_t)2 * nh > P.hist_elems) {
-        P.hist_elems = (size_t)2 * nh;
-        KIFMM_CUDA_TRY(plan_alloc(P, (void **)&P.hist, sizeof(uint32_t) * P.hist_elems));
-    }
-    if (scan_tmp_needed(nh) + 8 > P.scan_tmp_elems) {
-        P.scan_tmp_elems = scan_tmp_needed(nh) + 8;
-        KIFMM_CUDA_TRY(plan_alloc(P, (void **)&P.scan_tmp, sizeof(uint32_t) * P.scan_tmp_elems));
-    }
+    KIFMM_CUDA_TRY(hist_reserve(P, (size_t)2 * nh));
+    KIFMM_CUDA_TRY(scan_tmp_reserve(P, scan_tmp_needed(nh) + 8));
     ++g_launches, k_child8<<<grid_for(nb, 256), 256, 0, s>>>(nb, P.child_first, P.nchild, P.cx, P.cy, P.cz, P.child8);
     const dim3 grid((unsigned)nblk, 4);
     ++g_launches, k_part_hist<<<grid, kBlock, 0, s>>>(nb, nblk, P.nv, P.nchild, P.lvl, P.wsrc_flag, P.cx, P.cy, P.cz,
@@ -1455,8 +1443,7 @@ cudaError_t same_boxes(Plan &P, int *differs, cudaStream_t s) {
 cudaError_t save_boxes(Plan &P, cudaStream_t s) {
     if (P.nb > P.prev_cap) {
         const int64_t cap = P.nb + P.nb / 4 + 256;
-        KIFMM_CUDA_TRY(plan_alloc(P, (void **)&P.prev_tree, sizeof(int32_t) * 8 * cap));
-        P.prev_cap = cap;
+        KIFMM_CUDA_TRY(plan_replace(P, &P.prev_cap, cap, {{(void **)&P.prev_tree, sizeof(int32_t) * 8 * cap}}));
     }
     if (P.nb > 0)
         ++g_launches, k_boxes_save<<<grid_for(P.nb, 256), 256, 0, s>>>(P.nb, P.direct_thr, P.lvl, P.cx, P.cy, P.cz,
@@ -1598,8 +1585,8 @@ static cudaError_t build_levels(Plan &P, cudaStream_t s, int lsort) {
         const int ntiles = (int)((n + kOsTile - 1) / kOsTile);
         const size_t need_cnt = 2 * (size_t)lspec * std::max(ntiles, 1);  // counts, then first indices
         if (need_cnt > P.os_cnt_elems) {
+            KIFMM_CUDA_TRY(plan_grow(P, (void **)&P.os_cnt, sizeof(uint32_t) * need_cnt, 0));
             P.os_cnt_elems = need_cnt;
-            KIFMM_CUDA_TRY(plan_alloc(P, (void **)&P.os_cnt, sizeof(uint32_t) * P.os_cnt_elems));
         }
         const int M = P.desc.leaf_cap, D = P.desc.max_depth;
         if (ntiles > 0)
@@ -1848,17 +1835,15 @@ bool lists_finish(Plan &P) {
 
 cudaError_t grow_lists(Plan &P) {
     // grow the list storage (set_sources may allocate; evaluate never does)
-    if (P.n_u > P.u_cap) {
-        P.u_cap = P.n_u + P.n_u / 4 + 1024;
-        KIFMM_CUDA_TRY(plan_alloc(P, (void **)&P.u_idx, sizeof(int32_t) * P.u_cap));
-        if (P.periodic) KIFMM_CUDA_TRY(plan_alloc(P, (void **)&P.u_sh, P.u_cap));
-    }
-    if (P.n_w > P.w_cap) {
-        P.w_cap = P.n_w + P.n_w / 4 + 1024;
-        KIFMM_CUDA_TRY(plan_alloc(P, (void **)&P.w_idx, sizeof(int32_t) * P.w_cap));
-        if (P.periodic) KIFMM_CUDA_TRY(plan_alloc(P, (void **)&P.w_sh, P.w_cap));
-    }
-    return cudaSuccess;
+    auto grow = [&](int64_t n, int64_t *cap, int32_t **idx, int8_t **sh) -> cudaError_t {
+        if (n <= *cap) return cudaSuccess;
+        const int64_t c = n + n / 4 + 1024;
+        std::vector<BufSize> b = {{(void **)idx, sizeof(int32_t) * c}};
+        if (P.periodic) b.push_back({(void **)sh, (size_t)c});
+        return plan_replace(P, cap, c, b);
+    };
+    KIFMM_CUDA_TRY(grow(P.n_u, &P.u_cap, &P.u_idx, &P.u_sh));
+    return grow(P.n_w, &P.w_cap, &P.w_idx, &P.w_sh);
 }
 
 }  // namespace kifmm
