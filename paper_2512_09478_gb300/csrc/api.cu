@@ -188,7 +188,7 @@ static cudaError_t ensure_box_arrays(Plan &P) {
         {&P.u_chk, esz * P.ns * cap},
         {&P.d_chk, esz * P.ns * cap},
         {&P.up_dens, esz * P.ns * cap},
-        {&P.tmp_chk, esz * P.ns * cap},
+        {&P.tmp_chk, esz * (P.ns + 1) * cap},  // (m2l_exact: rows with the mean column)
         {&P.dn_dens, esz * P.ns * cap},
         {&P.adj_e1, esz * P.ns * cap},
         {&P.adj_e2, esz * P.ns * cap},
@@ -480,6 +480,7 @@ static kifmm_status set_sources_impl(Plan &P, const void *xyz, const void *q, cu
         API_CUDA(m2l_tiles_build(P, s));
         if (P.desc.precision == KIFMM_MIXED_FP16) API_CUDA(m2l_tensor_prepare(P));
         API_CUDA(m2l_exact_prepare(P));
+        m2l_part_prepare(P);
     }
     if (!P.lists_reused) {
         P.prev_nb = P.nb;

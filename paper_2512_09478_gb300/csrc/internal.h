@@ -117,8 +117,10 @@ struct Plan {
     void *m2l_tc = nullptr;     // layout owned by the tensor-core kernel
     void *m2l_ex = nullptr;     // operator slices of the exact-split M2L (FP64 / FP32 modes, every adjoint)
     void *m2l_tiles = nullptr;  // target tiles shared by both M2L kernels
-    void *m2l_part = nullptr;   // partial sums of their slot splits
+    void *m2l_part = nullptr;   // partial sums of their slot splits (at most kPartRoom bytes, or none)
     size_t m2l_part_bytes = 0;
+    size_t m2l_part_refused = 0;  // the smallest size the device had no room for
+    int m2l_part_retry = 0;       // requests until that size is asked for again
     float *m2l_tc_scale = nullptr;
     int *slot_off = nullptr;    // [8][189] V slot -> M2L offset index (-1 unused)
     // Compressed M2L (desc.m2l_eps > 0, tensor-core mode): d = U C_o W u with
@@ -228,7 +230,7 @@ struct Plan {
     int32_t *part_list[4] = {nullptr, nullptr, nullptr, nullptr};
     std::vector<int64_t> part_start[4];  // host: exclusive prefix of the key counts (257 entries)
     int32_t *child8 = nullptr;       // [nb][8] child in each octant, -1 if none
-    void *tmp_chk = nullptr;         // [nb][ns] pseudo-inverse scratch
+    void *tmp_chk = nullptr;         // [nb][ns + 1] scratch rows (pseudo-inverses, child products, m2l_exact's sums)
     void *dn_dens = nullptr;         // [nb][ns] normalised downward densities of leaves
     int64_t list_cap = 0;            // boxes the per-box list/expansion arrays hold
 
@@ -331,7 +333,17 @@ void m2l_tensor_release(Plan &P);
 cudaError_t m2l_tiles_build(Plan &P, cudaStream_t s);
 int m2l_tiles_128(const Plan &P);          // tiles of 128 targets
 const int4 *m2l_tiles_dev(const Plan &P);  // (class, begin, end, 0) each
-cudaError_t m2l_part_reserve(Plan &P, size_t bytes);
+// The slot splits' partial sums, a workspace that the kernels can do without:
+// asked for last, bounded, kept while a larger one is not to be had.  The bound
+// (a 400th of the device) holds the 189 slots of some 5000 targets at p = 6 at
+// once; larger trees go in rounds, whose CTAs fill their pipelines anew.
+// Measured, 120k charges in a periodic cell (566 MB of partial products):
+// 1085 us in one round, 1109 in two (400 MB), 1117 in three (256 MB), 1122 in
+// nine (96 MB), 1228 unsplit.
+constexpr size_t kPartRoom = (size_t)640 << 20;
+void m2l_part_prepare(Plan &P);
+size_t m2l_tensor_part_bytes(Plan &P, size_t room);  // what the best shape within `room` takes
+size_t m2l_exact_part_bytes(Plan &P);
 
 // ---- m2l_exact.cu (FP64 and FP32 modes, Stokeslet, every plan's adjoint) ----
 // dir 0 forward, 1 adjoint; ops [316][n_s][ld], device, compute type

@@ -212,6 +212,7 @@ struct ExArgs {
     T *d;                    // [nb][ns]
     double *dbar;            // [nb]: output column ns (the mean row), or nullptr
     T *part;                 // [slot split][target][ld] partial sums, or nullptr (one split)
+    int z0, zn, part_add;    // this launch: slot ranges z0 .. z0 + gridDim.z - 1 of zn; 1: added to part
     int64_t n_targets;
     int ns, ld, np, nt, kblocks, chunk_blocks, nchunks, nstages, nbuf, accumulate;
     long long wait_polls;
@@ -247,8 +248,8 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
     const int4 tile = a.tiles[blockIdx.x];
     const int cls = tile.x;
     // this CTA's slots
-    const int s_lo = (int)((int64_t)kVSlots * blockIdx.z / gridDim.z);
-    const int s_hi = (int)((int64_t)kVSlots * (blockIdx.z + 1) / gridDim.z);
+    const int s_lo = kVSlots * (a.z0 + (int)blockIdx.z) / a.zn;
+    const int s_hi = kVSlots * (a.z0 + (int)blockIdx.z + 1) / a.zn;
     const int NST = a.nstages, kblocks = a.kblocks;
     if (threadIdx.x < kTcRows) {
         const int i = tile.y + threadIdx.x;
@@ -526,7 +527,7 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
                     const int jc = c_first + col + j;
                     const T v = valid ? acc[g][j] : (T)NAN;
                     if (a.part) {
-                        if (jc < a.ld) out[jc] = v;
+                        if (jc < a.ld) out[jc] = a.part_add ? out[jc] + v : v;
                     } else if (jc < a.ns) {
                         out[jc] = a.accumulate ? out[jc] + v : v;
                     } else if (jc == a.ns && a.dbar) {
@@ -660,12 +661,16 @@ cudaError_t m2l_exact_setup(Plan &P, int dir, const void *ops, int ld) {
     return P.f64 ? ex_setup<double>(P, dir, (const double *)ops, ld) : ex_setup<float>(P, dir, (const float *)ops, ld);
 }
 
+// Slot ranges of one direction; they fix the order of the additions, so they
+// depend on the tree alone, not on the memory there is.
+static int ex_split(const Plan &P, const ExState &S, int dir) {
+    return m2l_slot_split((int64_t)m2l_tiles_128(P) * S.ncb[dir], P.num_sms);
+}
 static size_t ex_part_bytes(const Plan &P, const ExState &S, int dir, int z) {
     return (P.f64 ? sizeof(double) : sizeof(float)) * z * (size_t)P.m2l_class_start[8] * S.ld[dir];
 }
 
-// After set_sources: room for the sliced expansions and the slot splits'
-// partial sums (the adjoint's and the forward's are never live at once).
+// After set_sources: room for the sliced expansions.
 cudaError_t m2l_exact_prepare(Plan &P) {
     if (!P.m2l_ex) return cudaSuccess;
     ExState &S = ex_state(P);
@@ -677,13 +682,20 @@ cudaError_t m2l_exact_prepare(Plan &P) {
                                     {{(void **)&S.us, sizeof(uint16_t) * cap * S.kblocks * NS * kKB},
                                      {&S.rscale, esz * cap}}));
     }
+    return cudaSuccess;
+}
+
+// The slot splits' partial sums: at most 8 x 152 CTAs' accumulators (some
+// 100 MB), the adjoint's and the forward's never live at once.
+size_t m2l_exact_part_bytes(Plan &P) {
+    if (!P.m2l_ex) return 0;
+    const ExState &S = ex_state(P);
     size_t need = 0;
     for (int dir = 0; dir < 2; ++dir) {
-        if (!S.ops[dir].bs) continue;
-        const int z = m2l_slot_split((int64_t)m2l_tiles_128(P) * S.ncb[dir], P.num_sms);
+        const int z = S.ops[dir].bs ? ex_split(P, S, dir) : 1;
         if (z > 1) need = std::max(need, ex_part_bytes(P, S, dir, z));
     }
-    return m2l_part_reserve(P, need);
+    return need;
 }
 
 template <typename T>
@@ -718,13 +730,24 @@ static cudaError_t ex_run(Plan &P, int dir, const T *u, T *d, int accumulate, do
     a.accumulate = accumulate;
     a.wait_polls = P.m2l_wait_polls > 0 ? P.m2l_wait_polls : kWaitIters;
     a.status = P.status;
-    int z = m2l_slot_split((int64_t)ntiles * S.ncb[dir], P.num_sms);
-    if (ex_part_bytes(P, S, dir, z) > P.m2l_part_bytes) z = 1;  // no room for the partial sums
-    a.part = z > 1 ? (T *)P.m2l_part : nullptr;
+    const int z = ex_split(P, S, dir);
     const size_t smem = (size_t)a.nstages * SL::kSlices * (kTcRows + a.nt) * kRowB + 1024;
-    ++g_launches, k_m2l_exact<T><<<dim3((unsigned)ntiles, (unsigned)S.ncb[dir], (unsigned)z), ex_threads<T>(),
-                                 smem, s>>>(a);
-    if (z > 1) part_sum<T>(P, a.n_targets, z, a.ns, a.ld, a.part, d, accumulate, dbar, s);
+    auto launch = [&](int z0, int nz) {
+        a.z0 = z0;
+        a.part_add = nz == 1 && z0 > 0;
+        ++g_launches, k_m2l_exact<T><<<dim3((unsigned)ntiles, (unsigned)S.ncb[dir], (unsigned)nz), ex_threads<T>(),
+                                     smem, s>>>(a);
+    };
+    a.zn = z;
+    if (z == 1 || ex_part_bytes(P, S, dir, z) <= P.m2l_part_bytes) {
+        a.part = z > 1 ? (T *)P.m2l_part : nullptr;
+        launch(0, z);
+        if (z > 1) part_sum<T>(P, a.n_targets, z, a.ns, a.ld, a.part, d, accumulate, dbar, s);
+    } else {  // no room: the ranges one after the other into one set of rows, the same additions
+        a.part = (T *)P.tmp_chk;
+        for (int k = 0; k < z; ++k) launch(k, 1);
+        part_sum<T>(P, a.n_targets, 1, a.ns, a.ld, a.part, d, accumulate, dbar, s);
+    }
     return cudaGetLastError();
 }
 

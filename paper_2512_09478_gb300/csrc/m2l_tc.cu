@@ -67,7 +67,8 @@ struct TileArgs {
     const float *level_unscale;  // 1 / (sigma_A(level) sigma_B)
     float *d;                 // [nb][ns]
     double *dbar;             // [nb] output column ns (the mean row), or nullptr
-    float *part;              // SPLIT: [189][tile of 128][np][128] partial products
+    float *part;              // SPLIT: [slot of the round][tile of 128][np][128] partial products
+    int slot0, nslots;        // SPLIT: this round's slots
     int n_tiles;              // tiles of 128
     int ns, kp, np, nstages;  // np: operator rows (output columns) incl. padding
     int ncb;                  // column blocks (np = ncb NT)
@@ -142,8 +143,8 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
     const uint32_t tmem = tmem_base_s;
     const int kblocks = kp / kKBlock;
     // this CTA's slots
-    const int s_lo = SPLIT ? (int)(kVSlots * blockIdx.z / gridDim.z) : 0;
-    const int s_hi = SPLIT ? (int)(kVSlots * (blockIdx.z + 1) / gridDim.z) : kVSlots;
+    const int s_lo = SPLIT ? a.slot0 + a.nslots * (int)blockIdx.z / (int)gridDim.z : 0;
+    const int s_hi = SPLIT ? a.slot0 + a.nslots * (int)(blockIdx.z + 1) / (int)gridDim.z : kVSlots;
     const int iters = (s_hi - s_lo) * kblocks;
 
     if (warp < kProdWarps) {
@@ -287,7 +288,7 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
             // every slot's partial product, columns of 128 rows (tile.w: the
             // CTA's first tile of 128): a warp stores whole 128-byte lines
             if (t < ntl) {
-                float *out = a.part + (((size_t)s_lo * a.n_tiles + tile.w + t) * a.np + cb * NT + c_base) * kTcRows +
+                float *out = a.part + (((size_t)(s_lo - a.slot0) * a.n_tiles + tile.w + t) * a.np + cb * NT + c_base) * kTcRows +
                              q * 32 + lane;
                 float *const first = out;
                 bool ok = true;
@@ -373,27 +374,34 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
 }
 
 // Slot splits: the running sums of the drain warps (slot order), from the
-// stored partial products; a thread per target row and output column, the
-// rows of a tile adjacent.
+// stored partial products of one round of slots; a thread per target row and
+// output column, the rows of a tile adjacent.  `carry` holds the sums between
+// rounds, in the partial products' layout.
+constexpr int kSumSlots = 21;  // loads in flight per thread; a round is a multiple of it
 __global__ void __launch_bounds__(128) k_m2l_slot_sum(const int32_t *__restrict__ targets, const int4 *__restrict__ tiles,
-                                                      int n_tiles, int ns, int np,
-                                                      const float *__restrict__ part, const int32_t *__restrict__ lvl,
+                                                      int n_tiles, int ns, int np, int nslots, float *carry,
+                                                      int first, int last, const float *__restrict__ part, const int32_t *__restrict__ lvl,
                                                       const float *__restrict__ level_unscale, float *__restrict__ d,
                                                       double *__restrict__ dbar) {
     static_assert(kTcRows == 128, "a thread per row");
     const int4 tile = tiles[blockIdx.x];
     const int i = tile.y + threadIdx.x, j = blockIdx.y;
     if (i >= tile.z) return;
-    const float *src = part + ((size_t)blockIdx.x * np + j) * kTcRows + threadIdx.x;
+    const size_t at = ((size_t)blockIdx.x * np + j) * kTcRows + threadIdx.x;
+    const float *src = part + at;
     const size_t step = (size_t)n_tiles * np * kTcRows;
-    float a = 0.f;
-    static_assert(kVSlots % 21 == 0, "slots in rounds of 21 loads");
-    for (int s0 = 0; s0 < kVSlots; s0 += 21) {
-        float v[21];
+    float a = first ? 0.f : carry[at];
+    static_assert(kVSlots % kSumSlots == 0, "whole groups of loads");
+    for (int s0 = 0; s0 < nslots; s0 += kSumSlots) {
+        float v[kSumSlots];
 #pragma unroll
-        for (int k = 0; k < 21; ++k) v[k] = src[(s0 + k) * step];
+        for (int k = 0; k < kSumSlots; ++k) v[k] = src[(s0 + k) * step];
 #pragma unroll
-        for (int k = 0; k < 21; ++k) a += v[k];
+        for (int k = 0; k < kSumSlots; ++k) a += v[k];
+    }
+    if (!last) {
+        carry[at] = a;
+        return;
     }
     const int32_t t = targets[i];
     const float v = a * level_unscale[lvl[t]];
@@ -570,7 +578,15 @@ constexpr int kVariants[3][2] = {{2, 1}, {4, 1}, {2, 2}};
 
 }  // namespace
 
+// The shape of an untuned launch.
+struct TcShape {
+    int z = 1, tl = 1;    // slot ranges, tiles per CTA
+    int round = kVSlots;  // slots per round
+    size_t bytes = 0;     // partial products and carried sums (z > 1)
+};
+
 struct TcState {
+    TcShape shape;            // of the last set_sources' tree
     int np = 0, kp = 0, nstages = 0;
     int nt = 0, ncb = 0;      // output columns per CTA (MMA N), column blocks (np = nt ncb)
     float sigma_b = 1.f;
@@ -612,16 +628,34 @@ static M2lTiles &tile_state(Plan &P) {
 int m2l_tiles_128(const Plan &P) { return P.m2l_tiles ? ((const M2lTiles *)P.m2l_tiles)->n_tiles[0] : 0; }
 const int4 *m2l_tiles_dev(const Plan &P) { return ((const M2lTiles *)P.m2l_tiles)->tiles; }
 
-cudaError_t m2l_part_reserve(Plan &P, size_t bytes) {
-    if (bytes <= P.m2l_part_bytes) return cudaSuccess;
-    P.m2l_part_bytes = 0;
-    const cudaError_t e = plan_alloc(P, &P.m2l_part, bytes);
-    if (e == cudaErrorMemoryAllocation) {  // run unsplit, which needs none
-        cudaGetLastError();
-        return cudaSuccess;
+// A buffer of at least `bytes` (a quarter more, while that stays within the
+// bound, so that a growing tree does not ask each time); false when the device
+// has no room: the old one is kept and the size not asked for again soon.
+static bool part_reserve(Plan &P, size_t bytes) {
+    if (bytes <= P.m2l_part_bytes) return true;
+    if (P.m2l_part_refused && bytes >= P.m2l_part_refused && P.m2l_part_retry-- > 0) return false;
+    for (const size_t ask : {std::max(bytes, std::min(bytes + bytes / 4, kPartRoom)), bytes}) {
+        if (plan_grow(P, &P.m2l_part, ask, 0) == cudaSuccess) {
+            P.m2l_part_bytes = ask;
+            P.m2l_part_refused = 0;
+            return true;
+        }
+        (void)cudaGetLastError();
     }
-    if (e == cudaSuccess) P.m2l_part_bytes = bytes;
-    return e;
+    P.m2l_part_refused = bytes;
+    P.m2l_part_retry = 16;
+    return false;
+}
+
+static void m2l_tensor_set_shape(Plan &P);
+
+void m2l_part_prepare(Plan &P) {
+    const size_t ex = m2l_exact_part_bytes(P);
+    for (size_t room = kPartRoom; room >= kPartRoom / 16; room /= 4) {
+        const size_t tc = P.desc.precision == KIFMM_MIXED_FP16 ? m2l_tensor_part_bytes(P, room) : 0;
+        if (part_reserve(P, std::max(ex, tc)) || tc == 0) break;
+    }
+    if (P.desc.precision == KIFMM_MIXED_FP16) m2l_tensor_set_shape(P);
 }
 
 static TcState &tc_state(Plan &P) {
@@ -740,38 +774,68 @@ cudaError_t m2l_tiles_build(Plan &P, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// Slot split z and tiles per CTA (of 128 targets) of an untuned launch: the
-// pair with the shortest estimated time.  An SM takes in a stage's bytes at
-// about 33 per clock, 68 KB per us (p = 6: 36 KB in 0.53 us with one tile per
-// CTA, 52 KB in 0.82 with two); a CTA costs about four slots of set-up and fill
-// beside its 189 / z.  A split stores every slot's partial products (2.6 TB/s
-// beside the products) and reads them back (5.4 TB/s).  Measured, both sides:
-// 12k particles (585 boxes) 957 -> 537 us a step; 120k in a periodic cell (4681
-// boxes) 1885 -> 1171 (with the root's own kernels); 1M (150 CTAs of two tiles)
-// runs unsplit as before, 2531 us.
-static void tc_shape(int n1, int n2, int ncb, int np, int kblocks, int num_sms, int *z_out,
-                     int *tl_out) {
+// Slot split z, tiles per CTA (of 128 targets) and slots per round of an
+// untuned launch: those with the shortest estimated time whose partial products
+// fit `room`.  An SM takes in a stage's bytes at about 33 per clock, 68 KB per
+// us (p = 6: 36 KB in 0.53 us with one tile per CTA, 52 KB in 0.82 with two); a
+// CTA costs about four slots of set-up and fill beside its own.  A split stores
+// every slot's partial products (2.6 TB/s beside the products) and reads them
+// back (5.4 TB/s).  The 189 slots go in rounds that write the same buffer, the
+// running sums carried over, so that no tree takes more than kPartRoom.
+// Measured, both sides: 12k particles (585 boxes) 957 -> 537 us a step; 120k in
+// a periodic cell (4681 boxes) 1885 -> 1171 (with the root's own kernels); 1M
+// (150 CTAs of two tiles) runs unsplit as before, 2531 us.
+static TcShape tc_shape(int n1, int n2, int ncb, int np, int kblocks, int num_sms, size_t room) {
+    TcShape best;
     double least = 1e30;
-    *z_out = 1;
-    *tl_out = 1;
-    const double part_bytes = 4.0 * kVSlots * kTcRows * (double)n1 * np;
-    for (int z = 1; z <= 63 && (z == 1 || (int64_t)n1 * ncb * z <= 8 * (int64_t)num_sms); ++z)
+    const size_t slot_bytes = sizeof(float) * kTcRows * (size_t)n1 * np;
+    constexpr int kGroups = kVSlots / kSumSlots;
+    // the fewest rounds that fit
+    int g = 0;
+    size_t bytes = 0;
+    for (const int k : {9, 5, 3, 2, 1}) {  // groups of kSumSlots slots: 1, 2, 3, 5 or 9 rounds
+        static_assert(kGroups == 9, "one to nine rounds");
+        bytes = slot_bytes * (k * kSumSlots + (k < kGroups ? 1 : 0));
+        if (n1 > 0 && bytes <= room) {
+            g = k;
+            break;
+        }
+    }
+    for (int z = 1; z <= std::min(63, g * kSumSlots) || z == 1; ++z) {
+        if (z > 1 && (int64_t)n1 * ncb * z > 8 * (int64_t)num_sms) break;
         for (int tl = 1; tl <= 2; ++tl) {
             if (tl == 2 && n2 == n1) continue;
             const int64_t ctas = (int64_t)(tl == 1 ? n1 : n2) * ncb * z;
+            const double waves = (double)((ctas + num_sms - 1) / num_sms);
             const double stage_us = (tl * 2.0 * kTcRows + 2.0 * np / ncb) * kRowBytes / 68e3;
-            double t = (double)((ctas + num_sms - 1) / num_sms) * ((kVSlots + z - 1) / z + 4.0) * kblocks * stage_us;
-            if (z > 1) t = std::max(t, part_bytes / 2.6e6) + part_bytes / 5.4e6 + 6.0;
+            double t = 0.0;
+            if (z == 1) {
+                t = waves * (kVSlots + 4.0) * kblocks * stage_us;
+            } else {
+                for (int left = kGroups; left > 0; left -= g) {
+                    const int slots = std::min(left, g) * kSumSlots;
+                    const double part = (double)slot_bytes * slots;
+                    t += std::max(waves * ((slots + z - 1) / z + 4.0) * kblocks * stage_us, part / 2.6e6) +
+                         part / 5.4e6 + 6.0;
+                }
+            }
             if (t < 0.98 * least) {
                 least = t;
-                *z_out = z;
-                *tl_out = tl;
+                best = z == 1 ? TcShape{1, tl, kVSlots, 0} : TcShape{z, tl, g * kSumSlots, bytes};
             }
         }
+    }
+    return best;
 }
-static size_t tc_part_bytes(int n1, int np) { return sizeof(float) * kVSlots * (size_t)n1 * kTcRows * np; }
+static TcShape tc_shape_of(Plan &P, size_t room) {
+    const TcState &S = tc_state(P);
+    const M2lTiles &TS = tile_state(P);
+    return tc_shape(TS.n_tiles[0], TS.n_tiles[1], S.ncb, S.np, S.kp / kKBlock, P.num_sms, room);
+}
+size_t m2l_tensor_part_bytes(Plan &P, size_t room) { return tc_shape_of(P, room).bytes; }
+static void m2l_tensor_set_shape(Plan &P) { tc_state(P).shape = tc_shape_of(P, P.m2l_part_bytes); }
 
-// Room for the split expansions and the slot splits' partial products.
+// Room for the split expansions.
 cudaError_t m2l_tensor_prepare(Plan &P) {
     TcState &S = tc_state(P);
     if (P.nb > S.u_cap) {
@@ -779,10 +843,7 @@ cudaError_t m2l_tensor_prepare(Plan &P) {
         KIFMM_CUDA_TRY(plan_replace(P, &S.u_cap, cap, {{(void **)&S.uh, sizeof(__half) * cap * S.kp},
                                                        {(void **)&S.ul, sizeof(__half) * cap * S.kp}}));
     }
-    const M2lTiles &TS = tile_state(P);
-    int z, tl;
-    tc_shape(TS.n_tiles[0], TS.n_tiles[1], S.ncb, S.np, S.kp / kKBlock, P.num_sms, &z, &tl);
-    return m2l_part_reserve(P, z > 1 ? tc_part_bytes(TS.n_tiles[0], S.np) : 0);
+    return cudaSuccess;
 }
 
 cudaError_t m2l_tensor(Plan &P, cudaStream_t s) {
@@ -820,12 +881,12 @@ cudaError_t m2l_tensor(Plan &P, cudaStream_t s) {
     a.kp = S.kp;
     a.np = S.np;
     a.status = P.status;
-    int z, tl_default;
-    tc_shape(TS.n_tiles[0], TS.n_tiles[1], S.ncb, S.np, S.kp / kKBlock, P.num_sms, &z,
-             &tl_default);
-    if (tc_part_bytes(TS.n_tiles[0], S.np) > P.m2l_part_bytes) z = 1;  // no room for the partial products
+    const TcShape shape = S.shape;
+    const int z = shape.z;
     a.part = z > 1 ? (float *)P.m2l_part : nullptr;
     a.n_tiles = TS.n_tiles[0];
+    a.slot0 = 0;
+    a.nslots = shape.round;
     auto launch_v = [&](auto pwc, auto tlc, auto spl, int nst) -> cudaError_t {
         constexpr int PW = decltype(pwc)::value, TL = decltype(tlc)::value;
         constexpr bool SP = decltype(spl)::value;
@@ -856,7 +917,7 @@ cudaError_t m2l_tensor(Plan &P, cudaStream_t s) {
         return pw == 4 ? launch_v(I4{}, I1{}, std::false_type{}, nst) : launch_v(I2{}, I1{}, std::false_type{}, nst);
     };
     if (!P.tuned_m2l) {
-        const bool two = tl_default == 2;  // each operator block read once for 256 targets
+        const bool two = shape.tl == 2;  // each operator block read once for 256 targets
         S.pw = 2;
         S.tl = two ? 2 : 1;
         S.nstages = two ? std::min(3, S.nstages_max(2)) : S.nstages_max(1);
@@ -888,12 +949,15 @@ cudaError_t m2l_tensor(Plan &P, cudaStream_t s) {
         S.tl = pick_tl;
         P.tuned_m2l = true;
     }
-    KIFMM_CUDA_TRY(launch_with(S.pw, S.tl, S.nstages));
-    if (z > 1) {
+    for (; a.slot0 < kVSlots; a.slot0 += shape.round) {  // one round, the whole, unless split
+        a.nslots = std::min(shape.round, kVSlots - a.slot0);
+        KIFMM_CUDA_TRY(launch_with(S.pw, S.tl, S.nstages));
+        if (z == 1) break;
         const int cols = S.n_out + (a.dbar ? 1 : 0);
+        float *carry = a.part + (size_t)shape.round * a.n_tiles * S.np * kTcRows;
         ++g_launches, k_m2l_slot_sum<<<dim3((unsigned)TS.n_tiles[0], (unsigned)cols), kTcRows, 0, s>>>(
-                          P.m2l_targets, TS.tiles, TS.n_tiles[0], a.ns, S.np, a.part, P.lvl, S.level_unscale,
-                          a.d, a.dbar);
+                          P.m2l_targets, TS.tiles, TS.n_tiles[0], a.ns, S.np, a.nslots, carry, a.slot0 == 0,
+                          a.slot0 + a.nslots == kVSlots, a.part, P.lvl, S.level_unscale, a.d, a.dbar);
     }
     if (comp) {  // back to the mean-free check potential of every target
         const int64_t nt = P.m2l_class_start[8];

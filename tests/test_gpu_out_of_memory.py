@@ -108,3 +108,55 @@ def test_a_refused_allocation_leaves_a_plan_that_works(precision, kernel, reuse)
     del base
     torch.cuda.empty_cache()
     assert 0 < refused < len(ROOM)  # the sweep met both outcomes
+
+
+@pytest.mark.parametrize("precision,kernel", [("mixed_fp16", "laplace"), ("fp64", "laplace"), ("fp32", "laplace"),
+                                              ("fp64", "stokeslet")])
+def test_the_bits_do_not_depend_on_the_room_for_partial_products(precision, kernel):
+    """The partial products of the slot splits are the last thing set_sources
+    asks for, and the kernels do without them: whatever room there is, a tree
+    that builds gives the same bits, forward and adjoint."""
+    from paper_2512_09478_gb300 import KifmmError, Plan
+    dtype = torch.float64 if precision == "fp64" else torch.float32
+    big = _Set(12_000, dtype, kernel, 65)
+    mk = lambda: Plan(p=4, leaf_cap=8, precision=precision, kernel=kernel, n_max=len(big.x), dtype=dtype)
+    plan = mk()
+    ref = [t.cpu() for t in big.run(plan, kernel)]
+    plan.close()
+    base = _hog(6 << 30)
+    taken = set()
+    for room in (m << 20 for m in range(16, 640, 24)):
+        plan = mk()
+        hog = _hog(room)
+        before = torch.cuda.mem_get_info()[0]
+        try:
+            got = [t.cpu() for t in big.run(plan, kernel)]
+            taken.add((before - torch.cuda.mem_get_info()[0]) >> 21)
+            assert all(torch.equal(a, b) for a, b in zip(got, ref)), room
+            assert plan.device_status() == 0
+        except KifmmError as e:
+            assert e.code == 3, room
+        del hog
+        torch.cuda.empty_cache()
+        plan.close()
+    del base
+    torch.cuda.empty_cache()
+    assert len(taken) > 1  # with the buffer and without
+
+
+def test_partial_products_are_bounded():
+    """A tree of some 5000 boxes at p = 8: unbounded, the 189 slots' partial
+    products of its 40 tiles would take 1.2 GB."""
+    from paper_2512_09478_gb300 import Plan
+    x, q = G.uniform_charges(120_000, 67)
+    xt, qt = (torch.tensor(a, dtype=torch.float32, device="cuda") for a in (x, q))
+    plan = Plan(p=8, leaf_cap=64, precision="mixed_fp16", n_max=len(x))
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    plan.set_sources(xt, qt)
+    taken = before - torch.cuda.mem_get_info()[0]
+    nb = plan.tree_info()["n_boxes"]
+    # per box (a quarter more boxes than there are): lists 1.6 KB, eight
+    # expansions of 296 values, their 16-bit slices; leaf pass lists
+    per_box = 1700 + 8 * 4 * 297 + 2 * 2 * 320 + 3 * 2 * 320
+    assert taken <= 1.25 * (nb + 256) * per_box + 8 * 6 * len(x) / 8 + (640 << 20) + (64 << 20)
