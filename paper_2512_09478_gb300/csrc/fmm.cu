@@ -2003,8 +2003,11 @@ __global__ void __launch_bounds__(kLeafThreads) k_adj_leaf(LeafCtx C, const int3
                     const V4 v = src[k], d = dip[k];
                     const T rx = x - v.x, ry = y - v.y, rz = z - v.z;
                     const T r2 = rx * rx + ry * ry + rz * rz;
-                    // the particle itself and coincident points add nothing
-                    const T ri = r2 > T(0) ? rsqrt_t<T>(r2) : T(0), ri2 = ri * ri, ri3 = ri * ri2;
+                    // the particle itself and coincident points are left out (a
+                    // zero weight would not do: an infinite dipole times zero is
+                    // NaN)
+                    if (!(r2 > T(0))) continue;
+                    const T ri = rsqrt_t<T>(r2), ri2 = ri * ri, ri3 = ri * ri2;
                     hess(rx, ry, rz, v.w, ri2, ri3);
                     const T gr = d.x * rx + d.y * ry + d.z * rz;
                     const T gr3 = T(3) * gr * ri2;
