@@ -359,6 +359,7 @@ inline bool m2l_uses_simt(const Plan &P) {
 }
 cudaError_t m2l_simt_setup(Plan &P);
 cudaError_t m2l_simt(Plan &P, const float *u, float *d, double *dbar, cudaStream_t s);
+size_t m2l_simt_part_bytes(const Plan &P, size_t room);  // partial products of a slot split within `room`
 
 // ---- fmm.cu ----
 // Autotuning: true when desc.autotune asks for it, something is still

@@ -652,8 +652,10 @@ static void m2l_tensor_set_shape(Plan &P);
 void m2l_part_prepare(Plan &P) {
     const size_t ex = m2l_exact_part_bytes(P);
     for (size_t room = kPartRoom; room >= kPartRoom / 16; room /= 4) {
-        const size_t tc = P.desc.precision == KIFMM_MIXED_FP16 ? m2l_tensor_part_bytes(P, room) : 0;
-        if (part_reserve(P, std::max(ex, tc)) || tc == 0) break;
+        const size_t own = P.desc.precision == KIFMM_MIXED_FP16 ? m2l_tensor_part_bytes(P, room)
+                           : m2l_uses_simt(P)                       ? m2l_simt_part_bytes(P, room)
+                                                                    : 0;
+        if (part_reserve(P, std::max(ex, own)) || own == 0) break;
     }
     if (P.desc.precision == KIFMM_MIXED_FP16) m2l_tensor_set_shape(P);
 }
