@@ -1411,13 +1411,14 @@ cudaError_t evaluate_t(Plan &P, void *pot, void *grad, double *energy, cudaStrea
     }
     const LeafW<T> W{(const T *)P.dn_dens, 1, (const T *)P.up_dens, 1, nullptr};
     if (!P.tuned_leaf && tuning_wanted(P, s)) {
-        // time every candidate table on this tree; keep the fastest
+        // time the default table and every candidate on this tree; keep the fastest
         float best = 1e30f;
         LeafTiling pick = P.leaf_tile;
         leaf_launch<T>(P, C, pts, surf, W, res, s);  // warm the caches first
-        for (int c = 0; c < kLeafTilingCandidates; ++c) {
+        for (int c = -1; c < kLeafTilingCandidates; ++c) {
             LeafCtx Cc = C;
-            Cc.tile = leaf_tiling_candidate(c);
+            if (c >= 0) Cc.tile = leaf_tiling_candidate(c);
+            if (c >= 0 && Cc.tile.packed == C.tile.packed) continue;  // the default, timed
             float ms = 1e30f;
             for (int rep = 0; rep < 2; ++rep)  // best of two
                 ms = std::min(ms, time_launch(s, [&] { leaf_launch<T>(P, Cc, pts, surf, W, res, s); }));

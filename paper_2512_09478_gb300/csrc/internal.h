@@ -37,10 +37,11 @@ struct LeafTiling {
     }
 };
 __host__ __device__ inline int leaf_variant(const LeafTiling &t, int n) { return t.for_targets(n > 0 ? n : 1); }
-// Candidate c of the tuner (c = 0 is the default): the variant for up to 8,
-// 16, 24, 32, 64 and more remaining targets.
+// Candidate c of the tuner (beside the plan's default: candidate 0, in the FP64
+// mode leaf_tiling_f64): the variant for up to 8, 16, 24, 32, 64 and more
+// remaining targets.
 LeafTiling leaf_tiling_candidate(int c);
-LeafTiling leaf_tiling_f64();  // the FP64 mode's default
+LeafTiling leaf_tiling_f64();
 
 struct DevBuf {
     void *ptr = nullptr;
