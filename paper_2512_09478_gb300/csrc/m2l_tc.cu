@@ -637,7 +637,7 @@ static bool part_reserve(Plan &P, size_t bytes) {
     for (const size_t ask : {std::max(bytes, std::min(bytes + bytes / 4, kPartRoom)), bytes}) {
         if (plan_grow(P, &P.m2l_part, ask, 0) == cudaSuccess) {
             P.m2l_part_bytes = ask;
-            P.m2l_part_refused = 0;
+            if (ask >= P.m2l_part_refused) P.m2l_part_refused = 0;  // (a smaller one says nothing about it)
             return true;
         }
         (void)cudaGetLastError();
