@@ -61,7 +61,8 @@ typedef enum {
     KIFMM_FP64 = 0,       /* every stage in double precision (parity path) */
     KIFMM_FP32 = 1,       /* single precision throughout ("plain FP32"): M2L as
                              sums of FP16 slices' exact products, closer to
-                             the exact translations than an FP32 product     */
+                             the exact translations than an FP32 product; as
+                             FP32 FMAs for the Stokeslet and periodic cells  */
     KIFMM_MIXED_FP16 = 3  /* M2L on tensor cores, 3xFP16 split with power-of-two
                              scaling, FP32 accumulate                         */
 } kifmm_precision;

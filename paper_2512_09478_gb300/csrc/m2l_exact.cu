@@ -1,6 +1,7 @@
 // M2L at full FP32 or FP64 accuracy on the Blackwell tensor cores (tcgen05 /
-// TMEM): the V-list translations of the FP64 and FP32 modes, of the Stokeslet
-// and of every plan's adjoint,
+// TMEM): the V-list translations of the FP64 mode, of the FP32 mode in free
+// space with the Laplace kernel (the other FP32 plans: m2l_simt.cu) and of every
+// adjoint,
 //     d(t) = sum_{s < 189} M_{off(c,s)} u(src(t, s)),
 // as sums of 16-bit products that the tensor core adds without rounding.
 //
@@ -34,11 +35,14 @@
 // What bounds it: the FP64 unit runs 2 lanes per clock and SM (conversions
 // included), so a SIMT product takes 128 x 152 x 152 / 2 = 1.5 M clocks per
 // slot of a 128-target tile; here the tensor core takes 36 (FP64) or 6 (FP32)
-// products of 128 x 160 x 160, 28 k and 5 k clocks, two FP64 operations per
-// output and slot are left, and the gathered rows' 16-byte copies feed the
-// stages (FP64: 96 KB each, some 13 bytes per clock and SM, the bound).
-// Measured, M2L alone: FP64, 60k Plummer, p = 6: 30.7 -> 2.4 ms; FP32, 200k
-// packing, p = 6: 3.30 -> 0.28 ms (the gathered SIMT product before).
+// products of 128 x 160 x 160, 28 k and 5 k clocks, and two FP64 operations per
+// output and slot are left.  FP32 waits for its stages' bytes, like the mixed
+// kernel.  FP64 has one set of accumulators (eight groups of 64 columns are all
+// of tensor memory), so a slot's products wait for the drain of the slot before:
+// its stages, 96 KB each, arrive at some 13 bytes per clock and SM where the
+// mixed kernel's reach 33.  Measured, M2L alone: FP64, 60k Plummer, p = 6: 30.7
+// -> 1.95 ms; FP32, 200k packing, p = 6: 3.30 -> 0.29 ms (the gathered SIMT
+// product before).
 //
 // Pipeline and bounded waits as in m2l_tc.cu: producer warps (cp.async
 // of the gathered rows, one bulk copy of the operator block per stage), one
@@ -73,7 +77,7 @@ struct Slicing<float> {
 template <>
 struct Slicing<double> {
     static constexpr int kSlices = 8, kGroups = 8, kCols = 64, kChunkBlocks = 5;  // K <= 160 per accumulation
-    static constexpr int kProd = 2;  // producer warps: with 12 or fewer warps the drain's 160 registers fit
+    static constexpr int kProd = 2;  // producer warps: 11 warps leave the drain 168 registers (64 bytes spill)
     static constexpr uint32_t kFmt = 1;                                           // BF16
 };
 
@@ -579,7 +583,8 @@ static void part_sum(const Plan &P, int64_t n_t, int nsplit, int ns, int ld, con
 // A rule for how many CTAs share a tile's 189 slots when `units` (tiles x
 // column blocks) CTAs would run at one per SM: the split z that minimises the
 // waves' length ceil(units z / SMs) (189 / z + 4), a CTA's set-up, pipeline
-// fill and partial store costing about four slots.  Few tiles (small trees)
+// fill and partial store costing about four slots (three without the partial
+// store, z = 1).  Few tiles (small trees)
 // would otherwise leave most SMs idle for 189 slots in a row.
 int m2l_slot_split(int64_t units, int num_sms) {
     if (units <= 0) return 1;
@@ -649,8 +654,6 @@ static cudaError_t ex_setup(Plan &P, int dir, const T *ops, int ld) {
     ++g_launches, k_slice_ops<T><<<(unsigned)((total + 255) / 256), 256>>>((int64_t)total, P.ns, ld, S.np[dir],
                                                                           S.nt[dir], S.kblocks, ops, oexp,
                                                                           S.ops[dir].bs);
-    const int smem = (int)(ex_stages<T>(S.nt[dir]) * (size_t)SL::kSlices * (kTcRows + S.nt[dir]) * kRowB + 1024);
-    (void)smem;
     // the largest any column-block width takes
     KIFMM_CUDA_TRY(cudaFuncSetAttribute(k_m2l_exact<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 2048));
     KIFMM_CUDA_TRY(cudaDeviceSynchronize());
