@@ -247,7 +247,6 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
     __shared__ uint32_t tmem_base_s;
     __shared__ int32_t tgt_s[kTcRows];
     __shared__ volatile int abort_s;
-    __shared__ int last_bulk_s;  // the last stage a bulk copy was issued for, -1: none
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int4 tile = a.tiles[blockIdx.x];
     const int cls = tile.x;
@@ -261,7 +260,6 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
     }
     if (threadIdx.x == 0) {
         abort_s = 0;
-        last_bulk_s = -1;
         for (int s = 0; s < NST; ++s) {
             mbar_init(smem_u32(&full_bar[s]), 32 * kProd + 1);  // producer cp.async arrivals + the bulk-copy leader
             mbar_init(smem_u32(&empty_bar[s]), 1);
@@ -302,7 +300,7 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
         }
         const bool leader = threadIdx.x == 0;
         int o_cur = 0, o_next = leader ? a.slot_off[cls * kVSlots + s_lo] : 0;
-        int it = 0;
+        int it = 0, last_it = -1;
         bool ok = true;
         for (int s = s_lo; s < s_hi && ok; ++s) {
 #pragma unroll
@@ -329,7 +327,7 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
                     const size_t boff = (((size_t)o_cur * kblocks + kb) * a.np + c_first) * (size_t)(NS * kKB);
                     mbar_arrive_expect_tx(fb, NS * b_slice);
                     bulk_g2s(sB, a.bs + boff, NS * b_slice, fb);
-                    last_bulk_s = it;
+                    last_it = it;
                 }
 #pragma unroll
                 for (int i = 0; i < kRows; ++i) {
@@ -344,7 +342,7 @@ __global__ void __launch_bounds__(ex_threads<T>(), 1) k_m2l_exact(ExArgs<T> a) {
             }
         }
         cp_async_wait_all();
-        wait_bulk_copies(full_bar, NST, 32 * kProd, it, &last_bulk_s, leader);
+        if (leader) wait_bulk_copies(full_bar, NST, last_it);
     } else if (warp == kProd) {
         // ---------------- MMA issuer ----------------
         // One accumulation per (slot, K chunk), in accumulator set w % nbuf.

@@ -102,7 +102,6 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
     __shared__ int32_t tgt_s[kRows];
 
     __shared__ volatile int abort_s;
-    __shared__ int last_bulk_s;  // the last stage a bulk copy was issued for, -1: none
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int4 tile = a.tiles[blockIdx.x];
@@ -116,7 +115,6 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
 
     if (threadIdx.x == 0) {
         abort_s = 0;
-        last_bulk_s = -1;
         for (int s = 0; s < NS; ++s) {
             mbar_init(smem_u32(&full_bar[s]), 32 * kProdWarps + 1);  // producer cp.async arrivals + the bulk-copy leader
             mbar_init(smem_u32(&empty_bar[s]), 1);
@@ -165,8 +163,8 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
         }
         const bool leader = threadIdx.x == 0;
         int o_cur = 0, o_next = leader ? a.slot_off[cls * kVSlots + s_lo] : 0;
-        int it = 0;
-        for (; it < iters; ++it) {
+        int last_it = -1;
+        for (int it = 0; it < iters; ++it) {
             const int stage = it % NS;
             const int s = s_lo + it / kblocks, kb = it - (s - s_lo) * kblocks;
             if (kb == 0) {
@@ -195,7 +193,7 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
                 const size_t boff = (((size_t)o_cur * kblocks + kb) * a.ncb + cb) * 2 * (size_t)NT * kKBlock;
                 mbar_arrive_expect_tx(fb, 2 * b_bytes);
                 bulk_g2s(sB, a.bhl + boff, 2 * b_bytes, fb);
-                last_bulk_s = it;
+                last_it = it;
             }
             const size_t koff = (size_t)kb * kKBlock + 8 * ch;
 #pragma unroll
@@ -211,7 +209,7 @@ __global__ void __launch_bounds__(tc_threads(PW, TL), 1) k_m2l_tc(TileArgs a) {
             cp_async_arrive_noinc(fb);
         }
         cp_async_wait_all();
-        wait_bulk_copies(full_bar, NS, 32 * kProdWarps, it, &last_bulk_s, leader);
+        if (leader) wait_bulk_copies(full_bar, NS, last_it);
     } else if (warp == kMmaWarp) {
         // ---------------- MMA issuer ----------------
         // Partial accumulator u = s ntl + t (slot s, tile t) goes to buffer

@@ -78,26 +78,21 @@ __device__ __forceinline__ void cp_async_arrive_noinc(uint32_t bar) {
 
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// The producer threads' end, time-out or not: the bulk copies of the last
-// n_stages stages up to *last (-1: none issued) must land before the CTA's
-// shared memory goes away.  `arrived`: the stages this thread arrived on; the
-// arrivals that a time-out made it stop short of are made up here, so that
-// every stage holding a bulk copy completes.  (The copy of stage k was issued
-// only after stage k - n_stages had been consumed, so no thread is more than
-// n_stages behind and each arrival lands in its own phase.)
-__device__ __forceinline__ void wait_bulk_copies(uint64_t *full, int n_stages, int threads, int arrived,
-                                                 const int *last_s, bool leader) {
-    __syncwarp();
-    asm volatile("barrier.cta.sync 1, %0;" ::"r"(threads) : "memory");  // the leader's *last is final
-    const int last = *last_s;
+// The leader's end, time-out or not: the bulk copies in flight, of the last
+// n_stages stages up to `last` (-1: none issued), must land before the CTA's
+// shared memory goes away.  Newest first: once its stage completes, every
+// producer thread has arrived on the stages before it, which complete as their
+// bytes land.  A stage that a thread stopped short of (a time-out) never
+// completes; its wait then runs to the bound, which outlasts any copy.
+__device__ __forceinline__ void wait_bulk_copies(uint64_t *full, int n_stages, int last) {
+    bool done = true;
 #pragma unroll 1
-    for (int k = arrived; k <= last; ++k) mbar_arrive(smem_u32(&full[k % n_stages]));
-    if (!leader) return;
+    for (int k = last; done && k >= 0 && k > last - n_stages; --k) {
+        done = false;
 #pragma unroll 1
-    for (int k = last >= n_stages ? last - n_stages + 1 : 0; k <= last; ++k)
-#pragma unroll 1
-        for (int i = 0; i < kCleanupPolls; ++i)
-            if (mbar_try_wait(smem_u32(&full[k % n_stages]), (uint32_t)(k / n_stages) & 1u)) break;
+        for (int i = 0; !done && i < kCleanupPolls; ++i)
+            done = mbar_try_wait(smem_u32(&full[k % n_stages]), (uint32_t)(k / n_stages) & 1u);
+    }
 }
 
 // Shared-memory matrix descriptor: K-major, 64-byte swizzle, rows of 64 bytes,
