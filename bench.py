@@ -66,8 +66,8 @@ _M2L_SRC = ("paper_2512_09478_gb300/csrc/m2l_tc.cu", "paper_2512_09478_gb300/csr
 _LEAF_SRC = ("paper_2512_09478_gb300/csrc/fmm.cu", "paper_2512_09478_gb300/csrc/common.cuh",
              "paper_2512_09478_gb300/csrc/internal.h")
 TRAFFIC = {
-    ("dem-coulomb-rsa-1M", "m2l"): (_M2L_SRC, "2930bb808ea1995153aa528a283826ff0089836c0692b1a886b3579915bdf02c", 96189952),
-    ("dem-coulomb-rsa-1M", "p2p"): (_LEAF_SRC, "878cc63175916d94552a1ff20aace24ffec7bd61c66ecd4b34b2f350e9ae4b9d", 76453120),
+    ("dem-coulomb-rsa-1M", "m2l"): (_M2L_SRC, "350ac454683d95ed902778452ee85970ef59c5fa0c81be79f5ae2db77402f349", 96449024),
+    ("dem-coulomb-rsa-1M", "p2p"): (_LEAF_SRC, "afd626f42d46f892bbd1aa5400fa48da2f67c2141fa249c1eea6b5c2a7bb490b", 76361728),
 }
 
 

@@ -392,8 +392,8 @@ kifmm_status kifmm_profile_read(kifmm_plan *plan, kifmm_profile_t *out);
 
 /* Tile shapes in use (no counterpart in the paper: the M2L and P2P tile
  * shapes are chosen by an autotuner on the live tree).  tuned: bit 0 leaf kernel,
- * bit 1 tensor-core M2L.  m2l_stages: shared-memory pipeline depth of the
- * tensor-core M2L (0 when the plan has none).  Leaf kernel: a leaf is
+ * bit 1 the mixed mode's M2L.  m2l_stages: shared-memory pipeline depth of the
+ * mixed mode's M2L (0 in the other modes).  Leaf kernel: a leaf is
  * covered by passes; with r of its targets still to cover, bucket
  * min((r - 1) / 8, 15) selects leaf_tpl targets per lane and leaf_groups
  * source groups for the next pass, which covers 32 / groups * tpl targets;
@@ -408,27 +408,29 @@ typedef struct {
     int m2l_rank_out;    /* compressed M2L: left rank (outputs, without the
                             mean column); 0 for a dense M2L               */
     int m2l_rank_in;     /* compressed M2L: right rank (inputs); 0 if dense  */
-    int m2l_producers;   /* tensor-core M2L: warps gathering the source rows
-                            (0 when the plan has none)                      */
-    int m2l_tiles;       /* tensor-core M2L: tiles of 128 targets per CTA that
+    int m2l_producers;   /* the mixed mode's M2L: warps gathering the source
+                            rows (0 in the other modes)                     */
+    int m2l_tiles;       /* the mixed mode's M2L: tiles of 128 targets per CTA that
                             share each operator block (1 or 2; 0: none)     */
 } kifmm_tuning_t;
 kifmm_status kifmm_get_tuning(kifmm_plan *plan, kifmm_tuning_t *out);
 
-/* Pins the tensor-core M2L variant instead of tuning it (a known-good choice
+/* Pins the mixed mode's M2L variant instead of tuning it (a known-good choice
  * replayed, or each variant tested): producers 2 or 4 warps, tiles 1 or 2
  * (two tiles take two producer warps), stages 2 .. the shared-memory
  * maximum for that tile count.  Every variant computes bit-identical
- * results.  KIFMM_ERR_ARG for other values or a plan without the
- * tensor-core M2L (FP64, FP32, Stokeslet).  Host only; no device work. */
+ * results (where a small tree's slots are split over blocks, both producer
+ * counts run two warps).  KIFMM_ERR_ARG for other values or a plan of another
+ * mode (FP64, FP32, Stokeslet: their M2L has one form).  Host only; no device
+ * work. */
 kifmm_status kifmm_set_m2l_tuning(kifmm_plan *plan, int producers, int tiles, int stages);
 
-/* Bound, in polls, of every barrier wait of the tensor-core M2L's pipeline
+/* Bound, in polls, of every barrier wait of a mixed plan's M2L pipelines
  * (0: the default, about 2^24).  Every wait of that kernel is bounded: on
  * time-out its blocks record KIFMM_ERR_TIMEOUT in the device status
  * (kifmm_get_device_status), wait for their own copies and products in flight
- * (with a bound of its own), free their tensor memory and return, so that the context
- * stays usable; the outputs of the particles below a box that timed out are
+ * (with a bound of their own), free their tensor memory and return, so that
+ * the context stays usable; the outputs of the particles below a box that timed out are
  * NaN.  A backward's M2L (exact-split products on the tensor cores in every
  * mode) is bounded in the same way and takes the same bound.  A tiny bound
  * makes the waits run out on purpose (the time-out path's test).

@@ -62,7 +62,7 @@ struct SimtArgs {
     double *dbar;            // [nb]: output column n (the mean row), or nullptr
     float *part;             // SPLIT: [slot of the round][target][ldp]
     int n, nkp, ldp, ncb;    // column blocks of 32 NC
-    int slot0, nslots;       // SPLIT: this round's slots
+    int slot0, nslots;       // SPLIT: the slots of this launch
 };
 
 constexpr int simt_blocks(int rt, int nc, bool split) {  // blocks per SM the registers are held to

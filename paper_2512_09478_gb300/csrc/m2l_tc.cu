@@ -68,7 +68,7 @@ struct TileArgs {
     float *d;                 // [nb][ns]
     double *dbar;             // [nb] output column ns (the mean row), or nullptr
     float *part;              // SPLIT: [slot of the round][tile of 128][np][128] partial products
-    int slot0, nslots;        // SPLIT: this round's slots
+    int slot0, nslots;        // SPLIT: the slots of this launch
     int n_tiles;              // tiles of 128
     int ns, kp, np, nstages;  // np: operator rows (output columns) incl. padding
     int ncb;                  // column blocks (np = ncb NT)
